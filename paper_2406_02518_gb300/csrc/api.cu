@@ -143,6 +143,7 @@ ddgs_status make_layout(int32_t R, const int64_t *n, const int64_t *n_iso, const
   s.R = R; s.V = v; s.tile = tile;
   s.n_total = g; s.total_tiles = tiles; s.records = recs; s.pixels = pix; s.n_blocks = blk;
   ddgs::plan_binning(L.view.data(), v, L.req.data(), tiles, tile, s);
+  ddgs::plan_slices(L.view.data(), v, L.req.data(), tile, s);
   L.hash = h ? h : 1;
   return DDGS_OK;
 }
@@ -161,8 +162,10 @@ ddgs_status ensure_tables(ddgs_workspace *ws, int64_t R, int64_t V) {
   if (ws->d_req) CK(cudaFree(ws->d_req));
   if (ws->d_view) CK(cudaFree(ws->d_view));
   if (ws->req_time) CK(cudaFree(ws->req_time));
+  if (ws->splits) CK(cudaFree(ws->splits));
   ws->d_req = nullptr;
   ws->d_view = nullptr;
+  ws->splits = nullptr;
   ws->req_time = nullptr;
   ws->req_cap = ws->view_cap = 0;
   CK(cudaHostAlloc(&ws->h_tab, rc * sizeof(ddgs::ReqTab) + vc * sizeof(ddgs::ViewTab),
@@ -170,6 +173,7 @@ ddgs_status ensure_tables(ddgs_workspace *ws, int64_t R, int64_t V) {
   CK(cudaMalloc(&ws->d_req, rc * sizeof(ddgs::ReqTab)));
   CK(cudaMalloc(&ws->d_view, vc * sizeof(ddgs::ViewTab)));
   CK(cudaMalloc(&ws->req_time, (1 + 2 * rc) * sizeof(unsigned long long)));
+  CK(cudaMalloc(&ws->splits, vc * ddgs::SLICE_MAX * sizeof(uint32_t)));
   ws->req_cap = rc;
   ws->view_cap = vc;
   ws->last_hash = 0;
@@ -202,7 +206,7 @@ ddgs_status upload_layout(ddgs_workspace *ws, Layout &L, bool no_sync, cudaStrea
 
 // Sort queues of the binning: sized by the tile and pair capacities.
 ddgs_status ensure_lists(ddgs_workspace *ws) {
-  const int64_t need = ddgs::list_capacity(ws->tile_cap, ws->pair_cap);
+  const int64_t need = ddgs::list_capacity(ws->vtile_cap, ws->pair_cap);
   if (need <= ws->list_cap && ws->lists) return DDGS_OK;
   const int64_t cap = need + need / 4;
   ddgs_status st = grow(ws->lists, ws->list_cap, cap, sizeof(uint64_t));
@@ -240,9 +244,15 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
     ddgs_status st;
     if ((st = grow(ws->ranges, ws->tile_cap, cap, sizeof(uint2)))) return st;
     if ((st = grow(ws->order, ws->tile_cap, cap, sizeof(uint32_t)))) return st;
-    int64_t pc = 0;  // the part sums follow the tiles
-    if ((st = grow(ws->part, pc, ddgs::part_capacity(cap), sizeof(uint64_t)))) return st;
     ws->tile_cap = cap;
+  }
+  if (s.total_vtiles > ws->vtile_cap || !ws->vranges) {
+    int64_t cap = s.total_vtiles + s.total_vtiles / 4 + 64;
+    ddgs_status st;
+    if ((st = grow(ws->vranges, ws->vtile_cap, cap, sizeof(uint2)))) return st;
+    int64_t pc = 0;  // the part sums follow the lists
+    if ((st = grow(ws->part, pc, ddgs::part_capacity(cap), sizeof(uint64_t)))) return st;
+    ws->vtile_cap = cap;
   }
   if (s.hist_slots > ws->hist_cap || !ws->hist) {
     int64_t cap = std::max<int64_t>(s.hist_slots + s.hist_slots / 4, 1024);
@@ -430,7 +440,7 @@ ddgs_status ddgs_workspace_destroy(ddgs_workspace *ws) {
   if (!ws) return DDGS_OK;
   void *dev[] = {ws->rec, ws->rect, ws->tiles_touched, ws->grad2d, ws->blk_total,
                  ws->keys[0], ws->keys[1], ws->vals, ws->hist, ws->part, ws->lists,
-                 ws->list_count, ws->ranges, ws->d_pairs, ws->d_status, ws->d_req, ws->d_view,
+                 ws->list_count, ws->ranges, ws->vranges, ws->splits, ws->d_pairs, ws->d_status, ws->d_req, ws->d_view,
                  ws->order, ws->queue, ws->req_time, ws->rec2, ws->grad_h,
                  ws->rads_keys, ws->rads_buf};
   for (void *p : dev)
@@ -452,7 +462,8 @@ ddgs_status ddgs_workspace_reserve(ddgs_workspace *ws, int64_t records, int64_t 
   // preprocess blocks (one partial block per request, up to 4096 requests)
   s.n_blocks = records / ddgs::PRE_THREADS + 4096;
   s.total_tiles = tiles;
-  s.hist_slots = ddgs::hist_slot_bound(tiles);
+  s.total_vtiles = ddgs::vtile_bound(tiles, records);
+  s.hist_slots = ddgs::hist_slot_bound(s.total_vtiles);
   ddgs_status st = ensure_records(ws, s);
   if (st) return st;
   st = ensure_pairs(ws, pairs);
@@ -477,8 +488,8 @@ ddgs_status render_common(const ddgs_gaussians &g, const ddgs_views &v, const dd
   ddgs::RenderShape &s = L.shape;
   if (c->no_sync) {
     if (s.records > ws->rec_cap || s.n_blocks > ws->blk_cap || s.total_tiles > ws->tile_cap ||
-        s.hist_slots > ws->hist_cap || !ws->keys[0] ||
-        ddgs::list_capacity(s.total_tiles, ws->pair_cap) > ws->list_cap)
+        s.total_vtiles > ws->vtile_cap || s.hist_slots > ws->hist_cap || !ws->keys[0] ||
+        ddgs::list_capacity(s.total_vtiles, ws->pair_cap) > ws->list_cap)
       return DDGS_ERR_CAPACITY;
     if (g.per_pixel && (!ws->rec2 || ws->pix_cap < s.records)) return DDGS_ERR_CAPACITY;
   } else {

@@ -97,6 +97,7 @@ struct BinItem {
   int64_t rec0, l0, l1;  // records of Gaussians [l0, l1) of the view start at rec0
   int64_t slot;          // first tile counter of the block
   int tx0, ty0, bw, bh;  // the band's first tile and size
+  int lg;                // each tile has 2^lg lists and counters, one per depth slice
 };
 
 __device__ __forceinline__ BinItem bin_item(const RenderShape &s, const ViewTab &vt, int64_t item) {
@@ -112,8 +113,48 @@ __device__ __forceinline__ BinItem bin_item(const RenderShape &s, const ViewTab 
   it.bh = vt.band_h;
   it.tx0 = (int)(band % vt.bands_x) * vt.band_w;
   it.ty0 = (int)(band / vt.bands_x) * vt.band_h;
-  it.slot = vt.hist_base + j * (int64_t)vt.band_w * vt.band_h;
+  it.lg = vt.lg_slices;
+  it.slot = vt.hist_base + j * (((int64_t)vt.band_w * vt.band_h) << it.lg);
   return it;
+}
+
+// The depth slice of a record: the number of slices that start at or below
+// its depth bits (sp[j] is slice j's first depth, j >= 1).
+__device__ __forceinline__ int depth_slice(uint32_t depth, const uint32_t *sp, int lg) {
+  int k = 0;
+  for (int step = lg ? 1 << (lg - 1) : 0; step > 0; step >>= 1)
+    if (depth >= sp[k + step]) k += step;
+  return k;
+}
+
+// First depths of the slices of every sliced view (one block each): the
+// quantiles of a strided sample of its records that touch a tile. Any
+// monotone cut gives the same lists; an uneven one only sorts slower.
+constexpr int SLICE_SAMPLE = 512;
+__global__ void __launch_bounds__(SLICE_SAMPLE) bin_slices_kernel(RenderShape s, const uint4 *info,
+                                                                  uint32_t *splits) {
+  __shared__ uint32_t s_d[SLICE_SAMPLE];
+  const ViewTab vt = s.view[blockIdx.x];
+  if (vt.lg_slices == 0) return;
+  const int t = threadIdx.x;
+  const int64_t n = s.req[vt.req].n;  // > SLICE_FROM >= SLICE_SAMPLE
+  const uint4 b = info[vt.rec_off + t * n / SLICE_SAMPLE];
+  s_d[t] = b.w ? b.z : 0xffffffffu;
+  const int m = __syncthreads_count(b.w != 0);
+  for (int w = 2; w <= SLICE_SAMPLE; w <<= 1)
+    for (int j = w >> 1; j > 0; j >>= 1) {
+      const int o = t ^ j;
+      if (o > t) {
+        const uint32_t x = s_d[t], y = s_d[o];
+        if ((x > y) == ((t & w) == 0)) {
+          s_d[t] = y;
+          s_d[o] = x;
+        }
+      }
+      __syncthreads();
+    }
+  const int slices = 1 << vt.lg_slices;
+  if (t > 0 && t < slices) splits[(int64_t)blockIdx.x * SLICE_MAX + t] = s_d[(int64_t)t * m / slices];
 }
 
 // The part of a record's tile rectangle inside the block's band; false when
@@ -131,12 +172,19 @@ __device__ __forceinline__ bool band_rect(const uint4 &b, const BinItem &it, int
 // count: the block's pairs per tile of its band -> hist[slot ...]
 // Eight blocks per SM (32 registers, a few bytes spilled): the count waits on
 // its record loads, and more warps hide them (0.128 -> 0.122 ms at 64 poses).
+// SLICED: some view is cut into depth slices (a separate instance: the slice
+// search cost the others 7 us of 123 at 64 poses).
+template <bool SLICED>
 __global__ void __launch_bounds__(BIN_THREADS, 8) bin_count_kernel(RenderShape s, const uint4 *info,
+                                                                  const uint32_t *splits,
                                                                   uint32_t *hist) {
   extern __shared__ uint32_t s_cnt[];
-  const ViewTab vt = s.view[find_item_view(s.view, s.V, blockIdx.x)];
+  __shared__ uint32_t s_sp[SLICE_MAX];
+  const int v = find_item_view(s.view, s.V, blockIdx.x);
+  const ViewTab vt = s.view[v];
   const BinItem it = bin_item(s, vt, blockIdx.x);
-  const int area = it.bw * it.bh;
+  const int area = (it.bw * it.bh) << (SLICED ? it.lg : 0);
+  if (SLICED && it.lg && threadIdx.x < (1 << it.lg)) s_sp[threadIdx.x] = splits[(int64_t)v * SLICE_MAX + threadIdx.x];
   for (int p = threadIdx.x; p < area; p += BIN_THREADS) s_cnt[p] = 0;
   __syncthreads();
   for (int64_t l0 = it.l0 + threadIdx.x; l0 < it.l1; l0 += BIN_LOADS * BIN_THREADS) {
@@ -150,47 +198,56 @@ __global__ void __launch_bounds__(BIN_THREADS, 8) bin_count_kernel(RenderShape s
     for (int k = 0; k < BIN_LOADS; ++k) {
       int x0, y0, x1, y1;
       if (!band_rect(b[k], it, x0, y0, x1, y1)) continue;
+      const int sl = SLICED ? depth_slice(b[k].z, s_sp, it.lg) : 0, lg = SLICED ? it.lg : 0;
       for (int y = y0; y <= y1; ++y)
-        for (int x = x0; x <= x1; ++x) atomicAdd(&s_cnt[(y - it.ty0) * it.bw + (x - it.tx0)], 1u);
+        for (int x = x0; x <= x1; ++x)
+          atomicAdd(&s_cnt[(((y - it.ty0) * it.bw + (x - it.tx0)) << lg) + sl], 1u);
     }
   }
   __syncthreads();
   for (int p = threadIdx.x; p < area; p += BIN_THREADS) hist[it.slot + p] = s_cnt[p];
 }
 
-// Where a tile's counters are: the band of the tile and its place in it.
+// Where a list's counters are: the band of its tile, the tile's place in it
+// and the depth slice.
 __device__ __forceinline__ bool tile_slot(const RenderShape &s, int64_t gt, int64_t &first,
                                           int64_t &stride, int &chunks) {
-  const ViewTab vt = s.view[find_view(s.view, s.V, gt)];
+  const int v = find_vtile_view(s.view, s.V, gt);
+  const ViewTab vt = s.view[v];
   chunks = vt.chunks;
   if (chunks == 0) return false;
-  const int64_t t = gt - vt.tile_base;
+  const int64_t t = (gt - vt.vtile_base) >> vt.lg_slices;
+  if (t >= s.view[v + 1].tile_base - vt.tile_base) {  // a gap that aligns the next view's lists
+    chunks = 0;
+    return false;
+  }
   const int ty = (int)(t / vt.tiles_x), tx = (int)(t - (int64_t)ty * vt.tiles_x);
   const int bx = tx / vt.band_w, by = ty / vt.band_h;
   const int64_t band = (int64_t)by * vt.bands_x + bx;
-  stride = (int64_t)vt.band_w * vt.band_h;
-  first = vt.hist_base + band * chunks * stride + (int64_t)(ty - by * vt.band_h) * vt.band_w +
-          (tx - bx * vt.band_w);
+  stride = ((int64_t)vt.band_w * vt.band_h) << vt.lg_slices;
+  first = vt.hist_base + band * chunks * stride +
+          (((int64_t)(ty - by * vt.band_h) * vt.band_w + (tx - bx * vt.band_w)) << vt.lg_slices) +
+          ((gt - vt.vtile_base) & ((1 << vt.lg_slices) - 1));
   return true;
 }
 
-// offsets, part 1: per tile, the chunks' counts become running offsets within
-// the tile's list; the tile total goes to ranges[gt].y, and each 1024-tile
-// group's sum of totals is added to part[group] (zeroed beforehand). A block
-// takes 32 tiles (one per lane) and splits their chunks over its 8 warps:
+// offsets, part 1: per list (a tile's, or one of its depth slices'), the
+// chunks' counts become running offsets within the list; its total goes to
+// vranges[gt].y, and each 1024-list group's sum of totals is added to
+// part[group] (zeroed beforehand). A block takes 32 lists (one per lane) and splits their chunks over its 8 warps:
 // each warp sums its share of the chunks, the warps' sums are scanned in
 // shared memory, and each warp then rewrites its share as running offsets.
 // Without pairs (counted = 0) every list is empty.
 constexpr int COL_WARPS = 8;
 __global__ void __launch_bounds__(COL_WARPS * 32) bin_column_kernel(RenderShape s, int counted,
-                                                                     uint32_t *hist, uint2 *ranges,
+                                                                     uint32_t *hist, uint2 *vranges,
                                                                      uint64_t *part) {
   __shared__ uint32_t s_sum[COL_WARPS][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t gt = (int64_t)blockIdx.x * 32 + lane;
   int64_t first = 0, stride = 0;
   int chunks = 0;
-  const bool has = gt < s.total_tiles && counted && tile_slot(s, gt, first, stride, chunks);
+  const bool has = gt < s.total_vtiles && counted && tile_slot(s, gt, first, stride, chunks);
   const int seg = (chunks + COL_WARPS - 1) / COL_WARPS;
   const int c0 = min(chunks, w * seg), c1 = min(chunks, c0 + seg);
   uint32_t *h = hist + first;
@@ -235,8 +292,8 @@ __global__ void __launch_bounds__(COL_WARPS * 32) bin_column_kernel(RenderShape 
     }
   }
   if (w == 0) {
-    if (gt < s.total_tiles) ranges[gt] = make_uint2(0u, total);
-    uint64_t t = total;  // the block's 32 tiles lie in one 1024-tile group
+    if (gt < s.total_vtiles) vranges[gt] = make_uint2(0u, total);
+    uint64_t t = total;  // the block's 32 lists lie in one 1024-list group
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
     if (lane == 0 && t) atomicAdd(reinterpret_cast<unsigned long long *>(part + (gt >> 10)), t);
@@ -260,17 +317,20 @@ __device__ __forceinline__ void list_append(const BinLists &L, int cls, uint64_t
   for (uint32_t c = 0; c < k; ++c) L.item[cls][base + c] = (gt << 24) | c;
 }
 
-// offsets, part 2: list ranges from the exclusive scan of the tile totals
-// ((0, 0) for an empty list), and each list of two or more entries queued for
-// its sort. A list that does not fit below the pair capacity is left empty
-// (whole lists only) and the capacity status is raised.
-__global__ void __launch_bounds__(1024) bin_offsets_kernel(int64_t n_tiles, uint2 *ranges,
+// offsets, part 2: list ranges from the exclusive scan of the totals ((0, 0)
+// for an empty list), and each list of two or more entries queued for its
+// sort. A tile whose lists do not all fit below the pair capacity is left
+// empty (whole tiles only) and the capacity status is raised. With depth
+// slices (ranges != vranges) a tile's range spans its 2^lg lists, which are
+// neighbours in the warp.
+__global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 *ranges, uint2 *vranges,
                                                              const uint64_t *part_off, uint64_t cap,
                                                              BinLists L, int32_t *status) {
   __shared__ uint64_t s_w[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t gt = (int64_t)blockIdx.x * 1024 + threadIdx.x;
-  const uint64_t cnt = gt < n_tiles ? ranges[gt].y : 0;
+  const bool in = gt < s.total_vtiles;
+  const uint64_t cnt = in ? vranges[gt].y : 0;
   uint64_t inc = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -282,12 +342,28 @@ __global__ void __launch_bounds__(1024) bin_offsets_kernel(int64_t n_tiles, uint
   uint64_t before = part_off[blockIdx.x];
   for (int w = 0; w < wid; ++w) before += s_w[w];
   const uint64_t off = before + inc - cnt;
+  uint64_t end = off + cnt;  // of the whole tile
   uint32_t n = 0;
-  if (gt < n_tiles) {
-    const bool fits = off + cnt <= cap;
+  if (s.sliced) {
+    const int v = in ? find_vtile_view(s.view, s.V, gt) : 0;
+    const ViewTab vt = s.view[v];
+    const int64_t local = gt - vt.vtile_base;
+    const int part = (1 << vt.lg_slices) - 1;
+    end = __shfl_sync(0xffffffffu, end, lane | (in ? part : 0));  // the tile's last list
+    if (in && (local >> vt.lg_slices) < s.view[v + 1].tile_base - vt.tile_base) {
+      const bool fits = end <= cap;
+      if (!fits) atomicOr(status, ST_CAPACITY);
+      n = fits ? (uint32_t)cnt : 0u;
+      vranges[gt] = n ? make_uint2((uint32_t)off, (uint32_t)(off + cnt)) : make_uint2(0u, 0u);
+      if ((local & part) == 0)
+        ranges[vt.tile_base + (local >> vt.lg_slices)] =
+            fits && end > off ? make_uint2((uint32_t)off, (uint32_t)end) : make_uint2(0u, 0u);
+    }
+  } else if (in) {
+    const bool fits = end <= cap;
     if (!fits) atomicOr(status, ST_CAPACITY);
     n = fits ? (uint32_t)cnt : 0u;
-    ranges[gt] = n ? make_uint2((uint32_t)off, (uint32_t)(off + cnt)) : make_uint2(0u, 0u);
+    ranges[gt] = n ? make_uint2((uint32_t)off, (uint32_t)end) : make_uint2(0u, 0u);
   }
   list_append(L, LIST_WARP, (uint64_t)gt, n >= 2 && n <= 32 ? 1u : 0u);
   list_append(L, LIST_SHORT, (uint64_t)gt, n > 32 && n <= SORT_SHORT ? 1u : 0u);
@@ -327,9 +403,18 @@ constexpr uint32_t CUR_ONE = 0x80000000u, CUR_DROP = 0xffffffffu;
 // then takes 74 KB and three fit an SM (0.59 -> 0.58 ms at 64 poses; 4,096
 // makes more chunks need a second window, 0.76 ms)
 constexpr int SCAT_STAGE = 5120;
+// with depth slices: a chunk's pairs are about three per Gaussian there, so
+// that a larger area saves most second windows, at two blocks per SM (500k
+// Gaussians, 64 views of 64^2: 5,120 0.93 ms, 6,144 0.87, 7,168 0.71, 8,192
+// 0.75; one pad counter per tile against bank conflicts 0.78, and the column
+// scan then read its counters unaligned, 0.08 -> 0.12 ms)
+constexpr int SCAT_STAGE_SLICED = 7168;
 
-__host__ __device__ constexpr size_t scatter_smem(int area, bool direct = false) {
-  return (direct ? 0 : (size_t)SCAT_STAGE * (sizeof(uint64_t) + sizeof(uint32_t))) +
+__host__ __device__ constexpr int scatter_stage(bool direct, bool sliced) {
+  return direct ? 0 : (sliced ? SCAT_STAGE_SLICED : SCAT_STAGE);
+}
+__host__ __device__ constexpr size_t scatter_smem(int area, bool direct, bool sliced) {
+  return (size_t)scatter_stage(direct, sliced) * (sizeof(uint64_t) + sizeof(uint32_t)) +
          (size_t)area * 3 * sizeof(uint32_t);
 }
 
@@ -370,19 +455,24 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t *a, int n, uin
 // the block's records. Chosen per render when the blocks average more pairs
 // than two staging windows (each further window would read the chunk's
 // records again): 2M Gaussians on eight 1024^2 views, 2.6 -> 1.1 ms.
-template <bool DIRECT>
+// SLICED: some view is cut into depth slices.
+template <bool DIRECT, bool SLICED>
 __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShape s, const uint4 *info,
+                                                                    const uint32_t *splits,
                                                                     const uint32_t *hist,
-                                                                    const uint2 *ranges,
+                                                                    const uint2 *vranges,
                                                                     uint64_t *keys, uint32_t *vals,
                                                                     uint64_t cap) {
   extern __shared__ __align__(16) unsigned char scat_smem[];
   __shared__ uint32_t s_wsum[SCAT_THREADS / 32];
-  const ViewTab vt = s.view[find_item_view(s.view, s.V, blockIdx.x)];
+  __shared__ uint32_t s_sp[SLICE_MAX];
+  const int v = find_item_view(s.view, s.V, blockIdx.x);
+  const ViewTab vt = s.view[v];
   const BinItem it = bin_item(s, vt, blockIdx.x);
   const int tiles_y = (vt.H + s.tile - 1) / s.tile;
-  const int area = it.bw * it.bh;
-  constexpr int STAGE = DIRECT ? 0 : SCAT_STAGE;
+  const int lg = SLICED ? it.lg : 0, area = (it.bw * it.bh) << lg;
+  if (SLICED && it.lg && threadIdx.x < (1 << it.lg)) s_sp[threadIdx.x] = splits[(int64_t)v * SLICE_MAX + threadIdx.x];
+  constexpr int STAGE = scatter_stage(DIRECT, SLICED);
   uint64_t *s_key = reinterpret_cast<uint64_t *>(scat_smem);  // [STAGE] staged pairs
   uint32_t *s_dst = reinterpret_cast<uint32_t *>(s_key + STAGE);  // [STAGE] their places
   uint32_t *s_base = s_dst + STAGE;  // [area] place of the tile's first pair of this block
@@ -391,10 +481,13 @@ __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShap
   const int64_t j = (int64_t)blockIdx.x - vt.item_base;
   const bool last_chunk = j % vt.chunks == vt.chunks - 1;
   for (int p = threadIdx.x; p < area; p += SCAT_THREADS) {
-    const int x = it.tx0 + p % it.bw, y = it.ty0 + p / it.bw;
+    const int q = p >> lg;
+    const int x = it.tx0 + q % it.bw, y = it.ty0 + q / it.bw;
     uint32_t base = CUR_DROP, cnt = 0;
     if (x < vt.tiles_x && y < tiles_y) {
-      const uint2 r = ranges[vt.tile_base + (int64_t)y * vt.tiles_x + x];
+      const int64_t local = (int64_t)y * vt.tiles_x + x;
+      const uint2 r = vranges[SLICED ? vt.vtile_base + (local << lg) + (p & ((1 << lg) - 1))
+                                   : vt.tile_base + local];
       if (r.y > r.x) {
         const uint32_t off = hist[it.slot + p];  // the chunk's offset within the list
         const uint32_t next = last_chunk ? r.y - r.x : hist[it.slot + area + p];
@@ -417,10 +510,11 @@ __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShap
       if (!band_rect(b, it, x0, y0, x1, y1)) continue;
       const uint32_t l = (uint32_t)l0;
       const uint64_t key = ((uint64_t)b.z << 32) | l;
+      const int sl = SLICED ? depth_slice(b.z, s_sp, it.lg) : 0;
       for (int y = y0; y <= y1; ++y) {
         const int row = (y - it.ty0) * it.bw;
         for (int x = x0; x <= x1; ++x) {
-          const int p = row + (x - it.tx0);
+          const int p = ((row + (x - it.tx0)) << lg) + sl;
           if (s_base[p] == CUR_DROP) continue;
           const uint32_t c = atomicAdd(&s_cur[p], 1u);
           const uint32_t dst = s_base[p] + (c - s_beg[p]);  // keeps the CUR_ONE flag
@@ -441,7 +535,7 @@ __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShap
     int lo = w0, hi = area;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if ((mid < area ? s_beg[mid] : all) - b0 <= (uint32_t)SCAT_STAGE) lo = mid; else hi = mid - 1;
+      if ((mid < area ? s_beg[mid] : all) - b0 <= (uint32_t)STAGE) lo = mid; else hi = mid - 1;
     }
     const bool direct = lo == w0;  // tile w0 alone has more pairs than the area
     const int w1 = direct ? w0 + 1 : lo;
@@ -460,10 +554,11 @@ __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShap
         if (!band_rect(b[k], it, x0, y0, x1, y1)) continue;
         const uint32_t l = (uint32_t)(l0 + k * SCAT_THREADS);
         const uint64_t key = ((uint64_t)b[k].z << 32) | l;
+        const int sl = SLICED ? depth_slice(b[k].z, s_sp, it.lg) : 0;
         for (int y = y0; y <= y1; ++y) {
           const int row = (y - it.ty0) * it.bw;
           for (int x = x0; x <= x1; ++x) {
-            const int p = row + (x - it.tx0);
+            const int p = ((row + (x - it.tx0)) << lg) + sl;
             if (p < w0 || p >= w1 || s_base[p] == CUR_DROP) continue;
             const uint32_t c = atomicAdd(&s_cur[p], 1u);
             const uint32_t dst = s_base[p] + (c - s_beg[p]);  // keeps the CUR_ONE flag
@@ -895,29 +990,38 @@ cudaError_t prepare_bin_kernels() {
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
   e = cudaFuncSetAttribute(bin_sort_block_kernel<SORT_LONG_THREADS, SORT_LONG_ITEMS, 1>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LONG_SMEM);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(bin_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)scatter_smem(BIN_HIST_MAX));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(bin_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)scatter_smem(BIN_HIST_MAX, true));
+  const struct { void (*k)(RenderShape, const uint4 *, const uint32_t *, const uint32_t *, const uint2 *, uint64_t *,
+                           uint32_t *, uint64_t); bool direct, sliced; } scat[] = {
+      {bin_scatter_kernel<false, false>, false, false}, {bin_scatter_kernel<true, false>, true, false},
+      {bin_scatter_kernel<false, true>, false, true}, {bin_scatter_kernel<true, true>, true, true}};
+  for (const auto &x : scat)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(x.k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)scatter_smem(BIN_HIST_MAX, x.direct, x.sliced));
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
   return e;
 }
 
 void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &ws,
                     cudaStream_t st) {
-  const int64_t T = s.total_tiles;
+  const int64_t T = s.total_vtiles;  // lists
   if (T <= 0) return;
   if (prepare_bin_kernels() != cudaSuccess) return;  // surfaces via cudaGetLastError
   const uint64_t cap = (uint64_t)ws.pair_cap;
   const size_t hsm = (size_t)s.hist_area * sizeof(uint32_t);  // <= 32 KiB
   const unsigned sms = (unsigned)device_sms();  // the sorts run persistent blocks per SM
   const bool pairs = pair_bound > 0 && s.n_items > 0;
+  uint2 *vranges = s.sliced ? ws.vranges : ws.ranges;
+  if (pairs && s.sliced) {
+    LaunchScope ls(KID_BIN_OFFSETS, st);
+    bin_slices_kernel<<<(unsigned)s.V, SLICE_SAMPLE, 0, st>>>(
+        s, reinterpret_cast<const uint4 *>(ws.rect), ws.splits);
+  }
   if (pairs) {
     LaunchScope ls(KID_BIN_COUNT, st);
-    bin_count_kernel<<<(unsigned)s.n_items, BIN_THREADS, hsm, st>>>(
-        s, reinterpret_cast<const uint4 *>(ws.rect), ws.hist);
+    auto k = s.sliced ? bin_count_kernel<true> : bin_count_kernel<false>;
+    k<<<(unsigned)s.n_items, BIN_THREADS, hsm, st>>>(s, reinterpret_cast<const uint4 *>(ws.rect),
+                                                     ws.splits, ws.hist);
   }
   const int64_t nb = (T + 1023) / 1024;
   uint64_t *part = ws.part, *part_off = ws.part + nb + 1;
@@ -933,7 +1037,7 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
     bin_column_kernel<<<(unsigned)((T + 31) / 32), COL_WARPS * 32, 0, st>>>(s, pairs ? 1 : 0, ws.hist,
-                                                                          ws.ranges, part);
+                                                                          vranges, part);
   }
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
@@ -941,19 +1045,18 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
   }
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
-    bin_offsets_kernel<<<(unsigned)nb, 1024, 0, st>>>(T, ws.ranges, part_off, cap, L, ws.d_status);
+    bin_offsets_kernel<<<(unsigned)nb, 1024, 0, st>>>(s, ws.ranges, vranges, part_off, cap, L,
+                                                      ws.d_status);
   }
   if (!pairs) return;
   {
     LaunchScope ls(KID_BIN_SCATTER, st);
     // the pair bound (the count, or the capacity without a sync) over the blocks
-    const bool direct = pair_bound > 2u * (uint64_t)SCAT_STAGE * (uint64_t)s.n_items;
-    if (direct)
-      bin_scatter_kernel<true><<<(unsigned)s.n_items, SCAT_THREADS, scatter_smem(s.hist_area, true), st>>>(
-          s, reinterpret_cast<const uint4 *>(ws.rect), ws.hist, ws.ranges, ws.keys[0], ws.vals, cap);
-    else
-      bin_scatter_kernel<false><<<(unsigned)s.n_items, SCAT_THREADS, scatter_smem(s.hist_area), st>>>(
-          s, reinterpret_cast<const uint4 *>(ws.rect), ws.hist, ws.ranges, ws.keys[0], ws.vals, cap);
+    const bool direct = pair_bound > 2u * (uint64_t)scatter_stage(false, s.sliced) * (uint64_t)s.n_items;
+    auto k = s.sliced ? (direct ? bin_scatter_kernel<true, true> : bin_scatter_kernel<false, true>)
+                      : (direct ? bin_scatter_kernel<true, false> : bin_scatter_kernel<false, false>);
+    k<<<(unsigned)s.n_items, SCAT_THREADS, scatter_smem(s.hist_area, direct, s.sliced), st>>>(
+        s, reinterpret_cast<const uint4 *>(ws.rect), ws.splits, ws.hist, vranges, ws.keys[0], ws.vals, cap);
   }
   // A list holds at most one entry per Gaussian of its request, so a render of
   // n_total Gaussians in all cannot fill the classes of longer lists: those
@@ -962,12 +1065,12 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
   if (nmax >= 2) {
     LaunchScope ls(KID_BIN_SORT, st);
     bin_sort_warp_kernel<<<sms * 4, 256, 0, st>>>(L.item[LIST_WARP], L.count + LIST_WARP,
-                                                   ws.ranges, ws.keys[0], ws.vals);
+                                                   vranges, ws.keys[0], ws.vals);
   }
   if (nmax > 32) {
     LaunchScope ls(KID_BIN_SORT, st);
     bin_sort_block_kernel<128, SORT_SHORT / 128, 8><<<sms * 8, 128, SHORT_SMEM, st>>>(
-        L.item[LIST_SHORT], L.count + LIST_SHORT, ws.ranges, ws.keys[0], ws.vals);
+        L.item[LIST_SHORT], L.count + LIST_SHORT, vranges, ws.keys[0], ws.vals);
   }
   if (nmax > SORT_SHORT) {
     LaunchScope ls(KID_BIN_SORT, st);
@@ -976,17 +1079,17 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
     // at 96 registers (which led before the padding, 0.69 against 0.72; four
     // at 128 registers measured 0.75)
     bin_sort_block_kernel<128, SORT_MID / 128, 6><<<sms * 6, 128, MID_SMEM, st>>>(
-        L.item[LIST_MID], L.count + LIST_MID, ws.ranges, ws.keys[0], ws.vals);
+        L.item[LIST_MID], L.count + LIST_MID, vranges, ws.keys[0], ws.vals);
   }
   if (nmax > SORT_MID) {
     LaunchScope ls(KID_BIN_SORT, st);
     bin_sort_block_kernel<SORT_LONG_THREADS, SORT_LONG_ITEMS, 1>
         <<<sms, SORT_LONG_THREADS, LONG_SMEM, st>>>(L.item[LIST_BLOCK], L.count + LIST_BLOCK,
-                                                   ws.ranges, ws.keys[0], ws.vals);
+                                                   vranges, ws.keys[0], ws.vals);
   }
   if (nmax > BIN_LIST_LONG) {
     LaunchScope ls(KID_BIN_MERGE, st);
-    bin_merge_kernel<<<sms * 2, 256, 0, st>>>(L.item[LIST_LONG], L.count + LIST_LONG, ws.ranges,
+    bin_merge_kernel<<<sms * 2, 256, 0, st>>>(L.item[LIST_LONG], L.count + LIST_LONG, vranges,
                                               ws.keys[0], ws.keys[1], ws.vals);
   }
 }

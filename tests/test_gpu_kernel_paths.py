@@ -60,3 +60,52 @@ def test_generic_radiosity_loads(n, k, L, bf16, shift, entangled, ws):
         cloud = dataclasses.replace(cloud, feat_iso=_shifted(cloud.feat_iso), feat_dir=_shifted(cloud.feat_dir))
     st = syn.Settings(near_plane=0.2)
     _check(scene, _two_views(45, 60, 8.0 / 56), st, cloud, B.config_from_settings(st), ws)
+
+
+def _column(n, seed, depths, spread):
+    """n Gaussians around the source-to-detector axis, on the given depths (or
+    spread over a depth range), so that a few tiles hold nearly all of them."""
+    sc = syn.uniform_cloud(n, seed=seed, extent=spread, log_scale_range=(-4.5, -3.5), alpha_range=(0.02, 0.1))
+    if depths is not None:
+        sc.means[:, 2] = np.asarray(depths, np.float32)[np.arange(n) % len(depths)]
+    return sc
+
+
+@pytest.mark.parametrize("n,size,tile,depths,spread", [
+    (2100, 8, 8, None, 0.3),        # two slices of one tile
+    (9000, 32, 8, None, 0.3),       # sixteen tiles just past the line
+    (60000, 16, 8, None, 0.3),      # the most slices a tile gets
+    (30000, 24, 8, (0.0, 0.1, 0.1001), 0.2),  # three depths: most slices empty
+    (20000, 16, 16, (0.05,), 0.1)])  # one depth: one slice of 20,000 (chunk sorts, merge)
+def test_depth_slices(n, size, tile, depths, spread, ws):
+    """Views with many Gaussians per tile: the tile lists, cut into depth
+    slices, must be the oracle's whole lists."""
+    scene = _column(n, 90 + size, depths, spread)
+    views = _views([syn.pose_matrix(np.eye(3), np.array([0.0, 0.0, 2.0])),
+                    syn.pose_matrix(syn.rot_y(0.3), np.array([0.02, 0.0, 2.1]))], 4.0, 1.2 / size, size, size)
+    st = syn.Settings(near_plane=0.2, tile=tile)
+    cloud, gv, cfg = B.cloud_from_arrays(scene), B.views_from_arrays(views), B.config_from_settings(st)
+    img, tf, nl = B.render(cloud, gv, cfg, ws)
+    torch.cuda.synchronize()
+    ref = oracle.bin32(scene, views, st)
+    compare_binning(_bins(ws, scene, views, st), ref)
+    # the same without a synchronisation, on a workspace reserved by the public sizes, and with
+    # room for about half of the pairs: whole tiles only
+    tiles = views.n_views * (-(-size // tile)) ** 2
+    for pairs, want in ((ref["m"], 0), (ref["m"] // 3, 2)):
+        w2 = B.Workspace()
+        w2.reserve(views.n_views * n, pairs, tiles)
+        i2, _, _ = B.render(cloud, gv, B.config_from_settings(st, no_sync=True), w2)
+        fits = ref["m"] <= pairs + pairs // 4 + 4096
+        assert w2.sync_status() == (0 if fits else 2)
+        got = _bins(w2, scene, views, st)
+        if fits:
+            compare_binning(got, ref)
+            assert torch.equal(i2, img)
+        else:
+            gr, rr = (x["ranges"].reshape(-1, 2).astype(np.int64) for x in (got, ref))
+            for t in range(tiles):
+                if gr[t, 1] > gr[t, 0]:
+                    assert np.array_equal(gr[t], rr[t])
+                    assert np.array_equal(got["vals"][gr[t, 0]:gr[t, 1]], ref["vals"][rr[t, 0]:rr[t, 1]])
+        w2.close()
