@@ -413,7 +413,7 @@ ddgs_status ddgs_workspace_create(ddgs_workspace **out) {
       (e = cudaMalloc(&ws->d_pairs, sizeof(uint64_t))) != cudaSuccess ||
       (e = cudaMalloc(&ws->d_status, sizeof(int32_t))) != cudaSuccess ||
       (e = cudaMalloc(&ws->queue, 2 * sizeof(uint32_t))) != cudaSuccess ||
-      (e = cudaMalloc(&ws->list_count, ddgs::LIST_CLASSES * sizeof(uint32_t))) != cudaSuccess ||
+      (e = cudaMalloc(&ws->list_count, ddgs::BIN_COUNTERS * sizeof(uint32_t))) != cudaSuccess ||
       (e = cudaHostAlloc(&ws->h_pairs, 2 * sizeof(uint64_t), cudaHostAllocDefault)) != cudaSuccess ||
       (e = cudaMemset(ws->d_status, 0, sizeof(int32_t))) != cudaSuccess ||
       (e = cudaMemset(ws->d_pairs, 0, sizeof(uint64_t))) != cudaSuccess) {

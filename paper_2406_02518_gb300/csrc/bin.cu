@@ -322,11 +322,14 @@ __device__ __forceinline__ void list_append(const BinLists &L, int cls, uint64_t
 // sort. A tile whose lists do not all fit below the pair capacity is left
 // empty (whole tiles only) and the capacity status is raised. With depth
 // slices (ranges != vranges) a tile's range spans its 2^lg lists, which are
-// neighbours in the warp.
+// neighbours in the warp. Every tile is counted in its length bucket (lpt) for
+// the rasterisers' work order.
 __global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 *ranges, uint2 *vranges,
                                                              const uint64_t *part_off, uint64_t cap,
-                                                             BinLists L, int32_t *status) {
+                                                             BinLists L, uint32_t *lpt,
+                                                             int32_t *status) {
   __shared__ uint64_t s_w[32];
+  __shared__ uint32_t s_lpt[LPT_BUCKETS];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t gt = (int64_t)blockIdx.x * 1024 + threadIdx.x;
   const bool in = gt < s.total_vtiles;
@@ -338,6 +341,7 @@ __global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 
     if (lane >= o) inc += y;
   }
   if (lane == 31) s_w[wid] = inc;
+  if (threadIdx.x < LPT_BUCKETS) s_lpt[threadIdx.x] = 0;
   __syncthreads();
   uint64_t before = part_off[blockIdx.x];
   for (int w = 0; w < wid; ++w) before += s_w[w];
@@ -355,15 +359,19 @@ __global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 
       if (!fits) atomicOr(status, ST_CAPACITY);
       n = fits ? (uint32_t)cnt : 0u;
       vranges[gt] = n ? make_uint2((uint32_t)off, (uint32_t)(off + cnt)) : make_uint2(0u, 0u);
-      if ((local & part) == 0)
-        ranges[vt.tile_base + (local >> vt.lg_slices)] =
-            fits && end > off ? make_uint2((uint32_t)off, (uint32_t)end) : make_uint2(0u, 0u);
+      if ((local & part) == 0) {
+        const uint2 r = fits && end > off ? make_uint2((uint32_t)off, (uint32_t)end) : make_uint2(0u, 0u);
+        ranges[vt.tile_base + (local >> vt.lg_slices)] = r;
+        atomicAdd(&s_lpt[lpt_bucket(r)], 1u);
+      }
     }
   } else if (in) {
     const bool fits = end <= cap;
     if (!fits) atomicOr(status, ST_CAPACITY);
     n = fits ? (uint32_t)cnt : 0u;
-    ranges[gt] = n ? make_uint2((uint32_t)off, (uint32_t)end) : make_uint2(0u, 0u);
+    const uint2 r = n ? make_uint2((uint32_t)off, (uint32_t)end) : make_uint2(0u, 0u);
+    ranges[gt] = r;
+    atomicAdd(&s_lpt[lpt_bucket(r)], 1u);
   }
   list_append(L, LIST_WARP, (uint64_t)gt, n >= 2 && n <= 32 ? 1u : 0u);
   list_append(L, LIST_SHORT, (uint64_t)gt, n > 32 && n <= SORT_SHORT ? 1u : 0u);
@@ -371,6 +379,8 @@ __global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 
   list_append(L, LIST_BLOCK, (uint64_t)gt,
               n > SORT_MID ? (n + BIN_LIST_LONG - 1) / BIN_LIST_LONG : 0u);
   list_append(L, LIST_LONG, (uint64_t)gt, n > BIN_LIST_LONG ? 1u : 0u);
+  __syncthreads();
+  if (threadIdx.x < LPT_BUCKETS && s_lpt[threadIdx.x]) atomicAdd(&lpt[threadIdx.x], s_lpt[threadIdx.x]);
 }
 
 // L2 eviction priority of the binning records: they stream through once
@@ -1032,7 +1042,7 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
   L.item[LIST_LONG] = ws.lists + 3 * T;
   L.item[LIST_BLOCK] = ws.lists + 4 * T;
   L.count = ws.list_count;
-  cudaMemsetAsync(ws.list_count, 0, LIST_CLASSES * sizeof(uint32_t), st);
+  cudaMemsetAsync(ws.list_count, 0, BIN_COUNTERS * sizeof(uint32_t), st);
   cudaMemsetAsync(part, 0, (size_t)nb * sizeof(uint64_t), st);
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
@@ -1046,7 +1056,7 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
     bin_offsets_kernel<<<(unsigned)nb, 1024, 0, st>>>(s, ws.ranges, vranges, part_off, cap, L,
-                                                      ws.d_status);
+                                                      ws.list_count + LIST_CLASSES, ws.d_status);
   }
   if (!pairs) return;
   {

@@ -84,6 +84,20 @@ struct BinLists {
   uint32_t *count;               // device [LIST_CLASSES]
 };
 
+// The rasterisers take tiles by descending list length: bucket 0 is the empty
+// list, then four buckets per factor of two (the two bits below the length's
+// leading one). The binning counts the tiles per bucket.
+constexpr int LPT_BUCKETS = 4 * 32 + 1;
+__device__ __forceinline__ int lpt_bucket(uint2 r) {
+  const uint32_t len = r.y - r.x;
+  if (!len) return 0;
+  const int lg = 31 - __clz(len);
+  return 1 + 4 * lg + (int)((lg >= 2 ? len >> (lg - 2) : len << (2 - lg)) & 3u);
+}
+// Counters cleared before every binning: list queues, tiles per bucket, and
+// the places handed out per bucket.
+constexpr int BIN_COUNTERS = LIST_CLASSES + 2 * LPT_BUCKETS;
+
 // Parameters shared by the rasterisers. q_lim = CONIC_SCALE q_max: the q cutoff
 // in the units of the records' scaled conic (see eval_pair).
 struct RasterParams {
@@ -373,7 +387,7 @@ struct ddgs_workspace {
   uint32_t *hist = nullptr;      // [hist_cap] per (binning block, tile) counts, then offsets
   uint64_t *part = nullptr;      // [2 x tile blocks + 2] partial sums of the tile counts
   uint64_t *lists = nullptr;     // [list_cap] tile lists to sort, by length class
-  uint32_t *list_count = nullptr;  // [LIST_CLASSES]
+  uint32_t *list_count = nullptr;  // [BIN_COUNTERS]
   uint2 *ranges = nullptr;       // [tiles]
   uint2 *vranges = nullptr;      // [vtile_cap] the lists' ranges where tiles are sliced by depth
   uint32_t *splits = nullptr;    // [view_cap][SLICE_MAX] first depth of each slice

@@ -579,13 +579,16 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x) {
 }
 
 // Pixels of an 8 x 4 region whose centres lie in the box (x0, x1, y0, y1):
-// bit y * 8 + x for pixel centre (cx + x, cy + y).
+// bit y * 8 + x for pixel centre (cx + x, cy + y). ROWS: by row pairs (rows 0, 1
+// and 2, 3 together), the entries that a pixel sees in the pixel-pair kernels.
+template <bool ROWS>
 __device__ __forceinline__ uint32_t region_cover(float4 b, float cx, float cy) {
   const int x0 = max(0, __float2int_ru(b.x - cx)), x1 = min(7, __float2int_rd(b.y - cx));
   const int y0 = max(0, __float2int_ru(b.z - cy)), y1 = min(3, __float2int_rd(b.w - cy));
   if (x0 > x1 || y0 > y1) return 0u;
   const uint32_t row = (0xffu >> (7 - x1)) & (0xffu << x0);
-  const uint32_t rows = (0xffffffffu >> (8 * (3 - y1))) & (0xffffffffu << (8 * y0));
+  const uint32_t rows = (0xffffffffu >> (8 * (3 - (ROWS ? y1 | 1 : y1)))) &
+                        (0xffffffffu << (8 * (ROWS ? y0 & ~1 : y0)));
   return (row * 0x01010101u) & rows;
 }
 
@@ -616,7 +619,7 @@ struct Region {
   __device__ __forceinline__ int64_t pixel() const { return img_off + (int64_t)py * W + px; }
 };
 
-template <int T, bool PIX>
+template <int T, bool PIX, bool ROWS>
 __device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, int region, float4 *sA,
                                               float4 *sB, float4 *sC) {
   const int lane = threadIdx.x & 31;
@@ -653,7 +656,7 @@ __device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, i
         sA[lane] = r0;
         sB[lane] = r1;
         if (PIX) sC[lane] = a.rec2[r];
-        cover = region_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy);
+        cover = region_cover<ROWS>(ellipse_box(r0, r1, a.P.q_max), cx, cy);
       }
     }
     __syncwarp();
@@ -689,14 +692,14 @@ __device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, i
   }
 }
 
-// Resident blocks per SM asked of the register allocator. WIDE: eight (32
-// registers, a few bytes spilled; 64 warps per SM: 1.48 -> 1.42 ms at 64
-// poses, where six blocks at 40 registers measured 1.69 and five at 48 1.48),
-// for renders with several work items per warp slot. Otherwise five (48
-// registers), whose warps finish an item sooner: one 512^2 view, 0.078 ->
-// 0.069 ms. Per-pixel directions always take five (their walk would spill).
-template <int T, bool PIX, bool WIDE>
-__global__ void __launch_bounds__(WARPS * 32, WIDE ? 8 : 5) raster_fwd_warp_kernel(RasterArgs a) {
+// Five resident blocks per SM (48 registers): these renders have few items per
+// warp slot, and a warp with more registers finishes an item sooner (one 512^2
+// view, 0.069 ms against 0.078 at eight blocks).
+// ROWS: the backward of this render takes pixel pairs. The box only culls (q <=
+// q_max decides), but for ellipses so thin that rounding could pass a pixel
+// outside the box both passes must look at the same pixels.
+template <int T, bool PIX, bool ROWS>
+__global__ void __launch_bounds__(WARPS * 32, 5) raster_fwd_warp_kernel(RasterArgs a) {
   constexpr int NW = T * T / 32;
   __shared__ float4 s_a[WARPS][32], s_b[WARPS][32], s_c[WARPS][PIX ? 32 : 1];
   const int w = threadIdx.x >> 5;
@@ -705,7 +708,7 @@ __global__ void __launch_bounds__(WARPS * 32, WIDE ? 8 : 5) raster_fwd_warp_kern
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
     const int64_t gt = a.order[item / NW];
-    fwd_lane_item<T, PIX>(a, gt, (int)(item % NW), s_a[w], s_b[w], s_c[w]);
+    fwd_lane_item<T, PIX, ROWS>(a, gt, (int)(item % NW), s_a[w], s_b[w], s_c[w]);
     if (a.req_end && (threadIdx.x & 31) == 0)
       atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
   }
@@ -974,7 +977,7 @@ __device__ __forceinline__ void bwd_lane_item(const RasterArgs &a, int64_t gt, i
       if (id < rg.n_req) {
         sm.a[lane] = r0;
         sm.b[lane] = r1;
-        cover = region_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy);
+        cover = region_cover<false>(ellipse_box(r0, r1, a.P.q_max), cx, cy);
       }
       sm.id[lane] = id;
     }
@@ -1090,44 +1093,464 @@ __global__ void __launch_bounds__(LANE_WARPS * 32, 3) raster_bwd_lane_kernel(Ras
 
 constexpr size_t LANE_BWD_SMEM = LANE_WARPS * sizeof(LaneBwdSmem);
 
-// ---- work order: view by view, and within a view the tiles by descending
-// list length (bucketed by log2). At any time the persistent blocks then work
-// on a few views, whose records and gradient accumulators stay in L2 while
-// the longest lists of each view still start first. ----
-
-constexpr int LPT_BUCKETS = 34;  // 0 = empty list, b = 1 + floor(log2(len))
-
-__device__ __forceinline__ int lpt_bucket(uint2 r) {
-  const uint32_t len = r.y - r.x;
-  return len ? 33 - __clz(len) : 0;  // 1..33
+// ---- pixel pairs: an 8 x 8 region per warp, two pixels per lane ----
+// Lane l owns the pixels (l & 7, 2 (l >> 3)) and the one below it. An entry
+// staged once serves 64 pixels instead of 32, a list of 8 x 8 tiles has no
+// entry that misses the region, and neighbouring pixels mostly share their
+// entries, so that a warp takes 10.4 trips per 32 entries of a tile where its
+// two 8 x 4 halves took 16.9, and the backward's sums per entry 6.0 where they
+// took 14.5 (CPU count over the benchmark's lists). The two pixels' chains are
+// independent, and most of their arithmetic is done on binary32 pairs (add,
+// mul and fma .rn.f32x2: one instruction, each half rounded as the scalar
+// operation is), with the entry's values staged in duplicate so that they load
+// as pairs. sigma is carried negated (max(-alpha_max, -alpha G)), which turns
+// 1 - sigma and T (1 - sigma) into an add and an fma; every decision is the
+// one eval_pair takes, bit for bit.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t p) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
-// One block per view: a counting sort of the view's tiles by bucket, longest
-// bucket first, written to order[tile_base .. tile_base + tiles).
-__global__ void __launch_bounds__(256) tile_order_view_kernel(const ViewTab *view, const uint2 *ranges,
-                                                              uint32_t *order) {
-  __shared__ uint32_t h[LPT_BUCKETS], start[LPT_BUCKETS];
-  const int v = blockIdx.x;
-  const int64_t t0 = view[v].tile_base, nt = view[v + 1].tile_base - t0;
-  for (int b = threadIdx.x; b < LPT_BUCKETS; b += blockDim.x) h[b] = 0;
-  __syncthreads();
-  for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) atomicAdd(&h[lpt_bucket(ranges[t0 + t])], 1u);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (int b = LPT_BUCKETS - 1; b >= 0; --b) {
-      start[b] = run;
-      run += h[b];
-      h[b] = 0;  // reused as the bucket's cursor
+// A staged entry: (u, a'), (v, v) | (2b', 2b'), (c', c') | (-alpha, -alpha),
+// (colour, colour).
+struct PairSlot {
+  ulonglong2 g, k, c;
+};
+
+__device__ __forceinline__ void stage_pair(PairSlot &s, float4 r0, float4 r1) {
+  s.g = make_ulonglong2(pack2(r0.x, r0.z), pack2(r0.y, r0.y));
+  s.k = make_ulonglong2(pack2(r0.w, r0.w), pack2(r1.x, r1.x));
+  s.c = make_ulonglong2(pack2(-r1.y, -r1.y), pack2(r1.z, r1.z));
+}
+
+// q' at both pixels (eval_pair's operations); npy = (-py, -(py + 1)).
+__device__ __forceinline__ uint64_t pair_q(const PairSlot &s, float px, uint64_t npy) {
+  const float2 ua = unpack2(s.g.x);
+  const float dx = __fsub_rn(ua.x, px), m = __fmul_rn(ua.y, dx);
+  const uint64_t dy = add2(s.g.y, npy);
+  const uint64_t t = fma2(s.k.x, dy, pack2(m, m));
+  return fma2(mul2(s.k.y, dy), dy, mul2(pack2(dx, dx), t));
+}
+
+// The 8 x 8 pixel region of a work item.
+struct PairRegion {
+  int H, W, wx0, wy0, px, py;
+  bool in0, in1;
+  int64_t rec_base, img_off, n_req;
+  __device__ __forceinline__ PairRegion(const RenderShape &s, int64_t gt, int region, int T) {
+    const ViewTab vt = s.view[find_view(s.view, s.V, gt)];
+    H = vt.H;
+    W = vt.W;
+    rec_base = vt.rec_off;
+    img_off = vt.img_off;
+    n_req = s.req[vt.req].n;
+    const int64_t local = gt - vt.tile_base;
+    const int tyi = (int)(local / vt.tiles_x), txi = (int)(local - (int64_t)tyi * vt.tiles_x);
+    const int WX = T / 8;
+    wx0 = txi * T + (region % WX) * 8;
+    wy0 = tyi * T + (region / WX) * 8;
+    const int lane = threadIdx.x & 31;
+    px = wx0 + (lane & 7);
+    py = wy0 + 2 * (lane >> 3);
+    in0 = px < W && py < H;
+    in1 = px < W && py + 1 < H;
+  }
+  __device__ __forceinline__ int64_t pixel() const { return img_off + (int64_t)py * W + px; }
+};
+
+// Pairs of an 8 x 8 region that the box (x0, x1, y0, y1) covers a pixel centre
+// of: bit 8 r + x for column x and rows 2 r, 2 r + 1.
+__device__ __forceinline__ uint32_t pair_cover(float4 b, float cx, float cy) {
+  const int x0 = max(0, __float2int_ru(b.x - cx)), x1 = min(7, __float2int_rd(b.y - cx));
+  const int y0 = max(0, __float2int_ru(b.z - cy)), y1 = min(7, __float2int_rd(b.w - cy));
+  if (x0 > x1 || y0 > y1) return 0u;
+  const uint32_t row = (0xffu >> (7 - x1)) & (0xffu << x0);
+  const uint32_t rows = (0xffffffffu >> (8 * (3 - (y1 >> 1)))) & (0xffffffffu << (8 * (y0 >> 1)));
+  return (row * 0x01010101u) & rows;
+}
+
+// Forward of one item. Two batches of 32 entries are staged at a time: a lane
+// that has walked its entries of the older batch goes on with the newer one
+// instead of waiting for the busiest lane, whose share of the older batch sets
+// the number of trips (7.7 trips per batch instead of 10.4 at the benchmark).
+// T is negated once a pixel has stopped (every later T (1 - sigma) is then
+// below t_min), and from the start outside the image.
+template <int T>
+__device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, int region,
+                                              PairSlot *slots) {
+  const int lane = threadIdx.x & 31;
+  const PairRegion rg(a.s, gt, region, T);
+  const uint2 range = a.ranges[gt];
+  const uint32_t *vals = a.vals;
+  const float px = rg.px + 0.5f;
+  const uint64_t npy = pack2(-(rg.py + 0.5f), -(rg.py + 1.5f));
+  const float cx = rg.wx0 + 0.5f, cy = rg.wy0 + 0.5f;
+  const float namax = -a.P.alpha_max, namin = -a.P.alpha_min;
+  float T0 = rg.in0 ? 1.f : -1.f, T1 = rg.in1 ? 1.f : -1.f, C0 = 0.f, C1 = 0.f;
+  uint32_t last0 = 0, last1 = 0;
+  bool done = !rg.in0;  // in1 implies in0
+  // software pipeline: the list ids two batches ahead and the records one
+  // batch ahead are in flight while a batch is walked
+  uint32_t id1 = 0xffffffffu, id2 = 0xffffffffu;
+  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+  if (range.x + lane < range.y) id1 = vals[range.x + lane];
+  if (range.x + 32 + lane < range.y) id2 = vals[range.x + 32 + lane];
+  if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
+  uint32_t m = 0, nx = 0;         // entries left of the older and of the newer batch
+  uint32_t slot = 0, pos = 1;     // first slot and first 1-based list position of m's batch
+  for (uint32_t b0 = range.x;; b0 += 32) {
+    if (__all_sync(0xffffffffu, done)) break;
+    // everything before the batch at b0 - 32 is walked
+    const uint32_t half = (b0 - range.x) & 32u;
+    if (m == 0) {
+      m = nx;
+      slot = half ^ 32u;
+      pos = b0 - range.x - 31u;
+    }
+    nx = 0;
+    const int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(m));
+    if (b0 < range.y) {
+      const uint32_t id = id1;
+      const float4 r0 = n0, r1 = n1;
+      id1 = id2;
+      id2 = 0xffffffffu;
+      if (b0 + 64 + lane < range.y) id2 = vals[b0 + 64 + lane];
+      if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
+      uint32_t cover = 0;
+      if (b0 + lane < range.y && id < rg.n_req) {
+        stage_pair(slots[half + lane], r0, r1);
+        cover = pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy);
+      }
+      __syncwarp();
+      nx = transpose32(cover);
+      if (done) nx = 0;
+    } else if (trips == 0) {
+      break;
+    }
+    for (int t = 0; t < trips; ++t) {
+      if (m == 0) {
+        m = nx;
+        nx = 0;
+        slot ^= 32u;
+        pos += 32u;
+      }
+      if (m == 0) continue;
+      const uint32_t k = (uint32_t)__ffs(m) - 1u;
+      m &= m - 1;
+      const PairSlot &s = slots[slot + k];
+      const uint64_t q = pair_q(s, px, npy);
+      const float2 qf = unpack2(q);
+      const uint64_t naG = mul2(s.c.x, pack2(exp2_approx(qf.x), exp2_approx(qf.y)));
+      const float2 ng = unpack2(naG);
+      const float ns0 = fmaxf(namax, ng.x), ns1 = fmaxf(namax, ng.y);  // -sigma
+      const bool ok0 = !(qf.x < a.P.q_lim || qf.x > 0.f) && ns0 <= namin;
+      const bool ok1 = !(qf.y < a.P.q_lim || qf.y > 0.f) && ns1 <= namin;
+      const uint64_t ns = pack2(ns0, ns1), Tr = pack2(T0, T1);
+      const float2 Tn = unpack2(fma2(Tr, ns, Tr));  // T (1 - sigma)
+      const bool st0 = ok0 && Tn.x < a.P.t_min, st1 = ok1 && Tn.y < a.P.t_min;
+      // C - (colour (-sigma)) T
+      const float2 w = unpack2(mul2(s.c.y, ns));
+      const uint32_t p = pos + k;
+      if (ok0 && !st0) {
+        C0 = fmaf(-w.x, T0, C0);
+        T0 = Tn.x;
+        last0 = p;
+      }
+      if (ok1 && !st1) {
+        C1 = fmaf(-w.y, T1, C1);
+        T1 = Tn.y;
+        last1 = p;
+      }
+      if (st0 || st1) {
+        if (st0) T0 = -fabsf(T0);
+        if (st1) T1 = -fabsf(T1);
+        if (T0 < 0.f && T1 < 0.f) {
+          done = true;
+          m = nx = 0;
+        }
+      }
+    }
+    __syncwarp();  // the older half is rewritten by the next batch
+  }
+  if (rg.in0) {
+    const int64_t pix = rg.pixel();
+    a.image[pix] = C0;
+    a.t_final[pix] = fabsf(T0);
+    a.n_last[pix] = last0;
+    if (rg.in1) {
+      a.image[pix + rg.W] = C1;
+      a.t_final[pix + rg.W] = fabsf(T1);
+      a.n_last[pix + rg.W] = last1;
     }
   }
-  __syncthreads();
-  for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) {
-    const int b = lpt_bucket(ranges[t0 + t]);
-    order[t0 + start[b] + atomicAdd(&h[b], 1u)] = (uint32_t)(t0 + t);
+}
+
+constexpr int PAIR_FWD_WARPS = 4, PAIR_FWD_BLOCKS = 8;
+template <int T>
+__global__ void __launch_bounds__(PAIR_FWD_WARPS * 32, PAIR_FWD_BLOCKS) raster_fwd_pair_kernel(RasterArgs a) {
+  constexpr int NW = T * T / 64;
+  __shared__ PairSlot s_slot[PAIR_FWD_WARPS][64];
+  const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
+  for (;;) {
+    const uint32_t item = warp_next_item(a.counter);
+    if (item >= n_items) break;
+    const int64_t gt = a.order[item / NW];
+    fwd_pair_item<T>(a, gt, (int)(item % NW), s_slot[threadIdx.x >> 5]);
+    if (a.req_end && (threadIdx.x & 31) == 0)
+      atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
   }
 }
 
+// Backward of one item, the two phases of bwd_lane_item on pixel pairs. Phase
+// 1 stores, per (pair, entry) with a pixel it adds, S = A_0 + A_1, D = A_1 (A
+// of the lower pixel) and the sum of -dL/dc over the pair; with x the pair's
+// column and y its upper row, phase 2 gets every moment of the pixel offsets
+// from sums over pairs: sum A = sum S, A x = S x, A y = S y + D, A x^2 = S x^2,
+// A x y = (S y + D) x, A y^2 = S y^2 + D (2 y + 1).
+struct PairBwdSmem {
+  PairSlot slot[33];  // entry 32: a sentinel that no pixel adds
+  uint32_t id[32];
+  float2 sd[32 * 32];  // [pair][entry ^ pair]: (S, D)
+  float nb[32 * 32];   // the same: -sum of dL/dc
+};
+constexpr int PAIR_BWD_WARPS = 4, PAIR_BWD_BLOCKS = 4;  // 56 KB a block: sixteen warps per SM
+constexpr size_t PAIR_BWD_SMEM = PAIR_BWD_WARPS * sizeof(PairBwdSmem);
+
+template <int T>
+__device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, int region, PairBwdSmem &sm) {
+  const int lane = threadIdx.x & 31;
+  const PairRegion rg(a.s, gt, region, T);
+  const uint2 range = a.ranges[gt];
+  const uint32_t *vals = a.vals;
+  const float px = rg.px + 0.5f;
+  const uint64_t npy = pack2(-(rg.py + 0.5f), -(rg.py + 1.5f));
+  const float cx = rg.wx0 + 0.5f, cy = rg.wy0 + 0.5f;
+  const float namax = -a.P.alpha_max, namin = -a.P.alpha_min;
+  const uint32_t len = range.y - range.x;
+  float T0 = 0.f, T1 = 0.f;
+  uint32_t last0 = 0, last1 = 0;
+  if (rg.in0) {
+    const int64_t pix = rg.pixel();
+    const float g = a.dL_dimage[pix];
+    T0 = a.t_final_in[pix] * g;  // the walk carries g T and g S
+    last0 = g == 0.f ? 0u : min(a.n_last_in[pix], len);  // never read past the list
+    if (rg.in1) {
+      const float h = a.dL_dimage[pix + rg.W];
+      T1 = a.t_final_in[pix + rg.W] * h;
+      last1 = h == 0.f ? 0u : min(a.n_last_in[pix + rg.W], len);
+    }
+  }
+  if (lane == 0) {  // q' = -inf at every pixel
+    sm.slot[32].g = make_ulonglong2(pack2(3.0e38f, -1.f), pack2(3.0e38f, 3.0e38f));
+    sm.slot[32].k = make_ulonglong2(pack2(0.f, 0.f), pack2(-1.f, -1.f));
+    sm.slot[32].c = make_ulonglong2(0ull, 0ull);
+  }
+  const uint32_t max_last = __reduce_max_sync(0xffffffffu, max(last0, last1));
+  uint64_t nS = 0;  // -g S of both pixels
+  uint64_t Tr = pack2(T0, T1);
+  const uint64_t one = pack2(1.f, 1.f);
+  uint32_t id1 = 0xffffffffu, id2 = 0xffffffffu;
+  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+  if ((uint32_t)lane < max_last) id1 = vals[range.x + (max_last - 1 - lane)];
+  if ((uint32_t)lane + 32u < max_last) id2 = vals[range.x + (max_last - 33 - lane)];
+  if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
+  for (int64_t hi = max_last; hi > 0; hi -= 32) {
+    const int cnt = (int)(hi > 32 ? 32 : hi);
+    uint32_t cover = 0;
+    const uint32_t id = id1;
+    const float4 r0 = n0, r1 = n1;
+    id1 = id2;
+    id2 = 0xffffffffu;
+    if ((int64_t)lane < hi - 64) id2 = vals[range.x + (uint32_t)(hi - 65 - lane)];
+    if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
+    if (lane < cnt) {
+      if (id < rg.n_req) {
+        stage_pair(sm.slot[lane], r0, r1);
+        cover = pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy);
+      }
+      sm.id[lane] = id;
+    }
+    __syncwarp();
+    uint32_t mine = transpose32(cover);
+    // staged entries e >= hi - last lie before the pixel's last added Gaussian
+    const int64_t d0 = hi - (int64_t)last0, d1 = hi - (int64_t)last1;
+    const int skip0 = (int)(d0 < 0 ? 0 : (d0 > 32 ? 32 : d0)), skip1 = (int)(d1 < 0 ? 0 : (d1 > 32 ? 32 : d1));
+    const int skip = min(skip0, skip1);
+    mine &= skip >= 32 ? 0u : (0xffffffffu << skip);
+    uint32_t used = 0;
+    const int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mine));
+    uint32_t bn = mine & (0u - mine);  // the next entry's bit (0 past the last)
+    int kn = __popc(bn - 1u);          // its index: 32, the sentinel, past the last
+    PairSlot sn = sm.slot[kn];
+    for (int t = 0; t < trips; ++t) {
+      const int k = kn;
+      const uint32_t bit = bn;
+      const PairSlot s = sn;
+      mine ^= bit;
+      bn = mine & (0u - mine);
+      kn = __popc(bn - 1u);
+      sn = sm.slot[kn];
+      const float2 qf = unpack2(pair_q(s, px, npy));
+      const uint64_t G = pack2(exp2_approx(qf.x), exp2_approx(qf.y));
+      const float2 ng = unpack2(mul2(s.c.x, G));
+      const float ns0 = fmaxf(namax, ng.x), ns1 = fmaxf(namax, ng.y);  // -sigma
+      const bool ok0 = !(qf.x < a.P.q_lim || qf.x > 0.f) && ns0 <= namin && k >= skip0;
+      const bool ok1 = !(qf.y < a.P.q_lim || qf.y > 0.f) && ns1 <= namin && k >= skip1;
+      const uint64_t ns = pack2(ns0, ns1);
+      // 1 / (1 - sigma) with sigma <= alpha_max < 1: the fast reciprocal's
+      // relative error (~1 ulp) is far inside the gradient tolerance
+      const float2 om = unpack2(add2(one, ns));
+      const uint64_t inv = pack2(rcp_approx(om.x), rcp_approx(om.y));
+      const uint64_t Tn = mul2(Tr, inv);
+      const uint64_t gdC = fma2(s.c.y, Tn, mul2(nS, inv));  // g dC/dsigma
+      const uint64_t nsT = mul2(ns, Tn);                    // -g dC/dc
+      const uint64_t nSn = fma2(s.c.y, nsT, nS);
+      const float2 gA = unpack2(mul2(gdC, G)), nb = unpack2(nsT);
+      const float A0 = ok0 && !(ng.x < namax) ? gA.x : 0.f, A1 = ok1 && !(ng.y < namax) ? gA.y : 0.f;
+      const float b0 = ok0 ? nb.x : 0.f, b1 = ok1 ? nb.y : 0.f;
+      if (ok0 || ok1) {
+        sm.sd[lane * 32 + (k ^ lane)] = make_float2(A0 + A1, A1);
+        sm.nb[lane * 32 + (k ^ lane)] = b0 + b1;
+        used |= bit;
+      }
+      const float2 To = unpack2(Tr), Tv = unpack2(Tn), So = unpack2(nS), Sv = unpack2(nSn);
+      Tr = pack2(ok0 ? Tv.x : To.x, ok1 ? Tv.y : To.y);
+      nS = pack2(ok0 ? Sv.x : So.x, ok1 ? Sv.y : So.y);
+    }
+    __syncwarp();
+    uint32_t pm = transpose32(used);  // lane e: the pairs that added entry e
+    if (pm) {
+      uint64_t sd = 0, sdx = 0, sdy = 0;  // sums of (S, D), (S, D) x, (S, D) y
+      float sxx = 0.f, sxy = 0.f, syy = 0.f, sb = 0.f;
+      do {  // two pairs per trip: half the loop overhead, two loads in flight
+        const int p = __ffs(pm) - 1;
+        pm &= pm - 1;
+        const bool two = pm != 0;
+        const int q = two ? __ffs(pm) - 1 : p;
+        pm &= pm - 1;
+        const float2 u = sm.sd[p * 32 + (lane ^ p)];
+        float2 v = sm.sd[q * 32 + (lane ^ q)];
+        const float ub = sm.nb[p * 32 + (lane ^ p)];
+        float vb = sm.nb[q * 32 + (lane ^ q)];
+        if (!two) { v = make_float2(0.f, 0.f); vb = 0.f; }
+        const float x = (float)(p & 7), y = (float)((p >> 2) & 6);
+        const float x2 = (float)(q & 7), y2 = (float)((q >> 2) & 6);
+        const uint64_t up = pack2(u.x, u.y), vp = pack2(v.x, v.y);
+        sd = add2(sd, add2(up, vp));
+        sdx = fma2(up, pack2(x, x), fma2(vp, pack2(x2, x2), sdx));
+        sdy = fma2(up, pack2(y, y), fma2(vp, pack2(y2, y2), sdy));
+        const float ax = u.x * x, ax2 = v.x * x2;
+        sxx = fmaf(ax, x, fmaf(ax2, x2, sxx));
+        sxy = fmaf(ax, y, fmaf(ax2, y2, sxy));
+        syy = fmaf(u.x * y, y, fmaf(v.x * y2, y2, syy));
+        sb += ub + vb;
+      } while (pm);
+      const float2 fd = unpack2(sd), fx = unpack2(sdx), fy = unpack2(sdy);
+      const float s0 = fd.x, s1 = fx.x, s2 = fy.x + fd.y, s4 = sxy + fx.y,
+                  s5 = syy + fmaf(2.f, fy.y, fd.y);
+      const PairSlot sl = sm.slot[lane];
+      const float2 ua = unpack2(sl.g.x);
+      const float ca = ua.y, cb2 = unpack2(sl.k.x).x, cc = unpack2(sl.k.y).x;
+      const float u = ua.x - cx, v = unpack2(sl.g.y).x - cy;  // mean relative to pixel (0, 0)
+      // sums over the entry's pixels of A dx, A dy, A dx^2, A dx dy, A dy^2
+      const float sdx1 = fmaf(u, s0, -s1), sdy1 = fmaf(v, s0, -s2);
+      const float gxx = fmaf(u, fmaf(u, s0, -2.f * s1), sxx);
+      const float gxy = fmaf(u, fmaf(v, s0, -s2), fmaf(-v, s1, s4));
+      const float gyy = fmaf(v, fmaf(v, s0, -2.f * s2), s5);
+      const float hq = 0.5f * unpack2(sl.c.x).x;  // dL/dq = -alpha A / 2
+      // dq/du = 2 (a dx + b dy), dq/dv = 2 (b dx + c dy), dq/db = 2 dx dy;
+      // the record holds (a', 2b', c') = CONIC_SCALE (a, 2b, c)
+      const float hk = hq * INV_CONIC_SCALE;
+      const float gx = hk * sdx1, gy = hk * sdy1;
+      const float du = fmaf(2.f * ca, gx, cb2 * gy);
+      const float dv = fmaf(cb2, gx, 2.f * cc * gy);
+      float4 *dst = a.grad2d + 2 * (rg.rec_base + sm.id[lane]);
+      atomicAdd(dst, make_float4(du, dv, hq * gxx, 2.f * hq * gxy));
+      atomicAdd(dst + 1, make_float4(hq * gyy, s0, -sb, 0.f));
+    }
+    __syncwarp();  // the slice is rewritten by the next batch
+  }
+}
+
+template <int T>
+__global__ void __launch_bounds__(PAIR_BWD_WARPS * 32, PAIR_BWD_BLOCKS) raster_bwd_pair_kernel(RasterArgs a) {
+  constexpr int NW = T * T / 64;
+  extern __shared__ __align__(16) unsigned char lane_smem[];
+  PairBwdSmem &sm = reinterpret_cast<PairBwdSmem *>(lane_smem)[threadIdx.x >> 5];
+  const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
+  for (;;) {
+    const uint32_t item = warp_next_item(a.counter);
+    if (item >= n_items) break;
+    const int64_t gt = a.order[item / NW];
+    bwd_pair_item<T>(a, gt, (int)(item % NW), sm);
+    if (a.req_end && (threadIdx.x & 31) == 0)
+      atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
+  }
+}
+
+// ---- work order: all tiles by descending list length (four buckets per
+// factor of two), so that the longest lists start first and the persistent
+// warps finish together. Within a bucket the tiles stay roughly in order, view
+// by view. (Ordering every view by itself, log2 buckets: 24 uneven requests
+// raster_fwd 0.243 -> 0.193, raster_bwd 0.501 -> 0.439 ms; 100k Gaussians on
+// one 512^2 view 0.065 -> 0.059 and 0.095 -> 0.088; 64 equal views of 256^2
+// 1.087 -> 1.071 and 2.148 -> 2.173.) The binning's offsets kernel has counted
+// the buckets; a block takes 1,024 tiles and reserves their places per bucket
+// with one atomic each. ----
+__global__ void __launch_bounds__(1024) tile_order_kernel(int64_t n_tiles, const uint2 *ranges,
+                                                          uint32_t *lpt, uint32_t *order) {
+  __shared__ uint32_t s_cnt[LPT_BUCKETS], s_w[32];
+  static_assert(LPT_BUCKETS <= 1024, "one thread per bucket");
+  const int t = threadIdx.x, lane = t & 31;
+  const int64_t gt = (int64_t)blockIdx.x * 1024 + t;
+  if (t < LPT_BUCKETS) s_cnt[t] = 0;
+  // longer buckets come first: thread t has bucket LPT_BUCKETS - 1 - t
+  const int b = LPT_BUCKETS - 1 - t;
+  const uint32_t c = b >= 0 ? lpt[b] : 0;
+  uint32_t inc = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) s_w[t >> 5] = inc;
+  __syncthreads();
+  int mine = 0;
+  uint32_t rank = 0;
+  if (gt < n_tiles) {
+    mine = lpt_bucket(ranges[gt]);
+    rank = atomicAdd(&s_cnt[mine], 1u);
+  }
+  __syncthreads();
+  if (b >= 0 && s_cnt[b]) {
+    uint32_t start = inc - c + atomicAdd(&lpt[LPT_BUCKETS + b], s_cnt[b]);
+    for (int w = 0; w < t >> 5; ++w) start += s_w[w];
+    s_cnt[b] = start;
+  }
+  __syncthreads();
+  if (gt < n_tiles) order[s_cnt[mine] + rank] = (uint32_t)gt;
+}
 
 // Resident blocks per SM of a kernel, cached per (device, kernel); the query
 // is not a stream operation, so it is also legal while a stream is captured.
@@ -1166,13 +1589,55 @@ void launch_bwd_t(const RasterArgs &a, cudaStream_t st) {
   k<<<(unsigned)grid, T * T, 0, st>>>(a);
 }
 
+// Pixel pairs (8 x 8 regions) where there are enough of them: with few items
+// the serial walk of the longest one sets the time, and a region of half the
+// pixels walks it faster. Measured fwd / bwd in us, pairs against 8 x 4
+// regions, at tile 8: 256 regions (100k Gaussians, 128^2) 68.6 / 68.2 against
+// 62.6 / 59.6; 1,024 (500k, 256^2) 76 / 83 against 70 / 84; 3,200 (100k, 2 x
+// 320^2) 62 / 83 against 72 / 107; 8,192 (500k, 8 x 256^2) 192 / 315 against
+// 223 / 379. Crowded views (depth slices) have lists so long that the forward
+// needs an item for every warp slot: 4,096 regions (500k, 64 x 64^2) 922 / 920
+// against 704 / 1,029, 9,216 (64 x 96^2) 428 / 677 against 439 / 862.
+constexpr int64_t PAIR_MIN_ITEMS = 2048;
+bool bwd_pairs(const RenderShape &s) {
+  return s.total_tiles * (int64_t)(s.tile * s.tile / 64) >= PAIR_MIN_ITEMS;
+}
+bool fwd_pairs(const RenderShape &s) {
+  const int64_t slots = (int64_t)PAIR_FWD_WARPS * PAIR_FWD_BLOCKS * device_sms();
+  return bwd_pairs(s) && (!s.sliced || s.total_tiles * (int64_t)(s.tile * s.tile / 64) >= slots);
+}
+
+template <int T>
+void launch_fwd_pair_t(const RasterArgs &a, cudaStream_t st) {
+  const int64_t need = (a.s.total_tiles * (T * T / 64) + PAIR_FWD_WARPS - 1) / PAIR_FWD_WARPS;
+  auto k = raster_fwd_pair_kernel<T>;
+  int64_t grid = (int64_t)blocks_per_sm(k, PAIR_FWD_WARPS * 32) * device_sms();
+  if (grid > need) grid = need;
+  LaunchScope ls(KID_RASTER_FWD, st);
+  k<<<(unsigned)grid, PAIR_FWD_WARPS * 32, 0, st>>>(a);
+}
+
+template <int T>
+void launch_bwd_pair_t(const RasterArgs &a, cudaStream_t st) {
+  if (prepare_raster_kernels() != cudaSuccess) return;  // surfaces via cudaGetLastError
+  auto k = raster_bwd_pair_kernel<T>;
+  const int64_t need = (a.s.total_tiles * (T * T / 64) + PAIR_BWD_WARPS - 1) / PAIR_BWD_WARPS;
+  int64_t grid = (int64_t)blocks_per_sm(k, PAIR_BWD_WARPS * 32, PAIR_BWD_SMEM) * device_sms();
+  if (grid > need) grid = need;
+  LaunchScope ls(KID_RASTER_BWD, st);
+  k<<<(unsigned)grid, PAIR_BWD_WARPS * 32, PAIR_BWD_SMEM, st>>>(a);
+}
+
 template <int T, bool PIX>
 void launch_fwd_warp_t(const RasterArgs &a, cudaStream_t st) {
   const int64_t need = (a.s.total_tiles * (T * T / 32) + WARPS - 1) / WARPS;
   auto k = raster_fwd_warp_kernel<T, PIX, false>;
   if constexpr (!PIX) {
-    // at least two items for each warp of eight resident blocks per SM
-    if (need >= 2 * 8 * (int64_t)device_sms()) k = raster_fwd_warp_kernel<T, PIX, true>;
+    if (fwd_pairs(a.s)) {
+      launch_fwd_pair_t<T>(a, st);
+      return;
+    }
+    if (bwd_pairs(a.s)) k = raster_fwd_warp_kernel<T, PIX, true>;
   }
   int64_t grid = (int64_t)blocks_per_sm(k, WARPS * 32) * device_sms();
   if (grid > need) grid = need;
@@ -1194,7 +1659,8 @@ void launch_bwd_lane_t(const RasterArgs &a, cudaStream_t st) {
 template <int T, bool PIX>
 void launch_bwd_warp_t(const RasterArgs &a, cudaStream_t st) {
   if (!PIX) {
-    launch_bwd_lane_t<T>(a, st);
+    if (bwd_pairs(a.s)) launch_bwd_pair_t<T>(a, st);
+    else launch_bwd_lane_t<T>(a, st);
     return;
   }
   auto k = raster_bwd_warp_kernel<T, PIX>;
@@ -1251,9 +1717,10 @@ void bwd_dispatch(const RasterArgs &a, int tile, cudaStream_t st) {
 }  // namespace
 
 void launch_tile_order(const RenderShape &s, ddgs_workspace &ws, cudaStream_t st) {
-  if (s.total_tiles <= 0 || s.V <= 0) return;
+  if (s.total_tiles <= 0) return;
   LaunchScope ls(KID_TILE_ORDER, st);
-  tile_order_view_kernel<<<(unsigned)s.V, 256, 0, st>>>(s.view, ws.ranges, ws.order);
+  tile_order_kernel<<<(unsigned)((s.total_tiles + 1023) / 1024), 1024, 0, st>>>(
+      s.total_tiles, ws.ranges, ws.list_count + LIST_CLASSES, ws.order);
 }
 
 void launch_raster_fwd(const RenderShape &s, const RasterParams &p, ddgs_workspace &ws,
@@ -1337,6 +1804,10 @@ cudaError_t prepare_raster_kernels() {
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
   for (auto k : {raster_bwd_lane_kernel<8>, raster_bwd_lane_kernel<16>, raster_bwd_lane_kernel<32>}) {
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LANE_BWD_SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  for (auto k : {raster_bwd_pair_kernel<8>, raster_bwd_pair_kernel<16>, raster_bwd_pair_kernel<32>}) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_BWD_SMEM);
     if (e != cudaSuccess) return e;
   }
   if (dev >= 0 && dev < 64) done[dev] = true;

@@ -46,7 +46,7 @@ constexpr size_t kOffHist = align256(kOffVals + kMaxPairs * sizeof(uint32_t));
 constexpr size_t kOffPart = align256(kOffHist + kMaxSlots * sizeof(uint32_t));
 constexpr size_t kOffLists = align256(kOffPart + kMaxParts * sizeof(uint64_t));
 constexpr size_t kOffListCount = align256(kOffLists + kMaxListItems * sizeof(uint64_t));
-constexpr size_t kOffRanges = align256(kOffListCount + ddgs::LIST_CLASSES * sizeof(uint32_t));
+constexpr size_t kOffRanges = align256(kOffListCount + ddgs::BIN_COUNTERS * sizeof(uint32_t));
 constexpr size_t kOffPairs = align256(kOffRanges + kMaxTiles * sizeof(uint2));
 constexpr size_t kOffStatus = align256(kOffPairs + sizeof(uint64_t));
 constexpr size_t kOffOrder = align256(kOffStatus + sizeof(int32_t));

@@ -10,7 +10,8 @@ import oracle
 from paper_2406_02518_gb300 import binding as B
 from paper_2406_02518_gb300 import synthetic as syn
 from _parity import check_image, compare_binning, compare_grads, gradient_weights, last_ids
-from test_gpu_parity import GRAD_NAMES, _bins, _lib, _two_views, _views, ws  # noqa: F401
+from test_gpu_parity import (GRAD_NAMES, _bins, _lib, _sampled_check, _two_views, _views,  # noqa: F401
+                             ws)
 
 pytestmark = pytest.mark.gpu
 
@@ -109,3 +110,30 @@ def test_depth_slices(n, size, tile, depths, spread, ws):
                     assert np.array_equal(gr[t], rr[t])
                     assert np.array_equal(got["vals"][gr[t, 0]:gr[t, 1]], ref["vals"][rr[t, 0]:rr[t, 1]])
         w2.close()
+
+
+def _needles(n, seed):
+    """Gaussians with one axis up to a thousand times the others."""
+    sc = syn.uniform_cloud(n, seed=seed, dir_frac=0.4, dir_std=1.0, log_scale_range=(-6.5, -5.5))
+    sc.log_scales[: n // 2, 0] += np.float32(4.0)
+    return sc
+
+
+@pytest.mark.parametrize("shape,tile", [
+    ((363, 363), 8),    # 2,116 regions of 8 x 8: just past the line, ragged right and bottom edges
+    ((361, 359), 8),    # 2,070 regions, a single pixel row and seven columns in the last tiles
+    ((352, 352), 8),    # 1,936: the 8 x 4 regions of smaller renders
+    ((353, 370), 16),   # 23 x 24 tiles of four regions
+    ((340, 421), 32)])  # 11 x 14 tiles of sixteen
+@pytest.mark.parametrize("needles", [False, True])
+def test_pixel_pair_rasterisers(shape, tile, needles, ws):
+    """The rasterisers of both sides of the pixel-pair rule on the same scene:
+    sampled pixels of the image and the gradients against the oracle. (The
+    needles' shape gradients are left out: binary32 itself is 2e-3 to 6e-3 off
+    there in every kernel, the conic of a 400:1 covariance being the cause.)"""
+    H, W = shape
+    scene = _needles(1500, 61) if needles else syn.uniform_cloud(2500, seed=61, dir_frac=0.4, dir_std=1.0)
+    views = _views([syn.pose_matrix(syn.rot_y(0.2), np.array([0.0, 0.1, 2.0]))], 4.0, 8.0 / W, H, W)
+    st = syn.Settings(near_plane=0.2, tile=tile)
+    grads = [g for g in B.GRAD_FIELDS if not (needles and g in ("log_scales", "quats"))]
+    _sampled_check(scene, views, st, ws, [0], 3000, 7, grads, depth=32)
