@@ -394,7 +394,6 @@ struct ddgs_workspace {
   uint32_t *order = nullptr;     // [tiles] work order of the persistent rasterisers
   uint32_t *queue = nullptr;     // work-queue heads of the forward / backward rasterisers
   unsigned long long *req_time = nullptr;  // [1 + 2 R]: batch start, per-request fwd / bwd ends
-  int batch_depth = 256;         // list entries staged per round in the rasterisers
   // scalars
   uint64_t *d_pairs = nullptr;   // device pair count M
   uint64_t *h_pairs = nullptr;   // pinned host mirror

@@ -1,11 +1,12 @@
 // raster.cu -- per-tile front-to-back blending (Eq. 1) and its backward pass.
 //
-// One thread block renders one (view, tile) list; one thread owns one pixel.
-// Warps own 8 x 4 pixel blocks, so a Gaussian whose q <= q_max ellipse misses
-// a warp's block is skipped by the whole warp with one uniform test. Gaussians
-// of the list are staged in shared memory one batch (one per thread) at a
-// time: the batch is a gather by Gaussian index from the per-view records,
-// which is why it uses plain vector loads rather than a bulk tensor copy.
+// Persistent kernels: every warp takes a (tile, pixel region) item from a work
+// queue ordered by list length, stages the tile's list 32 entries at a time in
+// its own slice of shared memory and never waits for another warp. A region is
+// 8 x 8 pixels, two per lane (the pixel-pair kernels), or 8 x 4 pixels, one per
+// lane, for renders of few regions. Staging is a gather by Gaussian index from
+// the per-view records, which is why it uses plain vector loads rather than a
+// bulk tensor copy.
 //
 // Forward per pixel p, over the list in ascending depth (Eq. 1):
 //   q = (p - mu-hat)^T conic (p - mu-hat); skip if q > q_max;
@@ -17,15 +18,25 @@
 // the suffix sum S = sum over later Gaussians of c sigma T:
 //   dC/dc = sigma T,  dC/dsigma = c T - S / (1 - sigma),
 //   dsigma/dalpha = G and dsigma/dq = -alpha G / 2 unless sigma was clamped.
-// The per-pixel 2D gradients of one Gaussian are summed over the warp with
-// shuffles, over the block in shared memory, and reach global memory with one
-// vector atomic per (tile, Gaussian).
+// The per-pixel 2D gradients of one Gaussian are summed over the region in
+// registers (a lane per entry) and reach global memory with one vector atomic
+// per (region, Gaussian).
+//
+// The tile edge T fixes the lists, not the regions: in tiles of 16 or 32 pixels
+// most entries of a list miss a given region, so the entries that cover a pixel
+// of it are collected first (EntryStream, Picker) and a batch is 32 of those.
+// (Blocks of T x T threads that staged 128 to 512 entries for all their warps,
+// each warp testing every entry against its four 4 x 2 quarters, were the former
+// default for these tiles: 100k Gaussians, three 375 x 501 views at T = 16:
+// forward 176 -> 112, backward 358 -> 190 us. The staging depth a caller asks
+// for no longer selects a kernel.)
 //
 // PIX = true renders the Eq. 3 variant whose ray angles are each pixel's own:
 // a record then carries (a, h) instead of a colour, and the pair's colour is
 // c = sigmoid(a + Y_1(d_p) . h) with d_p the pixel ray's unit direction. The
-// backward pass sums dL/dz (z the logit) and dL/dh per (tile, Gaussian) and
+// backward pass sums dL/dz (z the logit) and dL/dh per (region, Gaussian) and
 // adds the pose gradient through each pixel's ray.
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <utility>
@@ -100,454 +111,7 @@ __device__ __forceinline__ float4 ellipse_box(float4 r0, float4 r1, float q_max)
   return make_float4(r0.x - e.x, r0.x + e.x, r0.y - e.y, r0.y + e.y);
 }
 
-__device__ __forceinline__ float4 empty_box() {
-  return make_float4(__int_as_float(0x7f800000), -__int_as_float(0x7f800000),
-                     __int_as_float(0x7f800000), -__int_as_float(0x7f800000));
-}
-
-// A warp's 8 x 4 pixels are split into groups of GW x 2 pixels, one lane per
-// pixel: four 4 x 2 quarters of 8 lanes (GW = 4) or eight 2 x 2 groups of 4
-// lanes (GW = 2, the warp-streamed forward). Each group walks only the list
-// entries whose box meets it. Smaller groups skip more entries but take more
-// ballots per batch; the backward keeps quarters, whose 8-lane gradient
-// reduction leaves one shared-memory accumulator update per lane (2 x 2 groups
-// measured slower there: 4.71 -> 4.95 ms at 64 poses, forward 1.99 -> 1.89).
-template <int T, int GW = 4>
-struct TileGeom {
-  static_assert(GW == 2 || GW == 4, "groups are 4 x 2 or 2 x 2 pixels");
-  static constexpr int LG = 2 * GW;  // lanes per group
-  static constexpr int NG = 32 / LG; // groups per warp
-  static constexpr int GX = 8 / GW;  // groups per pixel row of the warp
-  int v, txi, tyi, px, py, wx0, wy0, H, W;
-  bool inside;
-  int64_t gtile, rec_base, img_off, n_req;
-  // region: which 8 x 4 pixel block of the tile this warp owns
-  __device__ __forceinline__ TileGeom(const RenderShape &s, int64_t gt, int region) {
-    gtile = gt;
-    v = find_view(s.view, s.V, gt);
-    const ViewTab vt = s.view[v];
-    H = vt.H;
-    W = vt.W;
-    rec_base = vt.rec_off;
-    img_off = vt.img_off;
-    n_req = s.req[vt.req].n;
-    const int64_t local = gt - vt.tile_base;
-    tyi = (int)(local / vt.tiles_x);
-    txi = (int)(local - (int64_t)tyi * vt.tiles_x);
-    constexpr int WX = T / 8;
-    const int lane = threadIdx.x & 31;
-    const int wx = region % WX, wy = region / WX;
-    wx0 = txi * T + wx * 8;
-    wy0 = tyi * T + wy * 4;
-    const int g = lane / LG;
-    px = wx0 + (g % GX) * GW + lane % GW;
-    py = wy0 + (g / GX) * 2 + (lane / GW) % 2;
-    inside = px < W && py < H;
-  }
-  __device__ __forceinline__ int64_t pixel() const { return img_off + (int64_t)py * W + px; }
-  // does the box miss the GW x 2 pixel centres of group q of this warp?
-  __device__ __forceinline__ bool misses_q(float4 b, int q) const {
-    const float x0 = (float)(wx0 + (q % GX) * GW), y0 = (float)(wy0 + (q / GX) * 2);
-    return b.x > x0 + (GW - 0.5f) || b.y < x0 + 0.5f || b.z > y0 + 1.5f || b.w < y0 + 0.5f;
-  }
-};
-
-// Each lane tests list entry c0 + lane of the staged batch against the four
-// quarters of its warp (ok: the entry exists and passes the caller's test);
-// returns the entries this lane's quarter must evaluate, in list order.
-template <int T>
-__device__ __forceinline__ uint32_t quarter_todo(const TileGeom<T> &tg, float4 box, bool ok) {
-  static_assert(TileGeom<T>::NG == 4, "four quarters of 8 lanes");
-  const int q = (threadIdx.x & 31) >> 3;
-  const uint32_t m0 = __ballot_sync(0xffffffffu, ok && !tg.misses_q(box, 0));
-  const uint32_t m1 = __ballot_sync(0xffffffffu, ok && !tg.misses_q(box, 1));
-  const uint32_t m2 = __ballot_sync(0xffffffffu, ok && !tg.misses_q(box, 2));
-  const uint32_t m3 = __ballot_sync(0xffffffffu, ok && !tg.misses_q(box, 3));
-  return q == 0 ? m0 : (q == 1 ? m1 : (q == 2 ? m2 : m3));
-}
-
-// One (view, tile) work item of the forward pass; BATCH list entries are
-// staged in shared memory per round.
-template <int T, int BATCH, bool PIX>
-__device__ __forceinline__ void fwd_tile(const RasterArgs &a, int64_t gt, float4 *s_a, float4 *s_b,
-                                         float4 *s_box, float4 *s_c) {
-  constexpr int NT = T * T;
-  const int tid = threadIdx.x;
-  const TileGeom<T> tg(a.s, gt, threadIdx.x >> 5);
-  const uint2 range = a.ranges[tg.gtile];
-  const uint32_t *vals = a.vals;
-  const int64_t rec_base = tg.rec_base;
-  const float px = tg.px + 0.5f, py = tg.py + 0.5f;
-  PixRay ray;
-  if (PIX) pixel_ray(a.world_to_cam + 12 * tg.v, a.detector + 5 * tg.v, tg.H, tg.W, px, py, ray);
-  float Tr = 1.f, C = 0.f;
-  uint32_t last = 0;
-  bool done = !tg.inside;
-  for (uint32_t b0 = range.x; b0 < range.y; b0 += BATCH) {
-    if (__syncthreads_count(done) == NT) break;
-    for (int e = tid; e < BATCH; e += NT) {
-      const uint32_t j = b0 + e;
-      if (j < range.y) {
-        const uint32_t id = vals[j];
-        if (id < tg.n_req) {
-          const int64_t r = rec_base + id;
-          const float4 r0 = a.rec[2 * r], r1 = a.rec[2 * r + 1];
-          s_a[e] = r0;
-          s_b[e] = r1;
-          s_box[e] = ellipse_box(r0, r1, a.P.q_max);
-          if (PIX) s_c[e] = a.rec2[r];
-        } else {
-          s_box[e] = empty_box();  // only after a capacity overflow
-        }
-      }
-    }
-    __syncthreads();
-    const int cnt = (int)min((uint32_t)BATCH, range.y - b0);
-    // 32 entries at a time: each lane tests one entry's box against the four
-    // quarters of its warp; each quarter then walks its own entries, so one
-    // instruction serves up to four (quarter, entry) pairs.
-    const int lane = threadIdx.x & 31;
-    for (int c0 = 0; c0 < cnt; c0 += 32) {
-      const uint32_t dmask = __ballot_sync(0xffffffffu, done);
-      if (dmask == 0xffffffffu) break;
-      const int ec = c0 + lane;
-      const float4 box = ec < cnt ? s_box[ec] : empty_box();
-      uint32_t mine = quarter_todo<T>(tg, box, ec < cnt);
-      if (((dmask >> (lane & 24)) & 0xffu) == 0xffu) mine = 0;  // quarter finished
-      while (__any_sync(0xffffffffu, mine != 0)) {
-        if (mine == 0) continue;
-        const int k = c0 + __ffs(mine) - 1;
-        mine &= mine - 1;
-        if (done) continue;
-        const float4 A = s_a[k], B = s_b[k];
-        PairEval e;
-        if (!eval_pair(A.x, A.y, A.z, A.w, B.x, B.y, px, py, a.P, e)) continue;
-        const float Tn = __fmaf_rn(-Tr, e.sigma, Tr);  // T (1 - sigma)
-        if (Tn < a.P.t_min) {
-          done = true;
-          continue;
-        }
-        const float col = PIX ? pixel_colour(ray, s_c[k]) : B.z;
-        C = fmaf(col * e.sigma, Tr, C);
-        Tr = Tn;
-        last = b0 + (uint32_t)k - range.x + 1u;
-      }
-    }
-  }
-  if (tg.inside) {
-    const int64_t pix = tg.pixel();
-    a.image[pix] = C;
-    a.t_final[pix] = Tr;
-    a.n_last[pix] = last;
-  }
-}
-
-// Persistent forward rasteriser: each block takes work items from the queue
-// (longest tile lists first) until it is empty.
-// Minimum resident blocks per SM requested from the register allocator: six
-// 256-thread blocks (40 registers) for the forward, five (48) for the backward.
-template <int T>
-constexpr int fwd_min_blocks() { return T == 16 ? 6 : (T == 8 ? 16 : 1); }
-template <int T>
-constexpr int bwd_min_blocks() { return T == 16 ? 5 : (T == 8 ? 12 : 1); }
-
-template <int T, int BATCH, bool PIX>
-__global__ void __launch_bounds__(T *T, fwd_min_blocks<T>()) raster_fwd_kernel(RasterArgs a) {
-  __shared__ float4 s_a[BATCH], s_b[BATCH], s_box[BATCH], s_c[PIX ? BATCH : 1];
-  __shared__ uint32_t s_item;
-  for (;;) {
-    __syncthreads();  // the previous item is finished by every thread
-    if (threadIdx.x == 0) s_item = atomicAdd(a.counter, 1u);
-    __syncthreads();
-    const uint32_t item = s_item;
-    if (item >= (uint32_t)a.s.total_tiles) break;
-    const int64_t gt = a.order[item];
-    fwd_tile<T, BATCH, PIX>(a, gt, s_a, s_b, s_box, s_c);
-    if (a.req_end && threadIdx.x == 0)
-      atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
-  }
-}
-
-// Sum 8 per-lane values over each group of 8 lanes (a quarter) with 7
-// shuffles. Afterwards lane l of the quarter holds in v[0] the quarter's total
-// of component ((l >> 2) & 1) * 4 + ((l >> 1) & 1) * 2 + (l & 1), returned.
-__device__ __forceinline__ int quarter_reduce8(float v[8]) {
-  const int lane = threadIdx.x & 31;
-  bool hi = lane & 4;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float send = hi ? v[k] : v[k + 4];
-    float keep = hi ? v[k + 4] : v[k];
-    v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  hi = lane & 2;
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    float send = hi ? v[k] : v[k + 2];
-    float keep = hi ? v[k + 2] : v[k];
-    v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-  }
-  hi = lane & 1;
-  {
-    float send = hi ? v[0] : v[1];
-    float keep = hi ? v[1] : v[0];
-    v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-  }
-  return ((lane >> 2) & 1) * 4 + ((lane >> 1) & 1) * 2 + (lane & 1);
-}
-
-// Sum 10 per-lane values over each quarter (8 lanes) with 10 shuffles: v[8]
-// and v[9] first (lanes with l % 4 == 0 end with component 8, if bit 2 of the
-// lane is clear, or 9 in v[8]), then v[0..7] as quarter_reduce8 (lane l ends
-// with the component it returns in v[0]).
-__device__ __forceinline__ int quarter_reduce10(float v[10]) {
-  const int lane = threadIdx.x & 31;
-  const bool hi = lane & 4;
-  const float send = hi ? v[8] : v[9], keep = hi ? v[9] : v[8];
-  float w = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  w += __shfl_xor_sync(0xffffffffu, w, 2);
-  w += __shfl_xor_sync(0xffffffffu, w, 1);
-  v[8] = w;
-  return quarter_reduce8(v);
-}
-
-// Accumulated components per (tile, Gaussian): u, v, conic a, b, c, alpha and
-// the colour (or, with PIX, the logit z and h_0..h_2).
-template <bool PIX>
-constexpr int n_acc() { return PIX ? 12 : 8; }
-
-template <int BATCH, bool PIX>
-struct BwdSmem {
-  float4 a[BATCH], b[BATCH], box[BATCH], c[PIX ? BATCH : 1];
-  uint32_t id[BATCH];
-  float acc[BATCH][n_acc<PIX>()];
-  float pose[PIX ? 12 : 1];  // per-tile pose gradient through the pixel rays
-  uint32_t max_last;
-};
-
-// One (view, tile) work item of the backward pass.
-template <int T, int BATCH, bool PIX>
-__device__ __forceinline__ void bwd_tile(const RasterArgs &a, int64_t gt, BwdSmem<BATCH, PIX> &sm) {
-  float4 *s_a = sm.a, *s_b = sm.b, *s_box = sm.box, *s_c = sm.c;
-  uint32_t *s_id = sm.id;
-  float (*s_acc)[n_acc<PIX>()] = sm.acc;
-  uint32_t &s_max = sm.max_last;
-  constexpr int NT = T * T;
-  const int tid = threadIdx.x;
-  const TileGeom<T> tg(a.s, gt, threadIdx.x >> 5);
-  const uint2 range = a.ranges[tg.gtile];
-  const uint32_t *vals = a.vals;
-  const int64_t rec_base = tg.rec_base;
-  const float px = tg.px + 0.5f, py = tg.py + 0.5f;
-  PixRay ray;
-  float gY[3] = {0.f, 0.f, 0.f};  // dL/dY_1 of this pixel's ray
-  if (PIX) pixel_ray(a.world_to_cam + 12 * tg.v, a.detector + 5 * tg.v, tg.H, tg.W, px, py, ray);
-  float Tr = 1.f, g = 0.f;
-  uint32_t last = 0;
-  if (tg.inside) {
-    const int64_t pix = tg.pixel();
-    Tr = a.t_final_in[pix];
-    last = a.n_last_in[pix];
-    g = a.dL_dimage[pix];
-  }
-  if (g == 0.f) last = 0;  // nothing to propagate from this pixel
-  if (last > range.y - range.x) last = range.y - range.x;  // never read past the list
-  if (tid == 0) s_max = 0;
-  __syncthreads();
-  if (last) atomicMax(&s_max, last);
-  __syncthreads();
-  const uint32_t max_last = s_max;
-  // last list position any pixel of each quarter added (every lane learns all four)
-  uint32_t qlast = last;
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) qlast = max(qlast, __shfl_xor_sync(0xffffffffu, qlast, o));
-  const uint32_t ql0 = __shfl_sync(0xffffffffu, qlast, 0), ql1 = __shfl_sync(0xffffffffu, qlast, 8);
-  const uint32_t ql2 = __shfl_sync(0xffffffffu, qlast, 16), ql3 = __shfl_sync(0xffffffffu, qlast, 24);
-  float S = 0.f;
-  for (int64_t hi = max_last; hi > 0; hi -= BATCH) {
-    const int64_t lo = hi > BATCH ? hi - BATCH : 0;
-    for (int e = tid; e < BATCH; e += NT) {
-      const int64_t pos_t = hi - 1 - e;  // batches run back to front
-      if (pos_t >= lo) {
-        const uint32_t id = vals[range.x + (uint32_t)pos_t];
-        if (id < tg.n_req) {
-          const int64_t r = rec_base + id;
-          const float4 r0 = a.rec[2 * r], r1 = a.rec[2 * r + 1];
-          s_a[e] = r0;
-          s_b[e] = r1;
-          s_box[e] = ellipse_box(r0, r1, a.P.q_max);
-          if (PIX) s_c[e] = a.rec2[r];
-        } else {
-          s_box[e] = empty_box();  // only after a capacity overflow
-        }
-        s_id[e] = id;
-      }
-#pragma unroll
-      for (int c = 0; c < n_acc<PIX>(); ++c) s_acc[e][c] = 0.f;
-    }
-    __syncthreads();
-    const int cnt = (int)(hi - lo);
-    const int lane = threadIdx.x & 31;
-    for (int c0 = 0; c0 < cnt; c0 += 32) {
-      // each lane tests one entry against the four quarters: inside the
-      // quarter's box and before the last Gaussian the quarter added
-      const int ec = c0 + lane;
-      const bool ok = ec < cnt;
-      const float4 box = ok ? s_box[ec] : empty_box();
-      const uint32_t pe = (uint32_t)(hi - 1 - ec);
-      const uint32_t m0 = __ballot_sync(0xffffffffu, ok && pe < ql0 && !tg.misses_q(box, 0));
-      const uint32_t m1 = __ballot_sync(0xffffffffu, ok && pe < ql1 && !tg.misses_q(box, 1));
-      const uint32_t m2 = __ballot_sync(0xffffffffu, ok && pe < ql2 && !tg.misses_q(box, 2));
-      const uint32_t m3 = __ballot_sync(0xffffffffu, ok && pe < ql3 && !tg.misses_q(box, 3));
-      const int qi = lane >> 3;
-      uint32_t mine = qi == 0 ? m0 : (qi == 1 ? m1 : (qi == 2 ? m2 : m3));
-      while (__any_sync(0xffffffffu, mine != 0)) {
-        const bool has = mine != 0;
-        const int k = has ? c0 + __ffs(mine) - 1 : c0;
-        if (has) mine &= mine - 1;
-        const uint32_t pos = (uint32_t)(hi - 1 - k);
-        float gv[PIX ? 10 : 8];
-#pragma unroll
-        for (int c = 0; c < (PIX ? 10 : 8); ++c) gv[c] = 0.f;
-        bool act = has && pos < last;
-        if (act) {
-          const float4 A = s_a[k], B = s_b[k];
-          PairEval e;
-          act = eval_pair(A.x, A.y, A.z, A.w, B.x, B.y, px, py, a.P, e);
-          if (act) {
-            // 1 / (1 - sigma) with sigma <= alpha_max < 1: the fast reciprocal's
-            // relative error (~1 ulp) is far inside the gradient tolerance
-            const float inv_om = rcp_approx(__fsub_rn(1.f, e.sigma));
-            Tr = Tr * inv_om;  // transmittance before this Gaussian
-            float4 cz;
-            if (PIX) cz = s_c[k];
-            const float c = PIX ? pixel_colour(ray, cz) : B.z;
-            const float dC_dsigma = fmaf(c, Tr, -S * inv_om);
-            S = fmaf(c * e.sigma, Tr, S);
-            const float gs = g * dC_dsigma;
-            float gq = 0.f;
-            if (!(e.aG > a.P.alpha_max)) {
-              gv[5] = gs * e.G;
-              gq = -0.5f * gs * B.y * e.G;
-            }
-            // sums of gq dx, gq dy, gq dx^2, gq dx dy and gq dy^2; the mean and
-            // conic gradients are formed from them once per entry (below)
-            const float gdx = gq * e.dx, gdy = gq * e.dy;
-            gv[0] = gdx;
-            gv[1] = gdy;
-            gv[2] = gdx * e.dx;
-            gv[3] = gdx * e.dy;
-            gv[4] = gdy * e.dy;
-            const float dcol = g * e.sigma * Tr;  // dL/dc
-            if (PIX) {
-              const float dz = dcol * c * (1.f - c);
-              gv[6] = dz;
-              gv[7] = dz * ray.Y[0];
-              gv[8] = dz * ray.Y[1];
-              gv[9] = dz * ray.Y[2];
-              gY[0] = fmaf(dz, cz.y, gY[0]);
-              gY[1] = fmaf(dz, cz.z, gY[1]);
-              gY[2] = fmaf(dz, cz.w, gY[2]);
-            } else {
-              gv[6] = dcol;
-            }
-          }
-        }
-        // sum the quarter's 8 lanes (each quarter has its own entry k)
-        if (__any_sync(0xffffffffu, act)) {
-          if (PIX) {
-            const int comp = quarter_reduce10(gv);
-            if (has) {
-              if (gv[0] != 0.f) atomicAdd(&s_acc[k][comp], gv[0]);
-              if ((lane & 3) == 0 && gv[8] != 0.f) atomicAdd(&s_acc[k][(lane & 4) ? 9 : 8], gv[8]);
-            }
-          } else {
-            const int comp = quarter_reduce8(gv);
-            if (has && gv[0] != 0.f) atomicAdd(&s_acc[k][comp], gv[0]);
-          }
-        }
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < cnt; e += NT) {
-      const float *acc = s_acc[e];
-      bool nz = (acc[0] != 0.f) | (acc[1] != 0.f) | (acc[2] != 0.f) | (acc[3] != 0.f) |
-                (acc[4] != 0.f) | (acc[5] != 0.f) | (acc[6] != 0.f);
-      if (PIX) nz |= (acc[7] != 0.f) | (acc[8] != 0.f) | (acc[9] != 0.f);
-      if (nz) {
-        float4 *dst = a.grad2d + 2 * (rec_base + s_id[e]);
-        // dq/du = 2 (a dx + b dy), dq/dv = 2 (b dx + c dy), dq/db = 2 dx dy
-        // the record holds CONIC_SCALE (a, 2b, c)
-        const float ca = s_a[e].z * INV_CONIC_SCALE, cb = (0.5f * INV_CONIC_SCALE) * s_a[e].w,
-                    cc = s_b[e].x * INV_CONIC_SCALE;
-        const float du = 2.f * fmaf(ca, acc[0], cb * acc[1]);
-        const float dv = 2.f * fmaf(cb, acc[0], cc * acc[1]);
-        atomicAdd(dst, make_float4(du, dv, acc[2], 2.f * acc[3]));
-        atomicAdd(dst + 1, make_float4(acc[4], acc[5], acc[6], 0.f));
-        if (PIX) atomicAdd(a.grad_h + rec_base + s_id[e], make_float4(acc[7], acc[8], acc[9], 0.f));
-      }
-    }
-    __syncthreads();
-  }
-  if (PIX && a.pose_grad) {
-    // Y_1(d / |d|), d = W^T rc: dL/dW[r][c] = rc[r] dL/dd[c]
-    float w9[9];
-    const bool mine = tg.inside && ((gY[0] != 0.f) | (gY[1] != 0.f) | (gY[2] != 0.f));
-    const float ddh[3] = {-SH_C1 * gY[2], -SH_C1 * gY[0], SH_C1 * gY[1]};
-    const float dot = ddh[0] * ray.dh[0] + ddh[1] * ray.dh[1] + ddh[2] * ray.dh[2];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float dd = mine ? (ddh[c] - ray.dh[c] * dot) * ray.inv : 0.f;
-#pragma unroll
-      for (int r = 0; r < 3; ++r) w9[3 * r + c] = ray.rc[r] * dd;
-    }
-    if (__any_sync(0xffffffffu, mine)) {
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) w9[i] += __shfl_xor_sync(0xffffffffu, w9[i], o);
-      }
-      if ((tid & 31) == 0)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) atomicAdd(&sm.pose[i], w9[i]);
-    }
-    __syncthreads();
-    if (tid < 9) {
-      const float x = sm.pose[tid];
-      if (x != 0.f) atomicAdd(a.pose_grad + 12 * (int64_t)tg.v + 4 * (tid / 3) + tid % 3, x);
-      sm.pose[tid] = 0.f;
-    }
-  }
-}
-
-template <int T, int BATCH, bool PIX>
-__global__ void __launch_bounds__(T *T, bwd_min_blocks<T>()) raster_bwd_kernel(RasterArgs a) {
-  __shared__ BwdSmem<BATCH, PIX> sm;
-  __shared__ uint32_t s_item;
-  if (PIX && threadIdx.x < 12) sm.pose[threadIdx.x] = 0.f;
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_item = atomicAdd(a.counter, 1u);
-    __syncthreads();
-    const uint32_t item = s_item;
-    if (item >= (uint32_t)a.s.total_tiles) break;
-    const int64_t gt = a.order[item];
-    bwd_tile<T, BATCH, PIX>(a, gt, sm);
-    if (a.req_end && threadIdx.x == 0)
-      atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
-  }
-}
-
-// ---- warp-streamed rasterisers (staging depth 32) ----
-// Every warp takes its own (tile, 8 x 4 region) item from the queue, stages 32
-// list entries at a time in its own slice of shared memory and never waits
-// for the other warps of its block. Item i is region i % NW of tile
-// order[i / NW] (NW = regions per tile), so the regions of one tile are taken
-// together and share its list in L1/L2. The backward sums a batch's 2D
-// gradients per entry in the warp's slice and sends the non-zero sums to
-// global memory with vector atomics.
-
-constexpr int WARPS = 8;  // warps per block of the warp-streamed kernels
+constexpr int WARPS = 8;  // warps per block of the 8 x 4 kernels
 
 __device__ __forceinline__ uint32_t warp_next_item(uint32_t *counter) {
   uint32_t it = 0;
@@ -576,6 +140,122 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x) {
     x = (lane & d) ? ((x & ~LO[r]) | ((y >> d) & LO[r])) : ((x & LO[r]) | ((y << d) & ~LO[r]));
   }
   return x;
+}
+
+// A tile list (or its first n entries) in walk order, 32 entries at a time: front
+// to back, or back to front (BACK). Lane l holds the record of walk index j + l;
+// the ids one chunk ahead and the records of the chunk held are in flight while
+// earlier ones are used.
+constexpr uint32_t NO_ENTRY = 0xffffffffu;
+template <bool BACK>
+struct EntryStream {
+  const uint32_t *vals;
+  const float4 *rec;
+  int64_t n_req;
+  uint32_t n, j;
+  uint32_t id, id_next;
+  float4 r0, r1;
+  __device__ __forceinline__ uint32_t load_id(uint32_t i) const {
+    return i < n ? vals[BACK ? n - 1u - i : i] : NO_ENTRY;
+  }
+  // an id past n_req: no entry, or garbage after a capacity overflow
+  __device__ __forceinline__ bool valid(uint32_t i) const { return (int64_t)i < n_req; }
+  __device__ __forceinline__ void load_rec() {
+    if (valid(id)) {
+      r0 = rec[2 * (int64_t)id];
+      r1 = rec[2 * (int64_t)id + 1];
+    }
+  }
+  __device__ __forceinline__ EntryStream(const uint32_t *list, uint32_t len, const float4 *records, int64_t nr)
+      : vals(list), rec(records), n_req(nr), n(len), j(0) {
+    const uint32_t lane = threadIdx.x & 31;
+    id = load_id(lane);
+    id_next = load_id(32u + lane);
+    r0 = r1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    load_rec();
+  }
+  __device__ __forceinline__ bool more() const { return j < n; }
+  __device__ __forceinline__ void next() {
+    j += 32u;
+    id = id_next;
+    id_next = load_id(j + 32u + (threadIdx.x & 31));
+    load_rec();
+  }
+};
+
+// Collects 32 entries whose cover of the region is not empty from a stream
+// (fewer at its end). An entry that no longer fits the batch stays with its
+// lane for the next one. PICK = false: every entry is taken (8 x 8 regions of
+// T = 8 lists, where nearly all cover the region), and slot k of batch b is
+// walk index 32 b + k.
+template <bool PICK>
+struct Picker {
+  float4 c0, c1;
+  uint32_t id, j, cover;
+  __device__ __forceinline__ Picker() : id(NO_ENTRY), j(0), cover(0) {}
+  // stage(slot, r0, r1, id, j) writes an entry; cov(r0, r1) is its cover mask;
+  // s_cover, s_j: [32]. Returns the number of slots filled; `mask` is the cover
+  // of slot `lane`.
+  template <class Stream, class Cov, class Stage>
+  __device__ __forceinline__ int fill(Stream &st, uint32_t *s_cover, uint32_t *s_j, Cov cov,
+                                      Stage stage, uint32_t &mask) {
+    const uint32_t lane = threadIdx.x & 31;
+    mask = 0;
+    if constexpr (!PICK) {
+      const int cnt = (int)min(32u, st.n - st.j);
+      const uint32_t i = st.id, w = st.j + lane;
+      const float4 r0 = st.r0, r1 = st.r1;
+      st.next();
+      if (st.valid(i)) {
+        stage((int)lane, r0, r1, i, w);
+        mask = cov(r0, r1);
+      }
+      __syncwarp();
+      return cnt;
+    } else {
+      int n = 0;
+      for (;;) {
+        const uint32_t bal = __ballot_sync(0xffffffffu, cover != 0);
+        if (bal == 0) {
+          if (!st.more()) break;
+          id = st.id;
+          j = st.j + lane;
+          c0 = st.r0;
+          c1 = st.r1;
+          st.next();
+          cover = st.valid(id) ? cov(c0, c1) : 0u;
+          continue;
+        }
+        const int dst = n + __popc(bal & ((1u << lane) - 1u));
+        if (cover != 0 && dst < 32) {
+          stage(dst, c0, c1, id, j);
+          s_cover[dst] = cover;
+          s_j[dst] = j;
+          cover = 0;
+        }
+        n += __popc(bal);
+        if (n >= 32) {
+          n = 32;
+          break;
+        }
+      }
+      __syncwarp();
+      if ((int)lane < n) mask = s_cover[lane];
+      return n;
+    }
+  }
+  __device__ __forceinline__ bool left() const { return PICK && __any_sync(0xffffffffu, cover != 0); }
+};
+
+// Slots of a picked batch (walk indices s_j, ascending, cnt of them) that come
+// before walk index `first`.
+__device__ __forceinline__ int slots_before(const uint32_t *s_j, int cnt, uint32_t first) {
+  int k = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1)
+    if (k + step <= cnt && s_j[k + step - 1] < first) k += step;
+  if (k < cnt && s_j[k] < first) ++k;
+  return k;
 }
 
 // Pixels of an 8 x 4 region whose centres lie in the box (x0, x1, y0, y1):
@@ -619,56 +299,35 @@ struct Region {
   __device__ __forceinline__ int64_t pixel() const { return img_off + (int64_t)py * W + px; }
 };
 
-template <int T, bool PIX, bool ROWS>
-__device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, int region, float4 *sA,
-                                              float4 *sB, float4 *sC) {
-  const int lane = threadIdx.x & 31;
-  const Region rg(a.s, gt, region, T);
+struct LaneFwdSmem {
+  float4 a[32], b[32];
+};
+
+template <bool ROWS>
+__device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, int region, LaneFwdSmem &sm) {
+  const Region rg(a.s, gt, region, a.s.tile);
   const uint2 range = a.ranges[gt];
-  const uint32_t *vals = a.vals;
   const float px = rg.px + 0.5f, py = rg.py + 0.5f;
   const float cx = rg.wx0 + 0.5f, cy = rg.wy0 + 0.5f;
-  PixRay ray;
-  if (PIX) pixel_ray(a.world_to_cam + 12 * rg.v, a.detector + 5 * rg.v, rg.H, rg.W, px, py, ray);
   float Tr = 1.f, C = 0.f;
   uint32_t last = 0;
   bool done = !rg.inside;
-  // software pipeline: the list ids two batches ahead and the records one
-  // batch ahead are in flight while a batch is walked
-  uint32_t id1 = 0xffffffffu, id2 = 0xffffffffu;
-  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-  if (range.x + lane < range.y) id1 = vals[range.x + lane];
-  if (range.x + 32 + lane < range.y) id2 = vals[range.x + 32 + lane];
-  if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-  for (uint32_t b0 = range.x; b0 < range.y; b0 += 32) {
+  EntryStream<false> st(a.vals + range.x, range.y - range.x, a.rec + 2 * rg.rec_base, rg.n_req);
+  Picker<false> pk;
+  for (uint32_t b0 = 0; st.more(); b0 += 32) {
     if (__all_sync(0xffffffffu, done)) break;
-    const uint32_t j = b0 + lane;
-    uint32_t cover = 0;
-    const uint32_t id = id1;
-    const float4 r0 = n0, r1 = n1;
-    id1 = id2;
-    id2 = 0xffffffffu;
-    if (b0 + 64 + lane < range.y) id2 = vals[b0 + 64 + lane];
-    if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-    if (j < range.y) {
-      if (id < rg.n_req) {
-        const int64_t r = rg.rec_base + id;
-        sA[lane] = r0;
-        sB[lane] = r1;
-        if (PIX) sC[lane] = a.rec2[r];
-        cover = region_cover<ROWS>(ellipse_box(r0, r1, a.P.q_max), cx, cy);
-      }
-    }
-    __syncwarp();
+    uint32_t cover;
+    pk.fill(st, nullptr, nullptr,
+            [&](float4 r0, float4 r1) { return region_cover<ROWS>(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+            [&](int k, float4 r0, float4 r1, uint32_t, uint32_t) { sm.a[k] = r0; sm.b[k] = r1; }, cover);
     uint32_t mine = transpose32(cover);  // staged entries covering this lane's pixel
     if (done) mine = 0;
-    const uint32_t pos1 = b0 - range.x + 1u;  // 1 + list position of staged entry 0
     const int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mine));
     for (int t = 0; t < trips; ++t) {
       if (mine == 0) continue;
       const int k = __ffs(mine) - 1;
       mine &= mine - 1;
-      const float4 A = sA[k], B = sB[k];
+      const float4 A = sm.a[k], B = sm.b[k];
       PairEval e;
       if (!eval_pair(A.x, A.y, A.z, A.w, B.x, B.y, px, py, a.P, e)) continue;
       const float Tn = __fmaf_rn(-Tr, e.sigma, Tr);  // T (1 - sigma)
@@ -677,10 +336,9 @@ __device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, i
         mine = 0;
         continue;
       }
-      const float col = PIX ? pixel_colour(ray, sC[k]) : B.z;
-      C = fmaf(col * e.sigma, Tr, C);
+      C = fmaf(B.z * e.sigma, Tr, C);
       Tr = Tn;
-      last = pos1 + (uint32_t)k;
+      last = b0 + (uint32_t)k + 1u;
     }
     __syncwarp();  // the slice is rewritten by the next batch
   }
@@ -694,212 +352,22 @@ __device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, i
 
 // Five resident blocks per SM (48 registers): these renders have few items per
 // warp slot, and a warp with more registers finishes an item sooner (one 512^2
-// view, 0.069 ms against 0.078 at eight blocks).
+// view, 0.069 ms against 0.078 at eight blocks). Picking the covering entries of
+// T = 16 lists first, as the pair kernels do, only lengthens a warp's serial
+// chain here (100k Gaussians, one 128^2 view: 91 -> 100 us).
 // ROWS: the backward of this render takes pixel pairs. The box only culls (q <=
 // q_max decides), but for ellipses so thin that rounding could pass a pixel
 // outside the box both passes must look at the same pixels.
-template <int T, bool PIX, bool ROWS>
-__global__ void __launch_bounds__(WARPS * 32, 5) raster_fwd_warp_kernel(RasterArgs a) {
-  constexpr int NW = T * T / 32;
-  __shared__ float4 s_a[WARPS][32], s_b[WARPS][32], s_c[WARPS][PIX ? 32 : 1];
-  const int w = threadIdx.x >> 5;
-  const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
+template <bool ROWS>
+__global__ void __launch_bounds__(WARPS * 32, 5) raster_fwd_lane_kernel(RasterArgs a) {
+  const uint32_t nw = (uint32_t)(a.s.tile * a.s.tile / 32);
+  __shared__ LaneFwdSmem sm[WARPS];
+  const uint64_t n_items = (uint64_t)a.s.total_tiles * nw;
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
-    const int64_t gt = a.order[item / NW];
-    fwd_lane_item<T, PIX, ROWS>(a, gt, (int)(item % NW), s_a[w], s_b[w], s_c[w]);
-    if (a.req_end && (threadIdx.x & 31) == 0)
-      atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
-  }
-}
-
-template <int T, bool PIX>
-__device__ __forceinline__ void bwd_warp_item(const RasterArgs &a, int64_t gt, int region, float4 *sA,
-                                              float4 *sB, float4 *sC, uint32_t *sId,
-                                              float (*sAcc)[n_acc<PIX>()]) {
-  const int lane = threadIdx.x & 31;
-  const TileGeom<T> tg(a.s, gt, region);
-  const uint2 range = a.ranges[tg.gtile];
-  const uint32_t *vals = a.vals;
-  const float px = tg.px + 0.5f, py = tg.py + 0.5f;
-  PixRay ray;
-  float gY[3] = {0.f, 0.f, 0.f};
-  if (PIX) pixel_ray(a.world_to_cam + 12 * tg.v, a.detector + 5 * tg.v, tg.H, tg.W, px, py, ray);
-  float Tr = 1.f, g = 0.f;
-  uint32_t last = 0;
-  if (tg.inside) {
-    const int64_t pix = tg.pixel();
-    Tr = a.t_final_in[pix];
-    last = a.n_last_in[pix];
-    g = a.dL_dimage[pix];
-  }
-  if (g == 0.f) last = 0;  // nothing to propagate from this pixel
-  if (last > range.y - range.x) last = range.y - range.x;  // never read past the list
-  uint32_t max_last = last;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) max_last = max(max_last, __shfl_xor_sync(0xffffffffu, max_last, o));
-  uint32_t qlast = last;
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) qlast = max(qlast, __shfl_xor_sync(0xffffffffu, qlast, o));
-  const uint32_t ql0 = __shfl_sync(0xffffffffu, qlast, 0), ql1 = __shfl_sync(0xffffffffu, qlast, 8);
-  const uint32_t ql2 = __shfl_sync(0xffffffffu, qlast, 16), ql3 = __shfl_sync(0xffffffffu, qlast, 24);
-  float S = 0.f;
-  for (int64_t hi = max_last; hi > 0; hi -= 32) {
-    const int64_t lo = hi > 32 ? hi - 32 : 0;
-    const int cnt = (int)(hi - lo);
-    // lane e stages list position hi - 1 - e (batches run back to front)
-    const bool ok = lane < cnt;
-    float4 box = empty_box();
-    if (ok) {
-      const uint32_t id = vals[range.x + (uint32_t)(hi - 1 - lane)];
-      if (id < tg.n_req) {  // else only after a capacity overflow
-        const int64_t r = tg.rec_base + id;
-        const float4 r0 = a.rec[2 * r], r1 = a.rec[2 * r + 1];
-        sA[lane] = r0;
-        sB[lane] = r1;
-        if (PIX) sC[lane] = a.rec2[r];
-        box = ellipse_box(r0, r1, a.P.q_max);
-      }
-      sId[lane] = id;
-    }
-#pragma unroll
-    for (int c = 0; c < n_acc<PIX>(); ++c) sAcc[lane][c] = 0.f;
-    __syncwarp();
-    const uint32_t pe = (uint32_t)(hi - 1 - lane);
-    const uint32_t m0 = __ballot_sync(0xffffffffu, ok && pe < ql0 && !tg.misses_q(box, 0));
-    const uint32_t m1 = __ballot_sync(0xffffffffu, ok && pe < ql1 && !tg.misses_q(box, 1));
-    const uint32_t m2 = __ballot_sync(0xffffffffu, ok && pe < ql2 && !tg.misses_q(box, 2));
-    const uint32_t m3 = __ballot_sync(0xffffffffu, ok && pe < ql3 && !tg.misses_q(box, 3));
-    const int qi = lane >> 3;
-    uint32_t mine = qi == 0 ? m0 : (qi == 1 ? m1 : (qi == 2 ? m2 : m3));
-    while (__any_sync(0xffffffffu, mine != 0)) {
-      const bool has = mine != 0;
-      const int k = has ? __ffs(mine) - 1 : 0;
-      if (has) mine &= mine - 1;
-      const uint32_t pos = (uint32_t)(hi - 1 - k);
-      float gv[PIX ? 10 : 8];
-#pragma unroll
-      for (int c = 0; c < (PIX ? 10 : 8); ++c) gv[c] = 0.f;
-      bool act = has && pos < last;
-      if (act) {
-        const float4 A = sA[k], B = sB[k];
-        PairEval e;
-        act = eval_pair(A.x, A.y, A.z, A.w, B.x, B.y, px, py, a.P, e);
-        if (act) {
-          // 1 / (1 - sigma) with sigma <= alpha_max < 1
-          const float inv_om = rcp_approx(__fsub_rn(1.f, e.sigma));
-          Tr = Tr * inv_om;  // transmittance before this Gaussian
-          float4 cz;
-          if (PIX) cz = sC[k];
-          const float c = PIX ? pixel_colour(ray, cz) : B.z;
-          const float dC_dsigma = fmaf(c, Tr, -S * inv_om);
-          S = fmaf(c * e.sigma, Tr, S);
-          const float gs = g * dC_dsigma;
-          float gq = 0.f;
-          if (!(e.aG > a.P.alpha_max)) {
-            gv[5] = gs * e.G;
-            gq = -0.5f * gs * B.y * e.G;
-          }
-          // sums of gq dx, gq dy, gq dx^2, gq dx dy and gq dy^2; the mean and
-          // conic gradients are formed from them once per entry (below)
-          const float gdx = gq * e.dx, gdy = gq * e.dy;
-          gv[0] = gdx;
-          gv[1] = gdy;
-          gv[2] = gdx * e.dx;
-          gv[3] = gdx * e.dy;
-          gv[4] = gdy * e.dy;
-          const float dcol = g * e.sigma * Tr;  // dL/dc
-          if (PIX) {
-            const float dz = dcol * c * (1.f - c);
-            gv[6] = dz;
-            gv[7] = dz * ray.Y[0];
-            gv[8] = dz * ray.Y[1];
-            gv[9] = dz * ray.Y[2];
-            gY[0] = fmaf(dz, cz.y, gY[0]);
-            gY[1] = fmaf(dz, cz.z, gY[1]);
-            gY[2] = fmaf(dz, cz.w, gY[2]);
-          } else {
-            gv[6] = dcol;
-          }
-        }
-      }
-      if (__any_sync(0xffffffffu, act)) {
-        if (PIX) {
-          const int comp = quarter_reduce10(gv);
-          if (has) {
-            if (gv[0] != 0.f) atomicAdd(&sAcc[k][comp], gv[0]);
-            if ((lane & 3) == 0 && gv[8] != 0.f) atomicAdd(&sAcc[k][(lane & 4) ? 9 : 8], gv[8]);
-          }
-        } else {
-          const int comp = quarter_reduce8(gv);
-          if (has && gv[0] != 0.f) atomicAdd(&sAcc[k][comp], gv[0]);
-        }
-      }
-    }
-    __syncwarp();
-    if (ok) {  // lane e sends entry e's sums
-      const float *acc = sAcc[lane];
-      bool nz = (acc[0] != 0.f) | (acc[1] != 0.f) | (acc[2] != 0.f) | (acc[3] != 0.f) |
-                (acc[4] != 0.f) | (acc[5] != 0.f) | (acc[6] != 0.f);
-      if (PIX) nz |= (acc[7] != 0.f) | (acc[8] != 0.f) | (acc[9] != 0.f);
-      if (nz) {
-        const int64_t r = tg.rec_base + sId[lane];
-        float4 *dst = a.grad2d + 2 * r;
-        // dq/du = 2 (a dx + b dy), dq/dv = 2 (b dx + c dy), dq/db = 2 dx dy
-        // the record holds CONIC_SCALE (a, 2b, c)
-        const float ca = sA[lane].z * INV_CONIC_SCALE, cb = (0.5f * INV_CONIC_SCALE) * sA[lane].w,
-                    cc = sB[lane].x * INV_CONIC_SCALE;
-        const float du = 2.f * fmaf(ca, acc[0], cb * acc[1]);
-        const float dv = 2.f * fmaf(cb, acc[0], cc * acc[1]);
-        atomicAdd(dst, make_float4(du, dv, acc[2], 2.f * acc[3]));
-        atomicAdd(dst + 1, make_float4(acc[4], acc[5], acc[6], 0.f));
-        if (PIX) atomicAdd(a.grad_h + r, make_float4(acc[7], acc[8], acc[9], 0.f));
-      }
-    }
-    __syncwarp();
-  }
-  if (PIX && a.pose_grad) {
-    // Y_1(d / |d|), d = W^T rc: dL/dW[r][c] = rc[r] dL/dd[c], summed over the warp
-    const bool mine = tg.inside && ((gY[0] != 0.f) | (gY[1] != 0.f) | (gY[2] != 0.f));
-    if (__any_sync(0xffffffffu, mine)) {
-      float w9[9];
-      const float ddh[3] = {-SH_C1 * gY[2], -SH_C1 * gY[0], SH_C1 * gY[1]};
-      const float dot = ddh[0] * ray.dh[0] + ddh[1] * ray.dh[1] + ddh[2] * ray.dh[2];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float dd = mine ? (ddh[c] - ray.dh[c] * dot) * ray.inv : 0.f;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) w9[3 * r + c] = ray.rc[r] * dd;
-      }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) w9[i] += __shfl_xor_sync(0xffffffffu, w9[i], o);
-      }
-      if (lane < 9) {
-        float x = w9[0];
-#pragma unroll
-        for (int i = 1; i < 9; ++i) if (lane == i) x = w9[i];
-        if (x != 0.f) atomicAdd(a.pose_grad + 12 * (int64_t)tg.v + 4 * (lane / 3) + lane % 3, x);
-      }
-    }
-  }
-}
-
-template <int T, bool PIX>
-__global__ void __launch_bounds__(WARPS * 32, 4) raster_bwd_warp_kernel(RasterArgs a) {
-  constexpr int NW = T * T / 32;
-  __shared__ float4 s_a[WARPS][32], s_b[WARPS][32], s_c[WARPS][PIX ? 32 : 1];
-  __shared__ uint32_t s_id[WARPS][32];
-  __shared__ float s_acc[WARPS][32][n_acc<PIX>()];
-  const int w = threadIdx.x >> 5;
-  const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
-  for (;;) {
-    const uint32_t item = warp_next_item(a.counter);
-    if (item >= n_items) break;
-    const int64_t gt = a.order[item / NW];
-    bwd_warp_item<T, PIX>(a, gt, (int)(item % NW), s_a[w], s_b[w], s_c[w], s_id[w], s_acc[w]);
+    const int64_t gt = a.order[item / nw];
+    fwd_lane_item<ROWS>(a, gt, (int)(item % nw), sm[threadIdx.x >> 5]);
     if (a.req_end && (threadIdx.x & 31) == 0)
       atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
   }
@@ -923,16 +391,16 @@ constexpr int LANE_WARPS = 8;  // warps per block of the per-lane backward (3 bl
 
 struct LaneBwdSmem {
   float4 a[33], b[33];  // entry 32: a sentinel that no pixel adds
-  uint32_t id[32];
+  uint32_t id[32], cover[32], j[32];
   float2 ab[32 * AB_STRIDE];  // [pixel][entry ^ pixel]: (A, Bc)
 };
 
 template <int T>
 __device__ __forceinline__ void bwd_lane_item(const RasterArgs &a, int64_t gt, int region, LaneBwdSmem &sm) {
+  constexpr bool PICK = T > 8;
   const int lane = threadIdx.x & 31;
   const Region rg(a.s, gt, region, T);
   const uint2 range = a.ranges[gt];
-  const uint32_t *vals = a.vals;
   const float px = rg.px + 0.5f, py = rg.py + 0.5f;
   const float cx = rg.wx0 + 0.5f, cy = rg.wy0 + 0.5f;
   float Tr = 1.f, g = 0.f;
@@ -952,40 +420,27 @@ __device__ __forceinline__ void bwd_lane_item(const RasterArgs &a, int64_t gt, i
   // the walk carries g T and g S (Tr, S), so that g drops out of the per-pair
   // products: g dC/dsigma = c gT - gS / (1 - sigma), g dC/dc = sigma gT
   Tr *= g;
-  uint32_t max_last = last;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) max_last = max(max_last, __shfl_xor_sync(0xffffffffu, max_last, o));
+  const uint32_t max_last = __reduce_max_sync(0xffffffffu, last);
+  const uint32_t first = max_last - last;  // this pixel's first walk index
   float S = 0.f;
-  // software pipeline: the list ids two batches ahead and the records one
-  // batch ahead are in flight while a batch is walked
-  uint32_t id1 = 0xffffffffu, id2 = 0xffffffffu;
-  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-  if ((int64_t)lane < (int64_t)max_last) id1 = vals[range.x + (uint32_t)(max_last - 1 - lane)];
-  if ((int64_t)max_last > 32 && (int64_t)lane < (int64_t)max_last - 32)
-    id2 = vals[range.x + (uint32_t)(max_last - 33 - lane)];
-  if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-  for (int64_t hi = max_last; hi > 0; hi -= 32) {
-    const int cnt = (int)(hi > 32 ? 32 : hi);
-    uint32_t cover = 0;
-    const uint32_t id = id1;
-    const float4 r0 = n0, r1 = n1;
-    id1 = id2;
-    id2 = 0xffffffffu;
-    if (hi - 64 > 0 && (int64_t)lane < hi - 64) id2 = vals[range.x + (uint32_t)(hi - 65 - lane)];
-    if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-    if (lane < cnt) {
-      if (id < rg.n_req) {
-        sm.a[lane] = r0;
-        sm.b[lane] = r1;
-        cover = region_cover<false>(ellipse_box(r0, r1, a.P.q_max), cx, cy);
-      }
-      sm.id[lane] = id;
-    }
-    __syncwarp();
+  EntryStream<true> st(a.vals + range.x, max_last, a.rec + 2 * rg.rec_base, rg.n_req);
+  Picker<PICK> pk;
+  for (uint32_t b0 = 0; st.more() || pk.left(); b0 += 32) {
+    uint32_t cover;
+    const int cnt = pk.fill(
+        st, sm.cover, sm.j,
+        [&](float4 r0, float4 r1) { return region_cover<false>(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+        [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) { sm.a[k] = r0; sm.b[k] = r1; sm.id[k] = id; },
+        cover);
     uint32_t mine = transpose32(cover);
-    // staged entries e >= hi - last lie before this pixel's last added Gaussian
-    const int64_t skip = hi - (int64_t)last;
-    mine &= skip <= 0 ? 0xffffffffu : (skip >= 32 ? 0u : (0xffffffffu << skip));
+    // the first staged entries may lie past this pixel's last added Gaussian
+    int skip = 0;
+    if (PICK) {
+      if (cnt > 0 && first > sm.j[0]) skip = slots_before(sm.j, cnt, first);
+    } else {
+      skip = first > b0 ? (int)min(first - b0, 32u) : 0;
+    }
+    mine &= skip >= 32 ? 0u : (0xffffffffu << skip);
     uint32_t used = 0;
     const int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mine));
     // one entry per trip, written without branches (a lane past its last
@@ -1155,11 +610,12 @@ __device__ __forceinline__ uint64_t pair_q(const PairSlot &s, float px, uint64_t
 
 // The 8 x 8 pixel region of a work item.
 struct PairRegion {
-  int H, W, wx0, wy0, px, py;
+  int v, H, W, wx0, wy0, px, py;
   bool in0, in1;
   int64_t rec_base, img_off, n_req;
   __device__ __forceinline__ PairRegion(const RenderShape &s, int64_t gt, int region, int T) {
-    const ViewTab vt = s.view[find_view(s.view, s.V, gt)];
+    v = find_view(s.view, s.V, gt);
+    const ViewTab vt = s.view[v];
     H = vt.H;
     W = vt.W;
     rec_base = vt.rec_off;
@@ -1196,58 +652,60 @@ __device__ __forceinline__ uint32_t pair_cover(float4 b, float cx, float cy) {
 // the number of trips (7.7 trips per batch instead of 10.4 at the benchmark).
 // T is negated once a pixel has stopped (every later T (1 - sigma) is then
 // below t_min), and from the start outside the image.
-template <int T>
-__device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, int region,
-                                              PairSlot *slots) {
-  const int lane = threadIdx.x & 31;
+template <bool PIX>
+struct PairFwdSmem {
+  PairSlot slot[64];
+  uint32_t j[64], cover[32];
+  float4 z[PIX ? 64 : 1];  // (a, h_0, h_1, h_2)
+};
+
+template <int T, bool PIX>
+__device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, int region, PairFwdSmem<PIX> &sm) {
+  constexpr bool PICK = T > 8;
   const PairRegion rg(a.s, gt, region, T);
   const uint2 range = a.ranges[gt];
-  const uint32_t *vals = a.vals;
   const float px = rg.px + 0.5f;
   const uint64_t npy = pack2(-(rg.py + 0.5f), -(rg.py + 1.5f));
   const float cx = rg.wx0 + 0.5f, cy = rg.wy0 + 0.5f;
   const float namax = -a.P.alpha_max, namin = -a.P.alpha_min;
+  PixRay ray0, ray1;
+  if (PIX) {
+    pixel_ray(a.world_to_cam + 12 * rg.v, a.detector + 5 * rg.v, rg.H, rg.W, px, rg.py + 0.5f, ray0);
+    pixel_ray(a.world_to_cam + 12 * rg.v, a.detector + 5 * rg.v, rg.H, rg.W, px, rg.py + 1.5f, ray1);
+  }
   float T0 = rg.in0 ? 1.f : -1.f, T1 = rg.in1 ? 1.f : -1.f, C0 = 0.f, C1 = 0.f;
   uint32_t last0 = 0, last1 = 0;
   bool done = !rg.in0;  // in1 implies in0
-  // software pipeline: the list ids two batches ahead and the records one
-  // batch ahead are in flight while a batch is walked
-  uint32_t id1 = 0xffffffffu, id2 = 0xffffffffu;
-  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-  if (range.x + lane < range.y) id1 = vals[range.x + lane];
-  if (range.x + 32 + lane < range.y) id2 = vals[range.x + 32 + lane];
-  if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
+  EntryStream<false> st(a.vals + range.x, range.y - range.x, a.rec + 2 * rg.rec_base, rg.n_req);
+  Picker<PICK> pk;
   uint32_t m = 0, nx = 0;         // entries left of the older and of the newer batch
   uint32_t slot = 0, pos = 1;     // first slot and first 1-based list position of m's batch
-  for (uint32_t b0 = range.x;; b0 += 32) {
+  for (uint32_t b0 = 0;; b0 += 32) {
     if (__all_sync(0xffffffffu, done)) break;
     // everything before the batch at b0 - 32 is walked
-    const uint32_t half = (b0 - range.x) & 32u;
+    const uint32_t half = b0 & 32u;
     if (m == 0) {
       m = nx;
       slot = half ^ 32u;
-      pos = b0 - range.x - 31u;
+      pos = b0 - 31u;
     }
     nx = 0;
     const int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(m));
-    if (b0 < range.y) {
-      const uint32_t id = id1;
-      const float4 r0 = n0, r1 = n1;
-      id1 = id2;
-      id2 = 0xffffffffu;
-      if (b0 + 64 + lane < range.y) id2 = vals[b0 + 64 + lane];
-      if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-      uint32_t cover = 0;
-      if (b0 + lane < range.y && id < rg.n_req) {
-        stage_pair(slots[half + lane], r0, r1);
-        cover = pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy);
-      }
-      __syncwarp();
+    if (st.more() || pk.left()) {
+      uint32_t cover;
+      pk.fill(st, sm.cover, sm.j + half,
+              [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+              [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) {
+                stage_pair(sm.slot[half + k], r0, r1);
+                if (PIX) sm.z[half + k] = a.rec2[rg.rec_base + id];
+              },
+              cover);
       nx = transpose32(cover);
       if (done) nx = 0;
     } else if (trips == 0) {
       break;
     }
+    uint32_t add0 = 0, add1 = 0;  // PICK: 1 + slot of the last entry added
     for (int t = 0; t < trips; ++t) {
       if (m == 0) {
         m = nx;
@@ -1258,7 +716,7 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
       if (m == 0) continue;
       const uint32_t k = (uint32_t)__ffs(m) - 1u;
       m &= m - 1;
-      const PairSlot &s = slots[slot + k];
+      const PairSlot &s = sm.slot[slot + k];
       const uint64_t q = pair_q(s, px, npy);
       const float2 qf = unpack2(q);
       const uint64_t naG = mul2(s.c.x, pack2(exp2_approx(qf.x), exp2_approx(qf.y)));
@@ -1270,17 +728,22 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
       const float2 Tn = unpack2(fma2(Tr, ns, Tr));  // T (1 - sigma)
       const bool st0 = ok0 && Tn.x < a.P.t_min, st1 = ok1 && Tn.y < a.P.t_min;
       // C - (colour (-sigma)) T
-      const float2 w = unpack2(mul2(s.c.y, ns));
-      const uint32_t p = pos + k;
+      uint64_t col = s.c.y;
+      if (PIX && (ok0 || ok1)) {
+        const float4 z = sm.z[slot + k];
+        col = pack2(pixel_colour(ray0, z), pixel_colour(ray1, z));
+      }
+      const float2 w = unpack2(mul2(col, ns));
+      const uint32_t p = PICK ? slot + k + 1u : pos + k;
       if (ok0 && !st0) {
         C0 = fmaf(-w.x, T0, C0);
         T0 = Tn.x;
-        last0 = p;
+        (PICK ? add0 : last0) = p;
       }
       if (ok1 && !st1) {
         C1 = fmaf(-w.y, T1, C1);
         T1 = Tn.y;
-        last1 = p;
+        (PICK ? add1 : last1) = p;
       }
       if (st0 || st1) {
         if (st0) T0 = -fabsf(T0);
@@ -1290,6 +753,10 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
           m = nx = 0;
         }
       }
+    }
+    if (PICK) {
+      if (add0) last0 = sm.j[add0 - 1u] + 1u;
+      if (add1) last1 = sm.j[add1 - 1u] + 1u;
     }
     __syncwarp();  // the older half is rewritten by the next batch
   }
@@ -1306,17 +773,23 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
   }
 }
 
+// 32 warps per SM at 64 registers (40 at 48: 1.09 -> 1.15 ms at 64 poses, 24 at
+// 80: 1.20); blocks of four warps spread a small render over more SMs than
+// blocks of eight. The picking and the per-pixel instances keep more state and
+// take 80 registers (100k Gaussians, 4 x 256^2 at T = 16: 71 us at 72, 66 at 80;
+// per-pixel rays, 200k, 8 x 256^2 at T = 8: 154, and 165 at 96).
 constexpr int PAIR_FWD_WARPS = 4, PAIR_FWD_BLOCKS = 8;
-template <int T>
-__global__ void __launch_bounds__(PAIR_FWD_WARPS * 32, PAIR_FWD_BLOCKS) raster_fwd_pair_kernel(RasterArgs a) {
+template <int T, bool PIX>
+__global__ void __launch_bounds__(PAIR_FWD_WARPS * 32, PIX || T > 8 ? 6 : PAIR_FWD_BLOCKS)
+raster_fwd_pair_kernel(RasterArgs a) {
   constexpr int NW = T * T / 64;
-  __shared__ PairSlot s_slot[PAIR_FWD_WARPS][64];
+  __shared__ PairFwdSmem<PIX> sm[PAIR_FWD_WARPS];
   const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
     const int64_t gt = a.order[item / NW];
-    fwd_pair_item<T>(a, gt, (int)(item % NW), s_slot[threadIdx.x >> 5]);
+    fwd_pair_item<T, PIX>(a, gt, (int)(item % NW), sm[threadIdx.x >> 5]);
     if (a.req_end && (threadIdx.x & 31) == 0)
       atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
   }
@@ -1327,22 +800,32 @@ __global__ void __launch_bounds__(PAIR_FWD_WARPS * 32, PAIR_FWD_BLOCKS) raster_f
 // of the lower pixel) and the sum of -dL/dc over the pair; with x the pair's
 // column and y its upper row, phase 2 gets every moment of the pixel offsets
 // from sums over pairs: sum A = sum S, A x = S x, A y = S y + D, A x^2 = S x^2,
-// A x y = (S y + D) x, A y^2 = S y^2 + D (2 y + 1).
+// A x y = (S y + D) x, A y^2 = S y^2 + D (2 y + 1). With per-pixel rays the
+// table holds dL/dz of both pixels instead, for the sums of dL/dz and dL/dz Y.
+template <bool PIX>
 struct PairBwdSmem {
   PairSlot slot[33];  // entry 32: a sentinel that no pixel adds
-  uint32_t id[32];
+  float4 z[PIX ? 33 : 1];   // (a, h_0, h_1, h_2)
+  float4 y[PIX ? 64 : 1];   // Y_1 of the rays of the upper and of the lower pixels
+  uint32_t id[32], cover[32], j[32];
   float2 sd[32 * 32];  // [pair][entry ^ pair]: (S, D)
-  float nb[32 * 32];   // the same: -sum of dL/dc
+  float2 dz[PIX ? 32 * 32 : 1];  // the same: dL/dz of the two pixels
+  float nb[PIX ? 1 : 32 * 32];   // the same: -sum of dL/dc
 };
-constexpr int PAIR_BWD_WARPS = 4, PAIR_BWD_BLOCKS = 4;  // 56 KB a block: sixteen warps per SM
-constexpr size_t PAIR_BWD_SMEM = PAIR_BWD_WARPS * sizeof(PairBwdSmem);
+// Blocks of four warps and 57 KB, sixteen warps per SM; with per-pixel rays
+// blocks of two and 40 KB, ten warps.
+template <bool PIX>
+struct PairBwd {
+  static constexpr int WARPS = PIX ? 2 : 4, BLOCKS = PIX ? 5 : 4;
+  static constexpr size_t SMEM = WARPS * sizeof(PairBwdSmem<PIX>);
+};
 
-template <int T>
-__device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, int region, PairBwdSmem &sm) {
+template <int T, bool PIX>
+__device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, int region, PairBwdSmem<PIX> &sm) {
+  constexpr bool PICK = T > 8;
   const int lane = threadIdx.x & 31;
   const PairRegion rg(a.s, gt, region, T);
   const uint2 range = a.ranges[gt];
-  const uint32_t *vals = a.vals;
   const float px = rg.px + 0.5f;
   const uint64_t npy = pack2(-(rg.py + 0.5f), -(rg.py + 1.5f));
   const float cx = rg.wx0 + 0.5f, cy = rg.wy0 + 0.5f;
@@ -1361,41 +844,48 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
       last1 = h == 0.f ? 0u : min(a.n_last_in[pix + rg.W], len);
     }
   }
+  PixRay ray0, ray1;
+  float gY0[3] = {0.f, 0.f, 0.f}, gY1[3] = {0.f, 0.f, 0.f};  // dL/dY_1 of the pixels' rays
+  if (PIX) {
+    pixel_ray(a.world_to_cam + 12 * rg.v, a.detector + 5 * rg.v, rg.H, rg.W, px, rg.py + 0.5f, ray0);
+    pixel_ray(a.world_to_cam + 12 * rg.v, a.detector + 5 * rg.v, rg.H, rg.W, px, rg.py + 1.5f, ray1);
+    sm.y[lane] = make_float4(ray0.Y[0], ray0.Y[1], ray0.Y[2], 0.f);
+    sm.y[32 + lane] = make_float4(ray1.Y[0], ray1.Y[1], ray1.Y[2], 0.f);
+  }
   if (lane == 0) {  // q' = -inf at every pixel
     sm.slot[32].g = make_ulonglong2(pack2(3.0e38f, -1.f), pack2(3.0e38f, 3.0e38f));
     sm.slot[32].k = make_ulonglong2(pack2(0.f, 0.f), pack2(-1.f, -1.f));
     sm.slot[32].c = make_ulonglong2(0ull, 0ull);
+    if (PIX) sm.z[32] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   const uint32_t max_last = __reduce_max_sync(0xffffffffu, max(last0, last1));
+  const uint32_t first0 = max_last - last0, first1 = max_last - last1;  // the pixels' first walk indices
   uint64_t nS = 0;  // -g S of both pixels
   uint64_t Tr = pack2(T0, T1);
   const uint64_t one = pack2(1.f, 1.f);
-  uint32_t id1 = 0xffffffffu, id2 = 0xffffffffu;
-  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-  if ((uint32_t)lane < max_last) id1 = vals[range.x + (max_last - 1 - lane)];
-  if ((uint32_t)lane + 32u < max_last) id2 = vals[range.x + (max_last - 33 - lane)];
-  if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-  for (int64_t hi = max_last; hi > 0; hi -= 32) {
-    const int cnt = (int)(hi > 32 ? 32 : hi);
-    uint32_t cover = 0;
-    const uint32_t id = id1;
-    const float4 r0 = n0, r1 = n1;
-    id1 = id2;
-    id2 = 0xffffffffu;
-    if ((int64_t)lane < hi - 64) id2 = vals[range.x + (uint32_t)(hi - 65 - lane)];
-    if (id1 < rg.n_req) { const int64_t r = rg.rec_base + id1; n0 = a.rec[2 * r]; n1 = a.rec[2 * r + 1]; }
-    if (lane < cnt) {
-      if (id < rg.n_req) {
-        stage_pair(sm.slot[lane], r0, r1);
-        cover = pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy);
-      }
-      sm.id[lane] = id;
-    }
-    __syncwarp();
+  EntryStream<true> st(a.vals + range.x, max_last, a.rec + 2 * rg.rec_base, rg.n_req);
+  Picker<PICK> pk;
+  for (uint32_t b0 = 0; st.more() || pk.left(); b0 += 32) {
+    uint32_t cover;
+    const int cnt = pk.fill(
+        st, sm.cover, sm.j,
+        [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+        [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) {
+          stage_pair(sm.slot[k], r0, r1);
+          sm.id[k] = id;
+          if (PIX) sm.z[k] = a.rec2[rg.rec_base + id];
+        },
+        cover);
     uint32_t mine = transpose32(cover);
-    // staged entries e >= hi - last lie before the pixel's last added Gaussian
-    const int64_t d0 = hi - (int64_t)last0, d1 = hi - (int64_t)last1;
-    const int skip0 = (int)(d0 < 0 ? 0 : (d0 > 32 ? 32 : d0)), skip1 = (int)(d1 < 0 ? 0 : (d1 > 32 ? 32 : d1));
+    // the first staged entries may lie past a pixel's last added Gaussian
+    int skip0, skip1;
+    if (PICK) {
+      skip0 = cnt > 0 && first0 > sm.j[0] ? slots_before(sm.j, cnt, first0) : 0;
+      skip1 = cnt > 0 && first1 > sm.j[0] ? slots_before(sm.j, cnt, first1) : 0;
+    } else {
+      skip0 = first0 > b0 ? (int)min(first0 - b0, 32u) : 0;
+      skip1 = first1 > b0 ? (int)min(first1 - b0, 32u) : 0;
+    }
     const int skip = min(skip0, skip1);
     mine &= skip >= 32 ? 0u : (0xffffffffu << skip);
     uint32_t used = 0;
@@ -1423,15 +913,39 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
       const float2 om = unpack2(add2(one, ns));
       const uint64_t inv = pack2(rcp_approx(om.x), rcp_approx(om.y));
       const uint64_t Tn = mul2(Tr, inv);
-      const uint64_t gdC = fma2(s.c.y, Tn, mul2(nS, inv));  // g dC/dsigma
-      const uint64_t nsT = mul2(ns, Tn);                    // -g dC/dc
-      const uint64_t nSn = fma2(s.c.y, nsT, nS);
+      uint64_t col = s.c.y;
+      float4 z;
+      float2 cf;
+      if (PIX) {
+        z = sm.z[k];
+        cf = make_float2(pixel_colour(ray0, z), pixel_colour(ray1, z));
+        col = pack2(cf.x, cf.y);
+      }
+      const uint64_t gdC = fma2(col, Tn, mul2(nS, inv));  // g dC/dsigma
+      const uint64_t nsT = mul2(ns, Tn);                  // -g dC/dc
+      const uint64_t nSn = fma2(col, nsT, nS);
       const float2 gA = unpack2(mul2(gdC, G)), nb = unpack2(nsT);
       const float A0 = ok0 && !(ng.x < namax) ? gA.x : 0.f, A1 = ok1 && !(ng.y < namax) ? gA.y : 0.f;
-      const float b0 = ok0 ? nb.x : 0.f, b1 = ok1 ? nb.y : 0.f;
+      const float b0_ = ok0 ? nb.x : 0.f, b1_ = ok1 ? nb.y : 0.f;
       if (ok0 || ok1) {
-        sm.sd[lane * 32 + (k ^ lane)] = make_float2(A0 + A1, A1);
-        sm.nb[lane * 32 + (k ^ lane)] = b0 + b1;
+        const int at = lane * 32 + (k ^ lane);
+        sm.sd[at] = make_float2(A0 + A1, A1);
+        if (PIX) {
+          const float z0 = -b0_ * cf.x * (1.f - cf.x), z1 = -b1_ * cf.y * (1.f - cf.y);
+          sm.dz[at] = make_float2(ok0 ? z0 : 0.f, ok1 ? z1 : 0.f);
+          if (ok0) {
+            gY0[0] = fmaf(z0, z.y, gY0[0]);
+            gY0[1] = fmaf(z0, z.z, gY0[1]);
+            gY0[2] = fmaf(z0, z.w, gY0[2]);
+          }
+          if (ok1) {
+            gY1[0] = fmaf(z1, z.y, gY1[0]);
+            gY1[1] = fmaf(z1, z.z, gY1[1]);
+            gY1[2] = fmaf(z1, z.w, gY1[2]);
+          }
+        } else {
+          sm.nb[at] = b0_ + b1_;
+        }
         used |= bit;
       }
       const float2 To = unpack2(Tr), Tv = unpack2(Tn), So = unpack2(nS), Sv = unpack2(nSn);
@@ -1442,18 +956,30 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
     uint32_t pm = transpose32(used);  // lane e: the pairs that added entry e
     if (pm) {
       uint64_t sd = 0, sdx = 0, sdy = 0;  // sums of (S, D), (S, D) x, (S, D) y
-      float sxx = 0.f, sxy = 0.f, syy = 0.f, sb = 0.f;
+      float sxx = 0.f, sxy = 0.f, syy = 0.f, sb = 0.f, sh[3] = {0.f, 0.f, 0.f};
       do {  // two pairs per trip: half the loop overhead, two loads in flight
         const int p = __ffs(pm) - 1;
         pm &= pm - 1;
         const bool two = pm != 0;
         const int q = two ? __ffs(pm) - 1 : p;
         pm &= pm - 1;
-        const float2 u = sm.sd[p * 32 + (lane ^ p)];
-        float2 v = sm.sd[q * 32 + (lane ^ q)];
-        const float ub = sm.nb[p * 32 + (lane ^ p)];
-        float vb = sm.nb[q * 32 + (lane ^ q)];
-        if (!two) { v = make_float2(0.f, 0.f); vb = 0.f; }
+        const int ip = p * 32 + (lane ^ p), iq = q * 32 + (lane ^ q);
+        const float2 u = sm.sd[ip];
+        float2 v = sm.sd[iq];
+        if (!two) v = make_float2(0.f, 0.f);
+        if (PIX) {
+          const float2 zu = sm.dz[ip];
+          float2 zv = sm.dz[iq];
+          if (!two) zv = make_float2(0.f, 0.f);
+          sb += (zu.x + zu.y) + (zv.x + zv.y);
+          const float4 yu0 = sm.y[p], yu1 = sm.y[32 + p], yv0 = sm.y[q], yv1 = sm.y[32 + q];
+          sh[0] = fmaf(zu.x, yu0.x, fmaf(zu.y, yu1.x, fmaf(zv.x, yv0.x, fmaf(zv.y, yv1.x, sh[0]))));
+          sh[1] = fmaf(zu.x, yu0.y, fmaf(zu.y, yu1.y, fmaf(zv.x, yv0.y, fmaf(zv.y, yv1.y, sh[1]))));
+          sh[2] = fmaf(zu.x, yu0.z, fmaf(zu.y, yu1.z, fmaf(zv.x, yv0.z, fmaf(zv.y, yv1.z, sh[2]))));
+        } else {
+          const float ub = sm.nb[ip], vb = sm.nb[iq];
+          sb -= ub + (two ? vb : 0.f);
+        }
         const float x = (float)(p & 7), y = (float)((p >> 2) & 6);
         const float x2 = (float)(q & 7), y2 = (float)((q >> 2) & 6);
         const uint64_t up = pack2(u.x, u.y), vp = pack2(v.x, v.y);
@@ -1464,7 +990,6 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
         sxx = fmaf(ax, x, fmaf(ax2, x2, sxx));
         sxy = fmaf(ax, y, fmaf(ax2, y2, sxy));
         syy = fmaf(u.x * y, y, fmaf(v.x * y2, y2, syy));
-        sb += ub + vb;
       } while (pm);
       const float2 fd = unpack2(sd), fx = unpack2(sdx), fy = unpack2(sdy);
       const float s0 = fd.x, s1 = fx.x, s2 = fy.x + fd.y, s4 = sxy + fx.y,
@@ -1485,25 +1010,60 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
       const float gx = hk * sdx1, gy = hk * sdy1;
       const float du = fmaf(2.f * ca, gx, cb2 * gy);
       const float dv = fmaf(cb2, gx, 2.f * cc * gy);
-      float4 *dst = a.grad2d + 2 * (rg.rec_base + sm.id[lane]);
-      atomicAdd(dst, make_float4(du, dv, hq * gxx, 2.f * hq * gxy));
-      atomicAdd(dst + 1, make_float4(hq * gyy, s0, -sb, 0.f));
+      const int64_t r = rg.rec_base + sm.id[lane];
+      atomicAdd(a.grad2d + 2 * r, make_float4(du, dv, hq * gxx, 2.f * hq * gxy));
+      atomicAdd(a.grad2d + 2 * r + 1, make_float4(hq * gyy, s0, sb, 0.f));
+      if (PIX) atomicAdd(a.grad_h + r, make_float4(sh[0], sh[1], sh[2], 0.f));
     }
     __syncwarp();  // the slice is rewritten by the next batch
   }
+  if (PIX && a.pose_grad) {
+    // Y_1(d / |d|), d = W^T rc: dL/dW[r][c] = rc[r] dL/dd[c], summed over the warp
+    float w9[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) w9[i] = 0.f;
+    auto add = [&](const PixRay &ray, const float gY[3]) {
+      if (gY[0] == 0.f && gY[1] == 0.f && gY[2] == 0.f) return;
+      const float ddh[3] = {-SH_C1 * gY[2], -SH_C1 * gY[0], SH_C1 * gY[1]};
+      const float dot = ddh[0] * ray.dh[0] + ddh[1] * ray.dh[1] + ddh[2] * ray.dh[2];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float dd = (ddh[c] - ray.dh[c] * dot) * ray.inv;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) w9[3 * r + c] = fmaf(ray.rc[r], dd, w9[3 * r + c]);
+      }
+    };
+    add(ray0, gY0);
+    add(ray1, gY1);
+    const bool mine = (w9[0] != 0.f) | (w9[1] != 0.f) | (w9[2] != 0.f) | (w9[3] != 0.f) | (w9[4] != 0.f) |
+                      (w9[5] != 0.f) | (w9[6] != 0.f) | (w9[7] != 0.f) | (w9[8] != 0.f);
+    if (__any_sync(0xffffffffu, mine)) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w9[i] += __shfl_xor_sync(0xffffffffu, w9[i], o);
+      }
+      if (lane < 9) {
+        float x = w9[0];
+#pragma unroll
+        for (int i = 1; i < 9; ++i) if (lane == i) x = w9[i];
+        if (x != 0.f) atomicAdd(a.pose_grad + 12 * (int64_t)rg.v + 4 * (lane / 3) + lane % 3, x);
+      }
+    }
+  }
 }
 
-template <int T>
-__global__ void __launch_bounds__(PAIR_BWD_WARPS * 32, PAIR_BWD_BLOCKS) raster_bwd_pair_kernel(RasterArgs a) {
+template <int T, bool PIX>
+__global__ void __launch_bounds__(PairBwd<PIX>::WARPS * 32, PairBwd<PIX>::BLOCKS) raster_bwd_pair_kernel(RasterArgs a) {
   constexpr int NW = T * T / 64;
   extern __shared__ __align__(16) unsigned char lane_smem[];
-  PairBwdSmem &sm = reinterpret_cast<PairBwdSmem *>(lane_smem)[threadIdx.x >> 5];
+  PairBwdSmem<PIX> &sm = reinterpret_cast<PairBwdSmem<PIX> *>(lane_smem)[threadIdx.x >> 5];
   const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
     const int64_t gt = a.order[item / NW];
-    bwd_pair_item<T>(a, gt, (int)(item % NW), sm);
+    bwd_pair_item<T, PIX>(a, gt, (int)(item % NW), sm);
     if (a.req_end && (threadIdx.x & 31) == 0)
       atomicMax(a.req_end + a.s.view[find_view(a.s.view, a.s.V, gt)].req, global_ns());
   }
@@ -1554,7 +1114,7 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(int64_t n_tiles, const
 
 // Resident blocks per SM of a kernel, cached per (device, kernel); the query
 // is not a stream operation, so it is also legal while a stream is captured.
-int blocks_per_sm(void (*k)(RasterArgs), int threads, size_t dyn_smem = 0) {
+int blocks_per_sm(void (*k)(RasterArgs), int threads, size_t dyn_smem) {
   static std::mutex mu;
   static std::map<std::pair<int, const void *>, int> cache;
   int dev = 0;
@@ -1567,26 +1127,6 @@ int blocks_per_sm(void (*k)(RasterArgs), int threads, size_t dyn_smem = 0) {
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, dyn_smem) != cudaSuccess || n < 1) n = 1;
   cache[key] = n;
   return n;
-}
-
-template <int T, int BATCH, bool PIX>
-void launch_fwd_t(const RasterArgs &a, cudaStream_t st) {
-  if (a.s.total_tiles <= 0) return;
-  auto k = raster_fwd_kernel<T, BATCH, PIX>;
-  int64_t grid = (int64_t)blocks_per_sm(k, T * T) * device_sms();
-  if (grid > a.s.total_tiles) grid = a.s.total_tiles;
-  LaunchScope ls(KID_RASTER_FWD, st);
-  k<<<(unsigned)grid, T * T, 0, st>>>(a);
-}
-
-template <int T, int BATCH, bool PIX>
-void launch_bwd_t(const RasterArgs &a, cudaStream_t st) {
-  if (a.s.total_tiles <= 0) return;
-  auto k = raster_bwd_kernel<T, BATCH, PIX>;
-  int64_t grid = (int64_t)blocks_per_sm(k, T * T) * device_sms();
-  if (grid > a.s.total_tiles) grid = a.s.total_tiles;
-  LaunchScope ls(KID_RASTER_BWD, st);
-  k<<<(unsigned)grid, T * T, 0, st>>>(a);
 }
 
 // Pixel pairs (8 x 8 regions) where there are enough of them: with few items
@@ -1607,110 +1147,52 @@ bool fwd_pairs(const RenderShape &s) {
   return bwd_pairs(s) && (!s.sliced || s.total_tiles * (int64_t)(s.tile * s.tile / 64) >= slots);
 }
 
-template <int T>
-void launch_fwd_pair_t(const RasterArgs &a, cudaStream_t st) {
-  const int64_t need = (a.s.total_tiles * (T * T / 64) + PAIR_FWD_WARPS - 1) / PAIR_FWD_WARPS;
-  auto k = raster_fwd_pair_kernel<T>;
-  int64_t grid = (int64_t)blocks_per_sm(k, PAIR_FWD_WARPS * 32) * device_sms();
-  if (grid > need) grid = need;
-  LaunchScope ls(KID_RASTER_FWD, st);
-  k<<<(unsigned)grid, PAIR_FWD_WARPS * 32, 0, st>>>(a);
-}
-
-template <int T>
-void launch_bwd_pair_t(const RasterArgs &a, cudaStream_t st) {
-  if (prepare_raster_kernels() != cudaSuccess) return;  // surfaces via cudaGetLastError
-  auto k = raster_bwd_pair_kernel<T>;
-  const int64_t need = (a.s.total_tiles * (T * T / 64) + PAIR_BWD_WARPS - 1) / PAIR_BWD_WARPS;
-  int64_t grid = (int64_t)blocks_per_sm(k, PAIR_BWD_WARPS * 32, PAIR_BWD_SMEM) * device_sms();
-  if (grid > need) grid = need;
-  LaunchScope ls(KID_RASTER_BWD, st);
-  k<<<(unsigned)grid, PAIR_BWD_WARPS * 32, PAIR_BWD_SMEM, st>>>(a);
+// A persistent grid: every resident block, at most one warp per item.
+template <class Kernel>
+void launch_items(Kernel k, int kid, const RasterArgs &a, int regions, int warps, size_t dyn, cudaStream_t st) {
+  const int64_t need = (a.s.total_tiles * regions + warps - 1) / warps;
+  const int64_t grid = std::min<int64_t>((int64_t)blocks_per_sm(k, warps * 32, dyn) * device_sms(), need);
+  LaunchScope ls((KernelId)kid, st);
+  k<<<(unsigned)grid, warps * 32, dyn, st>>>(a);
 }
 
 template <int T, bool PIX>
-void launch_fwd_warp_t(const RasterArgs &a, cudaStream_t st) {
-  const int64_t need = (a.s.total_tiles * (T * T / 32) + WARPS - 1) / WARPS;
-  auto k = raster_fwd_warp_kernel<T, PIX, false>;
-  if constexpr (!PIX) {
-    if (fwd_pairs(a.s)) {
-      launch_fwd_pair_t<T>(a, st);
-      return;
-    }
-    if (bwd_pairs(a.s)) k = raster_fwd_warp_kernel<T, PIX, true>;
-  }
-  int64_t grid = (int64_t)blocks_per_sm(k, WARPS * 32) * device_sms();
-  if (grid > need) grid = need;
-  LaunchScope ls(KID_RASTER_FWD, st);
-  k<<<(unsigned)grid, WARPS * 32, 0, st>>>(a);
-}
-
-template <int T>
-void launch_bwd_lane_t(const RasterArgs &a, cudaStream_t st) {
-  if (prepare_raster_kernels() != cudaSuccess) return;  // surfaces via cudaGetLastError
-  auto k = raster_bwd_lane_kernel<T>;
-  const int64_t need = (a.s.total_tiles * (T * T / 32) + LANE_WARPS - 1) / LANE_WARPS;
-  int64_t grid = (int64_t)blocks_per_sm(k, LANE_WARPS * 32, LANE_BWD_SMEM) * device_sms();
-  if (grid > need) grid = need;
-  LaunchScope ls(KID_RASTER_BWD, st);
-  k<<<(unsigned)grid, LANE_WARPS * 32, LANE_BWD_SMEM, st>>>(a);
-}
-
-template <int T, bool PIX>
-void launch_bwd_warp_t(const RasterArgs &a, cudaStream_t st) {
-  if (!PIX) {
-    if (bwd_pairs(a.s)) launch_bwd_pair_t<T>(a, st);
-    else launch_bwd_lane_t<T>(a, st);
+void launch_fwd_t(const RasterArgs &a, cudaStream_t st) {
+  if (PIX || fwd_pairs(a.s)) {
+    launch_items(raster_fwd_pair_kernel<T, PIX>, KID_RASTER_FWD, a, T * T / 64, PAIR_FWD_WARPS, 0, st);
     return;
   }
-  auto k = raster_bwd_warp_kernel<T, PIX>;
-  const int64_t need = (a.s.total_tiles * (T * T / 32) + WARPS - 1) / WARPS;
-  int64_t grid = (int64_t)blocks_per_sm(k, WARPS * 32) * device_sms();
-  if (grid > need) grid = need;
-  LaunchScope ls(KID_RASTER_BWD, st);
-  k<<<(unsigned)grid, WARPS * 32, 0, st>>>(a);
+  auto k = bwd_pairs(a.s) ? raster_fwd_lane_kernel<true> : raster_fwd_lane_kernel<false>;
+  launch_items(k, KID_RASTER_FWD, a, T * T / 32, WARPS, 0, st);
 }
 
-// The warp-streamed kernels count items in 32 bits.
-bool warp_mode(const RenderShape &s, const ddgs_workspace &ws) {
-  return ws.batch_depth == 32 && s.total_tiles * (int64_t)(s.tile * s.tile / 32) < (int64_t(1) << 32);
-}
-
-template <bool PIX>
-void fwd_warp_dispatch(const RasterArgs &a, int tile, cudaStream_t st) {
-  if (a.s.total_tiles <= 0) return;
-  switch (tile) {
-    case 8: launch_fwd_warp_t<8, PIX>(a, st); break;
-    case 16: launch_fwd_warp_t<16, PIX>(a, st); break;
-    default: launch_fwd_warp_t<32, PIX>(a, st); break;
-  }
+template <int T, bool PIX>
+void launch_bwd_t(const RasterArgs &a, cudaStream_t st) {
+  if (prepare_raster_kernels() != cudaSuccess) return;  // surfaces via cudaGetLastError
+  if (PIX || bwd_pairs(a.s))
+    launch_items(raster_bwd_pair_kernel<T, PIX>, KID_RASTER_BWD, a, T * T / 64, PairBwd<PIX>::WARPS,
+                 PairBwd<PIX>::SMEM, st);
+  else
+    launch_items(raster_bwd_lane_kernel<T>, KID_RASTER_BWD, a, T * T / 32, LANE_WARPS, LANE_BWD_SMEM, st);
 }
 
 template <bool PIX>
-void bwd_warp_dispatch(const RasterArgs &a, int tile, cudaStream_t st) {
-  if (a.s.total_tiles <= 0) return;
-  switch (tile) {
-    case 8: launch_bwd_warp_t<8, PIX>(a, st); break;
-    case 16: launch_bwd_warp_t<16, PIX>(a, st); break;
-    default: launch_bwd_warp_t<32, PIX>(a, st); break;
-  }
-}
-
-template <int BATCH, bool PIX>
 void fwd_dispatch(const RasterArgs &a, int tile, cudaStream_t st) {
+  if (a.s.total_tiles <= 0) return;
   switch (tile) {
-    case 8: launch_fwd_t<8, BATCH, PIX>(a, st); break;
-    case 16: launch_fwd_t<16, BATCH, PIX>(a, st); break;
-    default: launch_fwd_t<32, BATCH, PIX>(a, st); break;
+    case 8: launch_fwd_t<8, PIX>(a, st); break;
+    case 16: launch_fwd_t<16, PIX>(a, st); break;
+    default: launch_fwd_t<32, PIX>(a, st); break;
   }
 }
 
-template <int BATCH, bool PIX>
+template <bool PIX>
 void bwd_dispatch(const RasterArgs &a, int tile, cudaStream_t st) {
+  if (a.s.total_tiles <= 0) return;
   switch (tile) {
-    case 8: launch_bwd_t<8, BATCH, PIX>(a, st); break;
-    case 16: launch_bwd_t<16, BATCH, PIX>(a, st); break;
-    default: launch_bwd_t<32, BATCH, PIX>(a, st); break;
+    case 8: launch_bwd_t<8, PIX>(a, st); break;
+    case 16: launch_bwd_t<16, PIX>(a, st); break;
+    default: launch_bwd_t<32, PIX>(a, st); break;
   }
 }
 
@@ -1739,20 +1221,13 @@ void launch_raster_fwd(const RenderShape &s, const RasterParams &p, ddgs_workspa
   a.counter = ws.queue;
   a.req_end = ws.req_time ? ws.req_time + 1 : nullptr;
   cudaMemsetAsync(ws.queue, 0, sizeof(uint32_t), st);
-  if (pr) {  // per-pixel ray angles: one staging depth
+  if (pr) {  // per-pixel ray angles
     a.rec2 = ws.rec2;
     a.world_to_cam = pr->world_to_cam;
     a.detector = pr->detector;
-    if (warp_mode(s, ws)) fwd_warp_dispatch<true>(a, s.tile, st);
-    else fwd_dispatch<256, true>(a, s.tile, st);
-  } else if (warp_mode(s, ws)) {
-    fwd_warp_dispatch<false>(a, s.tile, st);
-  } else if (ws.batch_depth == 128) {
-    fwd_dispatch<128, false>(a, s.tile, st);
-  } else if (ws.batch_depth == 512) {
-    fwd_dispatch<512, false>(a, s.tile, st);
+    fwd_dispatch<true>(a, s.tile, st);
   } else {
-    fwd_dispatch<256, false>(a, s.tile, st);
+    fwd_dispatch<false>(a, s.tile, st);
   }
 }
 
@@ -1773,27 +1248,20 @@ void launch_raster_bwd(const RenderShape &s, const RasterParams &p, ddgs_workspa
   a.counter = ws.queue + 1;
   a.req_end = ws.req_time ? ws.req_time + 1 + s.R : nullptr;
   cudaMemsetAsync(ws.queue + 1, 0, sizeof(uint32_t), st);
-  if (pr) {  // per-pixel ray angles: one staging depth
+  if (pr) {  // per-pixel ray angles
     a.rec2 = ws.rec2;
     a.grad_h = ws.grad_h;
     a.world_to_cam = pr->world_to_cam;
     a.detector = pr->detector;
     a.pose_grad = pr->pose_grad;
-    if (warp_mode(s, ws)) bwd_warp_dispatch<true>(a, s.tile, st);
-    else bwd_dispatch<256, true>(a, s.tile, st);
-  } else if (warp_mode(s, ws)) {
-    bwd_warp_dispatch<false>(a, s.tile, st);
-  } else if (ws.batch_depth == 128) {
-    bwd_dispatch<128, false>(a, s.tile, st);
-  } else if (ws.batch_depth == 512) {
-    bwd_dispatch<512, false>(a, s.tile, st);
+    bwd_dispatch<true>(a, s.tile, st);
   } else {
-    bwd_dispatch<256, false>(a, s.tile, st);
+    bwd_dispatch<false>(a, s.tile, st);
   }
 }
 
 cudaError_t prepare_raster_kernels() {
-  // the per-lane backward keeps its (pixel, entry) tables in dynamic shared
+  // the backward kernels keep their (pixel, entry) tables in dynamic shared
   // memory beyond the default 48 KiB; set once per device, outside any capture
   static std::mutex mu;
   static bool done[64] = {};
@@ -1802,12 +1270,15 @@ cudaError_t prepare_raster_kernels() {
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lk(mu);
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-  for (auto k : {raster_bwd_lane_kernel<8>, raster_bwd_lane_kernel<16>, raster_bwd_lane_kernel<32>}) {
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LANE_BWD_SMEM);
-    if (e != cudaSuccess) return e;
-  }
-  for (auto k : {raster_bwd_pair_kernel<8>, raster_bwd_pair_kernel<16>, raster_bwd_pair_kernel<32>}) {
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_BWD_SMEM);
+  const struct { void (*k)(RasterArgs); size_t smem; } big[] = {
+      {raster_bwd_lane_kernel<8>, LANE_BWD_SMEM}, {raster_bwd_lane_kernel<16>, LANE_BWD_SMEM},
+      {raster_bwd_lane_kernel<32>, LANE_BWD_SMEM},
+      {raster_bwd_pair_kernel<8, false>, PairBwd<false>::SMEM}, {raster_bwd_pair_kernel<16, false>, PairBwd<false>::SMEM},
+      {raster_bwd_pair_kernel<32, false>, PairBwd<false>::SMEM},
+      {raster_bwd_pair_kernel<8, true>, PairBwd<true>::SMEM}, {raster_bwd_pair_kernel<16, true>, PairBwd<true>::SMEM},
+      {raster_bwd_pair_kernel<32, true>, PairBwd<true>::SMEM}};
+  for (const auto &x : big) {
+    e = cudaFuncSetAttribute(x.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)x.smem);
     if (e != cudaSuccess) return e;
   }
   if (dev >= 0 && dev < 64) done[dev] = true;

@@ -137,3 +137,18 @@ def test_pixel_pair_rasterisers(shape, tile, needles, ws):
     st = syn.Settings(near_plane=0.2, tile=tile)
     grads = [g for g in B.GRAD_FIELDS if not (needles and g in ("log_scales", "quats"))]
     _sampled_check(scene, views, st, ws, [0], 3000, 7, grads, depth=32)
+
+
+@pytest.mark.parametrize("shape,tile", [((90, 75), 8), ((90, 75), 16), ((75, 90), 32), ((347, 391), 16),
+                                        ((384, 381), 32)])
+@pytest.mark.parametrize("per_pixel", [False, True])
+def test_picked_batches(shape, tile, per_pixel, ws):
+    """Lists longer than several batches, of which a region's batches pick the
+    covering entries (tiles of 16 and 32), on both sides of the pixel-pair
+    rule; with per-pixel rays too."""
+    H, W = shape
+    scene = syn.uniform_cloud(4000, seed=33, dir_frac=0.5, dir_std=1.0, extent=0.7, log_scale_range=(-4.5, -2.5),
+                              alpha_range=(0.02, 0.6))
+    scene = dataclasses.replace(scene, per_pixel=per_pixel)
+    views = _views([syn.pose_matrix(syn.rot_y(0.2), np.array([0.0, 0.1, 2.0]))], 4.0, 4.0 / W, H, W)
+    _sampled_check(scene, views, syn.Settings(near_plane=0.2, tile=tile), ws, [0], 1500, 7, B.GRAD_FIELDS)
