@@ -1,6 +1,7 @@
 // api.cu -- the C ABI: argument checks, workspace management and the order of
 // the kernels of a render and of its backward pass.
 #include <algorithm>
+#include <climits>
 #include <atomic>
 #include <cstdio>
 #include <cstring>
@@ -92,6 +93,9 @@ struct Layout {
   uint64_t hash = 0;
 };
 
+// Tags the hash of a layout whose depth slices were dropped (drop_slices).
+constexpr uint64_t kUnsliced = 0x5bd1e9955bd1e995ull;
+
 uint64_t mix(uint64_t h, uint64_t x) {
   h ^= x + 0x9e3779b97f4a7c15ull + (h << 6) + (h >> 2);
   return h;
@@ -159,21 +163,21 @@ ddgs_status ensure_tables(ddgs_workspace *ws, int64_t R, int64_t V) {
     CK(cudaFreeHost(ws->h_tab));
     ws->h_tab = nullptr;
   }
-  if (ws->d_req) CK(cudaFree(ws->d_req));
-  if (ws->d_view) CK(cudaFree(ws->d_view));
-  if (ws->req_time) CK(cudaFree(ws->req_time));
-  if (ws->splits) CK(cudaFree(ws->splits));
+  if (ws->tab) CK(cudaFree(ws->tab));
+  ws->tab = nullptr;
   ws->d_req = nullptr;
   ws->d_view = nullptr;
-  ws->splits = nullptr;
   ws->req_time = nullptr;
   ws->req_cap = ws->view_cap = 0;
   CK(cudaHostAlloc(&ws->h_tab, rc * sizeof(ddgs::ReqTab) + vc * sizeof(ddgs::ViewTab),
                    cudaHostAllocDefault));
-  CK(cudaMalloc(&ws->d_req, rc * sizeof(ddgs::ReqTab)));
-  CK(cudaMalloc(&ws->d_view, vc * sizeof(ddgs::ViewTab)));
-  CK(cudaMalloc(&ws->req_time, (1 + 2 * rc) * sizeof(unsigned long long)));
-  CK(cudaMalloc(&ws->splits, vc * ddgs::SLICE_MAX * sizeof(uint32_t)));
+  // one device allocation: request table | view table | request times
+  auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
+  const size_t o_view = up(rc * sizeof(ddgs::ReqTab)), o_time = o_view + up(vc * sizeof(ddgs::ViewTab));
+  CK(cudaMalloc(&ws->tab, o_time + (1 + 2 * rc) * sizeof(unsigned long long)));
+  ws->d_req = reinterpret_cast<ddgs::ReqTab *>(ws->tab);
+  ws->d_view = reinterpret_cast<ddgs::ViewTab *>(ws->tab + o_view);
+  ws->req_time = reinterpret_cast<unsigned long long *>(ws->tab + o_time);
   ws->req_cap = rc;
   ws->view_cap = vc;
   ws->last_hash = 0;
@@ -216,7 +220,6 @@ ddgs_status ensure_lists(ddgs_workspace *ws) {
 }
 
 ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
-  const int64_t blk = s.n_blocks;
   if (s.records > ws->rec_cap || !ws->rec) {
     int64_t cap = s.records + s.records / 4 + 1024;
     ddgs_status st;
@@ -233,12 +236,8 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
     if ((st = grow(ws->grad_h, ws->pix_cap, ws->rec_cap, sizeof(float4)))) return st;
     ws->pix_cap = ws->rec_cap;
   }
-  if (blk > ws->blk_cap || !ws->blk_total) {
-    int64_t cap = blk + blk / 4 + 64;
-    ddgs_status st;
-    if ((st = grow(ws->blk_total, ws->blk_cap, cap, sizeof(uint32_t)))) return st;
-    ws->blk_cap = cap;
-  }
+  // preprocess blocks that no-sync renders may have (a limit, no storage)
+  if (s.n_blocks > ws->blk_cap) ws->blk_cap = s.n_blocks + s.n_blocks / 4 + 64;
   if (s.total_tiles > ws->tile_cap || !ws->ranges) {
     int64_t cap = s.total_tiles + s.total_tiles / 4 + 64;
     ddgs_status st;
@@ -246,12 +245,22 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
     if ((st = grow(ws->order, ws->tile_cap, cap, sizeof(uint32_t)))) return st;
     ws->tile_cap = cap;
   }
-  if (s.total_vtiles > ws->vtile_cap || !ws->vranges) {
+  if (s.sliced && (s.V > ws->split_cap || !ws->splits)) {
+    const int64_t cap = s.V + s.V / 4 + 64;
+    ddgs_status st = grow(ws->splits, ws->split_cap, cap * ddgs::SLICE_MAX, sizeof(uint32_t));
+    if (st) return st;
+    ws->split_cap = cap;
+  }
+  if (s.sliced && (s.total_vtiles > ws->vrange_cap || !ws->vranges)) {
     int64_t cap = s.total_vtiles + s.total_vtiles / 4 + 64;
-    ddgs_status st;
-    if ((st = grow(ws->vranges, ws->vtile_cap, cap, sizeof(uint2)))) return st;
-    int64_t pc = 0;  // the part sums follow the lists
-    if ((st = grow(ws->part, pc, ddgs::part_capacity(cap), sizeof(uint64_t)))) return st;
+    ddgs_status st = grow(ws->vranges, ws->vrange_cap, cap, sizeof(uint2));
+    if (st) return st;
+    ws->vrange_cap = cap;
+  }
+  if (s.total_vtiles > ws->vtile_cap || !ws->part) {  // the part sums follow the lists
+    int64_t cap = s.total_vtiles + s.total_vtiles / 4 + 64;
+    ddgs_status st = grow(ws->part, ws->vtile_cap, ddgs::part_capacity(cap), sizeof(uint64_t));
+    if (st) return st;
     ws->vtile_cap = cap;
   }
   if (s.hist_slots > ws->hist_cap || !ws->hist) {
@@ -261,6 +270,18 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
     ws->hist_cap = cap;
   }
   return ensure_lists(ws);
+}
+
+// A no-sync render on a workspace without room for its depth slices (made for
+// another layout, never reserved for this one) is binned without them.
+void drop_slices(const ddgs_workspace *ws, Layout &L) {
+  ddgs::RenderShape &s = L.shape;
+  if (!s.sliced || (s.total_vtiles <= ws->vtile_cap && s.total_vtiles <= ws->vrange_cap &&
+                    s.V <= ws->split_cap && s.hist_slots <= ws->hist_cap &&
+                    ddgs::list_capacity(s.total_vtiles, ws->pair_cap) <= ws->list_cap))
+    return;
+  ddgs::plan_binning(L.view.data(), L.V, L.req.data(), s.total_tiles, s.tile, s);
+  L.hash ^= kUnsliced;
 }
 
 ddgs_status ensure_pairs(ddgs_workspace *ws, int64_t pairs) {
@@ -286,7 +307,7 @@ struct ProfRec {
 std::vector<ProfRec> g_pending;
 std::vector<cudaEvent_t> g_pool;
 const char *const KERNEL_NAMES[ddgs::KID_COUNT] = {
-    "preprocess_fwd", "scan_blocks", "bin_count", "bin_offsets", "bin_scatter",
+    "preprocess_fwd", "bin_count", "bin_offsets", "bin_scatter",
     "bin_sort", "bin_merge", "raster_fwd", "l1_loss", "raster_bwd",
     "preprocess_bwd", "debug_copy", "tile_order", "rads_minmax", "rads_count", "rads_scan",
     "rads_emit", "rads_select", "rads_draw", "rads_knn"};
@@ -410,18 +431,14 @@ ddgs_status ddgs_workspace_create(ddgs_workspace **out) {
   if (!ws) return DDGS_ERR_OUT_OF_MEMORY;
   cudaError_t e;
   if ((e = cudaGetDevice(&ws->device)) != cudaSuccess ||
-      (e = cudaMalloc(&ws->d_pairs, sizeof(uint64_t))) != cudaSuccess ||
-      (e = cudaMalloc(&ws->d_status, sizeof(int32_t))) != cudaSuccess ||
-      (e = cudaMalloc(&ws->queue, 2 * sizeof(uint32_t))) != cudaSuccess ||
-      (e = cudaMalloc(&ws->list_count, ddgs::BIN_COUNTERS * sizeof(uint32_t))) != cudaSuccess ||
-      (e = cudaHostAlloc(&ws->h_pairs, 2 * sizeof(uint64_t), cudaHostAllocDefault)) != cudaSuccess ||
-      (e = cudaMemset(ws->d_status, 0, sizeof(int32_t))) != cudaSuccess ||
-      (e = cudaMemset(ws->d_pairs, 0, sizeof(uint64_t))) != cudaSuccess) {
+      (e = cudaMalloc(&ws->head, sizeof(ddgs::RenderHead))) != cudaSuccess ||
+      (e = cudaHostAlloc(&ws->h_head, 3 * sizeof(uint64_t), cudaHostAllocDefault)) != cudaSuccess ||
+      (e = cudaMemset(ws->head, 0, sizeof(ddgs::RenderHead))) != cudaSuccess) {
     ddgs_status st = cuda_fail(e, "workspace create");
     ddgs_workspace_destroy(ws);
     return st;
   }
-  ws->h_pairs[0] = ws->h_pairs[1] = 0;
+  ws->h_head[0] = ws->h_head[1] = ws->h_head[2] = 0;
   if (ensure_tables(ws, 0, 0) != DDGS_OK) {
     ddgs_workspace_destroy(ws);
     return DDGS_ERR_OUT_OF_MEMORY;
@@ -438,14 +455,12 @@ ddgs_status ddgs_workspace_create(ddgs_workspace **out) {
 
 ddgs_status ddgs_workspace_destroy(ddgs_workspace *ws) {
   if (!ws) return DDGS_OK;
-  void *dev[] = {ws->rec, ws->rect, ws->tiles_touched, ws->grad2d, ws->blk_total,
-                 ws->keys[0], ws->keys[1], ws->vals, ws->hist, ws->part, ws->lists,
-                 ws->list_count, ws->ranges, ws->vranges, ws->splits, ws->d_pairs, ws->d_status, ws->d_req, ws->d_view,
-                 ws->order, ws->queue, ws->req_time, ws->rec2, ws->grad_h,
-                 ws->rads_keys, ws->rads_buf};
+  void *dev[] = {ws->rec, ws->rect, ws->tiles_touched, ws->grad2d, ws->keys[0], ws->keys[1], ws->vals,
+                 ws->hist, ws->part, ws->lists, ws->ranges, ws->vranges, ws->head, ws->tab, ws->order,
+                 ws->rec2, ws->grad_h, ws->rads_keys, ws->rads_buf};
   for (void *p : dev)
     if (p) cudaFree(p);
-  if (ws->h_pairs) cudaFreeHost(ws->h_pairs);
+  if (ws->h_head) cudaFreeHost(ws->h_head);
   if (ws->h_tab) cudaFreeHost(ws->h_tab);
   delete ws;
   return DDGS_OK;
@@ -463,6 +478,8 @@ ddgs_status ddgs_workspace_reserve(ddgs_workspace *ws, int64_t records, int64_t 
   s.n_blocks = records / ddgs::PRE_THREADS + 4096;
   s.total_tiles = tiles;
   s.total_vtiles = ddgs::vtile_bound(tiles, records);
+  s.sliced = 1;  // a sliced view has more than SLICE_FROM records
+  s.V = (int32_t)std::min<int64_t>(records / ddgs::SLICE_FROM + 1, INT32_MAX / 2);
   s.hist_slots = ddgs::hist_slot_bound(s.total_vtiles);
   ddgs_status st = ensure_records(ws, s);
   if (st) return st;
@@ -487,6 +504,7 @@ ddgs_status render_common(const ddgs_gaussians &g, const ddgs_views &v, const dd
   ddgs_status st;
   ddgs::RenderShape &s = L.shape;
   if (c->no_sync) {
+    drop_slices(ws, L);
     if (s.records > ws->rec_cap || s.n_blocks > ws->blk_cap || s.total_tiles > ws->tile_cap ||
         s.total_vtiles > ws->vtile_cap || s.hist_slots > ws->hist_cap || !ws->keys[0] ||
         ddgs::list_capacity(s.total_vtiles, ws->pair_cap) > ws->list_cap)
@@ -503,37 +521,43 @@ ddgs_status render_common(const ddgs_gaussians &g, const ddgs_views &v, const dd
   }
   if ((st = upload_layout(ws, L, c->no_sync != 0, s_))) return st;
   ws->have_render = false;
-  // timing slots: batch start (min) and per-request ends (max)
-  CK(cudaMemsetAsync(ws->req_time, 0xff, sizeof(unsigned long long), s_));
-  CK(cudaMemsetAsync(ws->req_time + 1, 0, 2 * (size_t)s.R * sizeof(unsigned long long), s_));
+  CK(cudaMemsetAsync(reinterpret_cast<unsigned char *>(ws->head) + ddgs::HEAD_CLEARED, 0,
+                     sizeof(ddgs::RenderHead) - ddgs::HEAD_CLEARED, s_));
+  // the timing slots (batch start, per-request ends) and the list sums are
+  // cleared by the preprocess for the kernels after it
+  const int64_t n_part = ddgs::part_capacity(s.total_vtiles);
   uint64_t bound = 0;
   bool nonfinite = false;
   if (s.records > 0) {
-    ddgs::launch_preprocess_fwd(g, v, *c, s, *ws, s_);
+    ddgs::ZeroList zero;
+    zero.add(ws->req_time + 1, 4 * (int64_t)s.R);
+    zero.add(ws->part, 2 * n_part);
+    ddgs::launch_preprocess_fwd(g, v, *c, s, *ws, zero, s_);
     CK(cudaGetLastError());
-    ddgs::launch_scan_blocks(s.n_blocks, *ws, s_);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(ws->h_pairs, ws->d_pairs, sizeof(uint64_t), cudaMemcpyDeviceToHost, s_));
+    // the status word rides along with the pair count
+    CK(cudaMemcpyAsync(ws->h_head, ws->head, 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s_));
     if (!c->no_sync) {
-      // the status word rides along with the pair count: a non-finite input
-      // is reported by this call (and cleared), other bits stay latched
-      int32_t *h_st = reinterpret_cast<int32_t *>(ws->h_pairs + 1);
-      CK(cudaMemcpyAsync(h_st, ws->d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, s_));
+      // a non-finite input is reported by this call (and cleared), other bits
+      // stay latched
       CK(cudaStreamSynchronize(s_));
-      if (h_st[0] & ddgs::ST_NONFINITE) {
+      const int32_t status = *reinterpret_cast<const int32_t *>(ws->h_head);
+      if (status & ddgs::ST_NONFINITE) {
         nonfinite = true;
-        h_st[1] = h_st[0] & ~ddgs::ST_NONFINITE;
-        CK(cudaMemcpyAsync(ws->d_status, h_st + 1, sizeof(int32_t), cudaMemcpyHostToDevice, s_));
+        int32_t *keep = reinterpret_cast<int32_t *>(ws->h_head + 2);
+        *keep = status & ~ddgs::ST_NONFINITE;
+        CK(cudaMemcpyAsync(&ws->head->status, keep, sizeof(int32_t), cudaMemcpyHostToDevice, s_));
       }
-      bound = *ws->h_pairs;
+      bound = ws->h_head[1];
       if (bound > (uint64_t)ddgs::BIN_MAX_PAIRS) return DDGS_ERR_CAPACITY;
       if ((st = ensure_pairs(ws, (int64_t)bound))) return st;
     } else {
       bound = (uint64_t)ws->pair_cap;
     }
   } else {
-    *ws->h_pairs = 0;
-    CK(cudaMemsetAsync(ws->d_pairs, 0, sizeof(uint64_t), s_));
+    ws->h_head[1] = 0;
+    CK(cudaMemsetAsync(ws->req_time, 0xff, sizeof(unsigned long long), s_));  // no start: no times
+    CK(cudaMemsetAsync(ws->req_time + 1, 0, 2 * (size_t)s.R * sizeof(unsigned long long), s_));
+    CK(cudaMemsetAsync(ws->part, 0, (size_t)n_part * sizeof(uint64_t), s_));
   }
   if (s.total_tiles > 0) {
     ddgs::launch_binning(s, bound, *ws, s_);
@@ -559,7 +583,7 @@ ddgs_status backward_common(const ddgs_gaussians &g, const ddgs_views &v, const 
                             Layout &L, ddgs_workspace *ws, const float *dL_dimage,
                             const float *t_final, const uint32_t *n_last, const ddgs_grads *out,
                             cudaStream_t s_) {
-  if (!ws || !out || !ws->have_render || L.hash != ws->last_hash ||
+  if (!ws || !out || !ws->have_render || (L.hash != ws->last_hash && (L.hash ^ kUnsliced) != ws->last_hash) ||
       (g.per_pixel != 0) != ws->last_per_pixel || !on_workspace_device(ws))
     return DDGS_ERR_INVALID_ARG;
   ddgs::RenderShape &s = L.shape;
@@ -570,11 +594,20 @@ ddgs_status backward_common(const ddgs_gaussians &g, const ddgs_views &v, const 
       (out->feat_dir && !aligned16(out->feat_dir)))
     return DDGS_ERR_INVALID_ARG;
   const int kf = g.feat_dim ? g.feat_dim : ddgs::K, lsh = g.sh_degree ? g.sh_degree : 1;
-  if (out->b_iso) CK(cudaMemsetAsync(out->b_iso, 0, (size_t)s.R * kf * sizeof(float), s_));
-  if (out->B_dir)
-    CK(cudaMemsetAsync(out->B_dir, 0, (size_t)s.R * lsh * (lsh + 2) * kf * sizeof(float), s_));
-  if (out->world_to_cam)
-    CK(cudaMemsetAsync(out->world_to_cam, 0, (size_t)s.V * 12 * sizeof(float), s_));
+  // the gradients that blocks add to start at zero: cleared by the backward
+  // rasteriser for the backward preprocess, or by a memset where it does not run
+  // or (per-pixel rays) adds to the pose gradient itself
+  const bool rasters = s.n_total > 0 && s.records > 0 && s.total_tiles > 0 && ws->pair_bound > 0;
+  ddgs::ZeroList zero;
+  auto clear = [&](float *p, int64_t n, bool now) -> cudaError_t {
+    if (!p) return cudaSuccess;
+    if (now) return cudaMemsetAsync(p, 0, (size_t)n * sizeof(float), s_);
+    zero.add(p, n);
+    return cudaSuccess;
+  };
+  CK(clear(out->b_iso, (int64_t)s.R * kf, !rasters));
+  CK(clear(out->B_dir, (int64_t)s.R * lsh * (lsh + 2) * kf, !rasters));
+  CK(clear(out->world_to_cam, (int64_t)s.V * 12, !rasters || g.per_pixel));
   if (s.n_total == 0) return DDGS_OK;  // parameter gradients empty, pose/basis zero
   // The rasteriser accumulates 2D gradients into zeros, and the backward
   // preprocess clears every record it consumes, so the buffers are cleared
@@ -587,12 +620,12 @@ ddgs_status backward_common(const ddgs_gaussians &g, const ddgs_views &v, const 
   ws->grad_zero = false;  // until both kernels are queued
   ddgs::RasterParams P{c->alpha_min, c->alpha_max, c->t_min, c->q_max,
                           c->q_max * ddgs::CONIC_SCALE};
-  if (s.records > 0 && s.total_tiles > 0 && ws->pair_bound > 0) {
+  if (rasters) {
     ddgs::PixelRays pr;
     pr.world_to_cam = v.world_to_cam;
     pr.detector = v.detector;
     pr.pose_grad = out->world_to_cam;
-    ddgs::launch_raster_bwd(s, P, *ws, dL_dimage, t_final, n_last, g.per_pixel ? &pr : nullptr, s_);
+    ddgs::launch_raster_bwd(s, P, *ws, dL_dimage, t_final, n_last, g.per_pixel ? &pr : nullptr, zero, s_);
     CK(cudaGetLastError());
   }
   ddgs::launch_preprocess_bwd(g, v, *c, s, *ws, *out, s_);
@@ -734,13 +767,15 @@ ddgs_status ddgs_request_times(const ddgs_workspace *ws, uint64_t *fwd_ns, uint6
 
 ddgs_status ddgs_workspace_pairs(const ddgs_workspace *ws, int64_t *pairs) {
   if (!ws || !pairs) return DDGS_ERR_INVALID_ARG;
-  *pairs = (int64_t)*ws->h_pairs;
+  *pairs = (int64_t)ws->h_head[1];
   return DDGS_OK;
 }
 
 }  // extern "C"
 
 namespace {
+using ddgs::after_previous;
+
 __global__ void tiles_touched_kernel(const uint4 *info, int64_t n, uint32_t *out) {
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
        j += (int64_t)gridDim.x * blockDim.x)
@@ -759,17 +794,17 @@ __global__ void list_keys_kernel(ddgs::RenderShape s, const uint2 *ranges, const
   }
 }
 
-__global__ void l1_loss_kernel(const float *image, const float *target, int per_view, int64_t hw,
+__global__ void l1_loss_kernel(const float *image, const float *target, int per_view, int bx, int64_t hw,
                                float *loss, float *grad) {
-  // one block row per view: blockIdx.y = view
-  const int v = blockIdx.y;
+  // bx blocks per view
+  after_previous();
+  const int v = blockIdx.x / bx, b0 = blockIdx.x % bx;
   const float *img = image + (int64_t)v * hw;
   const float *tgt = target + (per_view ? (int64_t)v * hw : 0);
   float *gr = grad + (int64_t)v * hw;
   const float inv = 1.0f / (float)hw;
   float acc = 0.f;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < hw;
-       j += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t j = (int64_t)b0 * blockDim.x + threadIdx.x; j < hw; j += (int64_t)bx * blockDim.x) {
     const float d = img[j] - tgt[j];
     acc += fabsf(d);
     gr[j] = d > 0.f ? inv : (d < 0.f ? -inv : 0.f);
@@ -792,9 +827,9 @@ void launch_l1_loss(const float *image, const float *target, int per_view, int V
                     float *loss, float *grad, cudaStream_t st) {
   int64_t bx = (hw + 255) / 256;
   if (bx > 64) bx = 64;
-  dim3 grid((unsigned)bx, (unsigned)V);
   LaunchScope ls(KID_L1_LOSS, st);
-  l1_loss_kernel<<<grid, 256, 0, st>>>(image, target, per_view, hw, loss, grad);
+  launch_next(l1_loss_kernel, (unsigned)bx * (unsigned)V, 256u, 0, st, image, target, per_view, (int)bx, hw, loss,
+              grad);
 }
 }  // namespace ddgs
 
@@ -813,7 +848,7 @@ ddgs_status ddgs_debug_binning(const ddgs_workspace *ws, uint32_t *tiles_touched
                                                       s.records, tiles_touched);
     CK(cudaGetLastError());
   }
-  uint64_t m = *ws->h_pairs;
+  uint64_t m = ws->h_head[1];
   if (m > (uint64_t)ws->pair_cap) m = (uint64_t)ws->pair_cap;  // after an overflow
   if (keys && m && s.total_tiles > 0) {
     int64_t b = (s.total_tiles + 255) / 256;
@@ -846,8 +881,8 @@ ddgs_status ddgs_sync_status(ddgs_workspace *ws, void *stream) {
   cudaStream_t s_ = static_cast<cudaStream_t>(stream);
   int32_t h = 0;
   CK(cudaStreamSynchronize(s_));
-  CK(cudaMemcpy(&h, ws->d_status, sizeof(int32_t), cudaMemcpyDeviceToHost));
-  CK(cudaMemset(ws->d_status, 0, sizeof(int32_t)));
+  CK(cudaMemcpy(&h, &ws->head->status, sizeof(int32_t), cudaMemcpyDeviceToHost));
+  CK(cudaMemset(&ws->head->status, 0, sizeof(int32_t)));
   if (h & ddgs::ST_CAPACITY) return DDGS_ERR_CAPACITY;
   if (h & ddgs::ST_NONFINITE) return DDGS_ERR_NONFINITE;
   return DDGS_OK;

@@ -36,59 +36,7 @@ constexpr int SORT_SHORT = 1024;  // lists of one 128-thread block (8 entries a 
 constexpr int SORT_MID = 2048;    // lists of one 128-thread block (16 entries a thread)
 constexpr int MERGE_ITEMS = 8;    // outputs per thread per merge step
 constexpr int BIN_LOADS = 4;      // records a thread loads before using them
-
-// ---------------------------------------------------------------------------
-// Exclusive scan of block totals -> offsets (optional) and the total (one block)
-// ---------------------------------------------------------------------------
-template <typename In>
-__global__ void __launch_bounds__(1024) scan_blocks_kernel(const In *in, uint64_t *out, int64_t n,
-                                                            uint64_t *total) {
-  __shared__ uint64_t s_warp[32];
-  __shared__ uint64_t s_carry;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (tid == 0) s_carry = 0;
-  __syncthreads();
-  constexpr int PER = 4;
-  for (int64_t base = 0; base < n; base += 1024 * PER) {
-    uint64_t x[PER], sum = 0;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      int64_t j = base + (int64_t)tid * PER + k;
-      x[k] = j < n ? (uint64_t)in[j] : 0;
-      sum += x[k];
-    }
-    uint64_t inc = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) s_warp[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-      uint64_t w = s_warp[lane];
-      uint64_t wi = w;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        uint64_t y = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += y;
-      }
-      s_warp[lane] = wi - w;  // exclusive prefix of warp totals
-    }
-    __syncthreads();
-    uint64_t run = s_carry + s_warp[wid] + inc - sum;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      int64_t j = base + (int64_t)tid * PER + k;
-      if (j < n && out) out[j] = run;
-      run += x[k];
-    }
-    __syncthreads();
-    if (tid == 1023) s_carry = run;
-    __syncthreads();
-  }
-  if (tid == 0 && total) *total = s_carry;
-}
+constexpr uint64_t SORT_EARLY = uint64_t(1) << 22;  // pairs up to which the sorts' launches overlap
 
 // ---------------------------------------------------------------------------
 // Binning blocks: (view, chunk of its Gaussians, band of its tiles)
@@ -134,6 +82,7 @@ constexpr int SLICE_SAMPLE = 512;
 __global__ void __launch_bounds__(SLICE_SAMPLE) bin_slices_kernel(RenderShape s, const uint4 *info,
                                                                   uint32_t *splits) {
   __shared__ uint32_t s_d[SLICE_SAMPLE];
+  after_previous();
   const ViewTab vt = s.view[blockIdx.x];
   if (vt.lg_slices == 0) return;
   const int t = threadIdx.x;
@@ -180,6 +129,7 @@ __global__ void __launch_bounds__(BIN_THREADS, 8) bin_count_kernel(RenderShape s
                                                                   uint32_t *hist) {
   extern __shared__ uint32_t s_cnt[];
   __shared__ uint32_t s_sp[SLICE_MAX];
+  after_previous();
   const int v = find_item_view(s.view, s.V, blockIdx.x);
   const ViewTab vt = s.view[v];
   const BinItem it = bin_item(s, vt, blockIdx.x);
@@ -243,6 +193,7 @@ __global__ void __launch_bounds__(COL_WARPS * 32) bin_column_kernel(RenderShape 
                                                                      uint32_t *hist, uint2 *vranges,
                                                                      uint64_t *part) {
   __shared__ uint32_t s_sum[COL_WARPS][32];
+  after_previous();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t gt = (int64_t)blockIdx.x * 32 + lane;
   int64_t first = 0, stride = 0;
@@ -317,7 +268,7 @@ __device__ __forceinline__ void list_append(const BinLists &L, int cls, uint64_t
   for (uint32_t c = 0; c < k; ++c) L.item[cls][base + c] = (gt << 24) | c;
 }
 
-// offsets, part 2: list ranges from the exclusive scan of the totals ((0, 0)
+// offsets, part 2: list ranges from the exclusive sums of the totals ((0, 0)
 // for an empty list), and each list of two or more entries queued for its
 // sort. A tile whose lists do not all fit below the pair capacity is left
 // empty (whole tiles only) and the capacity status is raised. With depth
@@ -325,11 +276,12 @@ __device__ __forceinline__ void list_append(const BinLists &L, int cls, uint64_t
 // neighbours in the warp. Every tile is counted in its length bucket (lpt) for
 // the rasterisers' work order.
 __global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 *ranges, uint2 *vranges,
-                                                             const uint64_t *part_off, uint64_t cap,
+                                                             const uint64_t *part, uint64_t cap,
                                                              BinLists L, uint32_t *lpt,
                                                              int32_t *status) {
-  __shared__ uint64_t s_w[32];
+  __shared__ uint64_t s_w[32], s_p[32];
   __shared__ uint32_t s_lpt[LPT_BUCKETS];
+  after_previous();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t gt = (int64_t)blockIdx.x * 1024 + threadIdx.x;
   const bool in = gt < s.total_vtiles;
@@ -342,8 +294,16 @@ __global__ void __launch_bounds__(1024) bin_offsets_kernel(RenderShape s, uint2 
   }
   if (lane == 31) s_w[wid] = inc;
   if (threadIdx.x < LPT_BUCKETS) s_lpt[threadIdx.x] = 0;
+  // the lists of the groups before (every block sums its own predecessors: one
+  // launch less than a scan of the group sums)
+  uint64_t before = 0;
+  for (int64_t g = threadIdx.x; g < blockIdx.x; g += 1024) before += part[g];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if (lane == 0) s_p[wid] = before;
   __syncthreads();
-  uint64_t before = part_off[blockIdx.x];
+  before = 0;
+  for (int w = 0; w < 32; ++w) before += s_p[w];
   for (int w = 0; w < wid; ++w) before += s_w[w];
   const uint64_t off = before + inc - cnt;
   uint64_t end = off + cnt;  // of the whole tile
@@ -474,6 +434,7 @@ __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShap
                                                                     uint64_t *keys, uint32_t *vals,
                                                                     uint64_t cap) {
   extern __shared__ __align__(16) unsigned char scat_smem[];
+  after_previous();
   __shared__ uint32_t s_wsum[SCAT_THREADS / 32];
   __shared__ uint32_t s_sp[SLICE_MAX];
   const int v = find_item_view(s.view, s.V, blockIdx.x);
@@ -612,6 +573,7 @@ __global__ void __launch_bounds__(256) bin_sort_warp_kernel(const uint64_t *item
                                                               const uint32_t *count,
                                                               const uint2 *ranges,
                                                               const uint64_t *keys, uint32_t *vals) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const uint32_t n_items = *count;
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
@@ -757,6 +719,7 @@ __global__ void __launch_bounds__(NT, MINB) bin_sort_block_kernel(const uint64_t
   __shared__ uint32_t s_red[4][NW];
   uint32_t *bc = s_bk;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  after_previous();
   const uint32_t n_items = *count;
   // the next item's keys are copied to s_buf asynchronously while the
   // current one is placed (once its keys have left s_buf)
@@ -933,6 +896,7 @@ __global__ void __launch_bounds__(NT, MINB) bin_sort_block_kernel(const uint64_t
 __global__ void __launch_bounds__(256) bin_merge_kernel(const uint64_t *items, const uint32_t *count,
                                                          const uint2 *ranges, uint64_t *keys0,
                                                          uint64_t *keys1, uint32_t *vals) {
+  after_previous();
   const uint32_t n_items = *count;
   for (uint32_t i = blockIdx.x; i < n_items; i += gridDim.x) {
     const uint2 r = ranges[items[i] >> 24];
@@ -974,18 +938,13 @@ constexpr size_t LONG_SMEM = 2 * (size_t)BIN_LIST_LONG * sizeof(uint64_t);
 
 }  // namespace
 
-void launch_scan_blocks(int64_t nblk, ddgs_workspace &ws, cudaStream_t st) {
-  LaunchScope ls(KID_SCAN_BLOCKS, st);
-  scan_blocks_kernel<uint32_t><<<1, 1024, 0, st>>>(ws.blk_total, nullptr, nblk, ws.d_pairs);
-}
-
 int64_t list_capacity(int64_t tiles, int64_t pairs) {
   // per class at most one entry per tile, plus one per BIN_LIST_LONG pairs for
   // the chunks of long lists
   return LIST_CLASSES * tiles + pairs / BIN_LIST_LONG + 64;
 }
 
-int64_t part_capacity(int64_t tiles) { return 2 * ((tiles + 1023) / 1024) + 2; }
+int64_t part_capacity(int64_t tiles) { return (tiles + 1023) / 1024 + 1; }
 
 
 cudaError_t prepare_bin_kernels() {
@@ -1022,41 +981,33 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
   const unsigned sms = (unsigned)device_sms();  // the sorts run persistent blocks per SM
   const bool pairs = pair_bound > 0 && s.n_items > 0;
   uint2 *vranges = s.sliced ? ws.vranges : ws.ranges;
+  const uint4 *info = reinterpret_cast<const uint4 *>(ws.rect);
   if (pairs && s.sliced) {
     LaunchScope ls(KID_BIN_OFFSETS, st);
-    bin_slices_kernel<<<(unsigned)s.V, SLICE_SAMPLE, 0, st>>>(
-        s, reinterpret_cast<const uint4 *>(ws.rect), ws.splits);
+    launch_next(bin_slices_kernel, (unsigned)s.V, SLICE_SAMPLE, 0, st, s, info, ws.splits);
   }
   if (pairs) {
     LaunchScope ls(KID_BIN_COUNT, st);
     auto k = s.sliced ? bin_count_kernel<true> : bin_count_kernel<false>;
-    k<<<(unsigned)s.n_items, BIN_THREADS, hsm, st>>>(s, reinterpret_cast<const uint4 *>(ws.rect),
-                                                     ws.splits, ws.hist);
+    launch_next(k, (unsigned)s.n_items, BIN_THREADS, hsm, st, s, info, ws.splits, ws.hist);
   }
   const int64_t nb = (T + 1023) / 1024;
-  uint64_t *part = ws.part, *part_off = ws.part + nb + 1;
   BinLists L;  // at most T entries per class, except the chunks of long lists (last)
   L.item[LIST_WARP] = ws.lists;
   L.item[LIST_SHORT] = ws.lists + T;
   L.item[LIST_MID] = ws.lists + 2 * T;
   L.item[LIST_LONG] = ws.lists + 3 * T;
   L.item[LIST_BLOCK] = ws.lists + 4 * T;
-  L.count = ws.list_count;
-  cudaMemsetAsync(ws.list_count, 0, BIN_COUNTERS * sizeof(uint32_t), st);
-  cudaMemsetAsync(part, 0, (size_t)nb * sizeof(uint64_t), st);
+  L.count = ws.head->counters;
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
-    bin_column_kernel<<<(unsigned)((T + 31) / 32), COL_WARPS * 32, 0, st>>>(s, pairs ? 1 : 0, ws.hist,
-                                                                          vranges, part);
+    launch_next(bin_column_kernel, (unsigned)((T + 31) / 32), COL_WARPS * 32, 0, st, s, pairs ? 1 : 0, ws.hist,
+                vranges, ws.part);
   }
   {
     LaunchScope ls(KID_BIN_OFFSETS, st);
-    scan_blocks_kernel<uint64_t><<<1, 1024, 0, st>>>(part, part_off, nb, nullptr);
-  }
-  {
-    LaunchScope ls(KID_BIN_OFFSETS, st);
-    bin_offsets_kernel<<<(unsigned)nb, 1024, 0, st>>>(s, ws.ranges, vranges, part_off, cap, L,
-                                                      ws.list_count + LIST_CLASSES, ws.d_status);
+    launch_next(bin_offsets_kernel, (unsigned)nb, 1024u, 0, st, s, ws.ranges, vranges, ws.part, cap, L,
+                ws.head->counters + LIST_CLASSES, &ws.head->status);
   }
   if (!pairs) return;
   {
@@ -1065,22 +1016,24 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
     const bool direct = pair_bound > 2u * (uint64_t)scatter_stage(false, s.sliced) * (uint64_t)s.n_items;
     auto k = s.sliced ? (direct ? bin_scatter_kernel<true, true> : bin_scatter_kernel<false, true>)
                       : (direct ? bin_scatter_kernel<true, false> : bin_scatter_kernel<false, false>);
-    k<<<(unsigned)s.n_items, SCAT_THREADS, scatter_smem(s.hist_area, direct, s.sliced), st>>>(
-        s, reinterpret_cast<const uint4 *>(ws.rect), ws.splits, ws.hist, vranges, ws.keys[0], ws.vals, cap);
+    launch_next(k, (unsigned)s.n_items, SCAT_THREADS, scatter_smem(s.hist_area, direct, s.sliced), st, s, info,
+                ws.splits, ws.hist, vranges, ws.keys[0], ws.vals, cap);
   }
   // A list holds at most one entry per Gaussian of its request, so a render of
   // n_total Gaussians in all cannot fill the classes of longer lists: those
   // sorts (and the merge) are not launched.
   const int64_t nmax = s.n_total;
+  // the sorts of many pairs fill the SMs for long: no early start (launch_kernel)
+  const bool early = pair_bound <= SORT_EARLY;
   if (nmax >= 2) {
     LaunchScope ls(KID_BIN_SORT, st);
-    bin_sort_warp_kernel<<<sms * 4, 256, 0, st>>>(L.item[LIST_WARP], L.count + LIST_WARP,
-                                                   vranges, ws.keys[0], ws.vals);
+    launch_kernel(early, bin_sort_warp_kernel, sms * 4, 256u, 0, st, L.item[LIST_WARP], L.count + LIST_WARP, vranges,
+                ws.keys[0], ws.vals);
   }
   if (nmax > 32) {
     LaunchScope ls(KID_BIN_SORT, st);
-    bin_sort_block_kernel<128, SORT_SHORT / 128, 8><<<sms * 8, 128, SHORT_SMEM, st>>>(
-        L.item[LIST_SHORT], L.count + LIST_SHORT, vranges, ws.keys[0], ws.vals);
+    launch_kernel(early, bin_sort_block_kernel<128, SORT_SHORT / 128, 8>, sms * 8, 128u, SHORT_SMEM, st, L.item[LIST_SHORT],
+                L.count + LIST_SHORT, vranges, ws.keys[0], ws.vals);
   }
   if (nmax > SORT_SHORT) {
     LaunchScope ls(KID_BIN_SORT, st);
@@ -1088,19 +1041,18 @@ void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &w
     // bucket counters 0.636 -> 0.629 ms for the sorts at 64 poses against five
     // at 96 registers (which led before the padding, 0.69 against 0.72; four
     // at 128 registers measured 0.75)
-    bin_sort_block_kernel<128, SORT_MID / 128, 6><<<sms * 6, 128, MID_SMEM, st>>>(
-        L.item[LIST_MID], L.count + LIST_MID, vranges, ws.keys[0], ws.vals);
+    launch_kernel(early, bin_sort_block_kernel<128, SORT_MID / 128, 6>, sms * 6, 128u, MID_SMEM, st, L.item[LIST_MID],
+                L.count + LIST_MID, vranges, ws.keys[0], ws.vals);
   }
   if (nmax > SORT_MID) {
     LaunchScope ls(KID_BIN_SORT, st);
-    bin_sort_block_kernel<SORT_LONG_THREADS, SORT_LONG_ITEMS, 1>
-        <<<sms, SORT_LONG_THREADS, LONG_SMEM, st>>>(L.item[LIST_BLOCK], L.count + LIST_BLOCK,
-                                                   vranges, ws.keys[0], ws.vals);
+    launch_kernel(early, bin_sort_block_kernel<SORT_LONG_THREADS, SORT_LONG_ITEMS, 1>, sms, SORT_LONG_THREADS, LONG_SMEM, st,
+                L.item[LIST_BLOCK], L.count + LIST_BLOCK, vranges, ws.keys[0], ws.vals);
   }
   if (nmax > BIN_LIST_LONG) {
     LaunchScope ls(KID_BIN_MERGE, st);
-    bin_merge_kernel<<<sms * 2, 256, 0, st>>>(L.item[LIST_LONG], L.count + LIST_LONG, vranges,
-                                              ws.keys[0], ws.keys[1], ws.vals);
+    launch_kernel(early, bin_merge_kernel, sms * 2, 256u, 0, st, L.item[LIST_LONG], L.count + LIST_LONG, vranges, ws.keys[0],
+                ws.keys[1], ws.vals);
   }
 }
 

@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/ddgs.h"
@@ -57,11 +58,12 @@ struct ViewTab {
   int64_t item_base;  // first binning block of the view
   int64_t hist_base;  // first tile counter of the view
   int32_t chunks;     // Gaussian chunks (0 for an empty request)
-  int32_t band_w, band_h, bands_x;  // bands of band_w x band_h tiles, row-major
-  int32_t lg_slices;                // each tile has 2^lg_slices lists, by depth
-  int64_t vtile_base;               // first list of the view: lists are numbered tile by
-                                    // tile, and within a tile by depth
+  uint16_t band_w, band_h, bands_x;  // bands of band_w x band_h tiles (at most BIN_HIST_MAX), row-major
+  uint16_t lg_slices;                // each tile has 2^lg_slices lists, by depth
+  uint32_t vtile_base;               // first list of the view: lists are numbered tile by
+                                     // tile, and within a tile by depth
 };
+static_assert(sizeof(ViewTab) == 72, "the pinned copy of the tables is made with every workspace");
 
 // Per-view constants staged in shared memory by the preprocess kernels
 // (IEEE-exact where the binning depends on them).
@@ -94,9 +96,75 @@ __device__ __forceinline__ int lpt_bucket(uint2 r) {
   const int lg = 31 - __clz(len);
   return 1 + 4 * lg + (int)((lg >= 2 ? len >> (lg - 2) : len << (2 - lg)) & 3u);
 }
-// Counters cleared before every binning: list queues, tiles per bucket, and
-// the places handed out per bucket.
+// Counters of one render: list queues, tiles per bucket, and the places handed
+// out per bucket.
 constexpr int BIN_COUNTERS = LIST_CLASSES + 2 * LPT_BUCKETS;
+
+// The small state of a workspace that the kernels update. Everything but the
+// latched status is cleared at the start of a render, by one memset; the status
+// and the pair count go to the host in one copy.
+struct RenderHead {
+  int32_t status;                   // latched status bits
+  int32_t pad;
+  unsigned long long pairs;         // (Gaussian, tile) pairs of the render
+  uint32_t queue[2];                // work-queue heads of the forward / backward rasterisers
+  uint32_t counters[BIN_COUNTERS];
+};
+constexpr size_t HEAD_CLEARED = offsetof(RenderHead, pairs);  // the memset starts here
+
+// Arrays that a kernel clears for the kernels after it (before its own work and
+// without reading them), in place of a memset each.
+struct ZeroList {
+  void *p[3] = {nullptr, nullptr, nullptr};
+  int64_t words[3] = {0, 0, 0};  // 4-byte words
+  void add(void *q, int64_t n) {
+    for (int k = 0; k < 3; ++k)
+      if (!p[k]) { p[k] = q; words[k] = n; return; }
+  }
+  __device__ __forceinline__ void clear() const {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words[k];
+           i += (int64_t)gridDim.x * blockDim.x)
+        static_cast<uint32_t *>(p[k])[i] = 0u;
+  }
+};
+
+// Launches with programmatic stream serialization: the kernel's blocks may be
+// scheduled once every block of the kernel before it in the stream has started,
+// and wait in after_previous() until that kernel has completed and its writes
+// are visible. The launch gap of a render's seventeen or so short kernels then
+// overlaps the kernel before (4,096 Gaussians on 128^2: the render 137 -> 105 us
+// with the memsets and scans that went too; 100k on 512^2: 295 -> 253). Every
+// kernel launched this way begins with after_previous(). early = false launches
+// without: a persistent kernel with much shared memory must not start on SMs
+// still set up for the small share of the kernel before it, where too few of its
+// blocks fit and stay (the sorts of 69 M pairs: the step 5.31 -> 5.63 ms; the
+// backward preprocess at 2M Gaussians: 6.64 -> 6.72).
+template <class... KArgs, class... Args>
+inline cudaError_t launch_kernel(bool early, void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem,
+                                 cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
+template <class... KArgs, class... Args>
+inline cudaError_t launch_next(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                               Args... args) {
+  return launch_kernel(true, k, grid, block, smem, st, args...);
+}
+__device__ __forceinline__ void after_previous() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
 
 // Parameters shared by the rasterisers. q_lim = CONIC_SCALE q_max: the q cutoff
 // in the units of the records' scaled conic (see eval_pair).
@@ -169,11 +237,11 @@ inline void plan_binning(ViewTab *view, int32_t V, const ReqTab *req, int64_t to
     t.item_base = items;
     t.hist_base = slots;
     t.chunks = (int32_t)chunks;
-    t.band_w = (int32_t)bw;
-    t.band_h = (int32_t)bh;
-    t.bands_x = (int32_t)((tx + bw - 1) / bw);
+    t.band_w = (uint16_t)bw;
+    t.band_h = (uint16_t)bh;
+    t.bands_x = (uint16_t)((tx + bw - 1) / bw);
     t.lg_slices = 0;
-    t.vtile_base = t.tile_base;
+    t.vtile_base = (uint32_t)t.tile_base;
     items += chunks * bands;
     slots += chunks * bands * bw * bh;
     if (chunks > 0 && bw * bh > area) area = (int32_t)(bw * bh);
@@ -182,7 +250,7 @@ inline void plan_binning(ViewTab *view, int32_t V, const ReqTab *req, int64_t to
   view[V].hist_base = slots;
   view[V].chunks = 0;
   view[V].lg_slices = 0;
-  view[V].vtile_base = total_tiles;
+  view[V].vtile_base = (uint32_t)total_tiles;
   s.n_items = items;
   s.hist_slots = slots;
   s.hist_area = area;
@@ -221,14 +289,14 @@ inline void plan_slices(ViewTab *view, int32_t V, const ReqTab *req, int32_t til
     int lg = 0;
     if (n > SLICE_FROM * nt)
       while ((SLICE_TARGET << lg) * nt < n && (2 << lg) <= SLICE_MAX && (nt << (lg + 1)) <= BIN_HIST_MAX) ++lg;
-    t.lg_slices = lg;
+    t.lg_slices = (uint16_t)lg;
     // a tile's lists are neighbours in one warp of the offsets kernel
     vtiles = ((vtiles + (int64_t(1) << lg) - 1) >> lg) << lg;
-    t.vtile_base = vtiles;
+    t.vtile_base = (uint32_t)vtiles;
     vtiles += nt << lg;
     any |= lg > 0;
   }
-  view[V].vtile_base = vtiles;
+  view[V].vtile_base = (uint32_t)vtiles;
   s.total_vtiles = vtiles;
   s.sliced = any;
   if (!any) return;
@@ -378,27 +446,26 @@ struct ddgs_workspace {
   float4 *grad_h = nullptr;      // (dL/dh_0, dL/dh_1, dL/dh_2, 0)
   int64_t pix_cap = 0;
   bool last_per_pixel = false;   // mode of the last forward render
-  // scan
-  uint32_t *blk_total = nullptr;
   // pairs: (depth bits << 32 | Gaussian) placed by tile, then each tile's
   // Gaussians in depth order
   uint64_t *keys[2] = {nullptr, nullptr};  // [pairs]; keys[1] only for merging long lists
   uint32_t *vals = nullptr;      // [pairs] the tile lists the rasterisers read
   uint32_t *hist = nullptr;      // [hist_cap] per (binning block, tile) counts, then offsets
-  uint64_t *part = nullptr;      // [2 x tile blocks + 2] partial sums of the tile counts
+  uint64_t *part = nullptr;      // [part_capacity] sums of the list lengths, 1024 lists each
   uint64_t *lists = nullptr;     // [list_cap] tile lists to sort, by length class
-  uint32_t *list_count = nullptr;  // [BIN_COUNTERS]
   uint2 *ranges = nullptr;       // [tiles]
-  uint2 *vranges = nullptr;      // [vtile_cap] the lists' ranges where tiles are sliced by depth
-  uint32_t *splits = nullptr;    // [view_cap][SLICE_MAX] first depth of each slice
+  uint2 *vranges = nullptr;      // [vrange_cap] the lists' ranges where tiles are sliced by depth
+  int64_t vrange_cap = 0;
+  uint32_t *splits = nullptr;    // [split_cap][SLICE_MAX] first depth of each slice of a view
+  int64_t split_cap = 0;         // views
   uint32_t *order = nullptr;     // [tiles] work order of the persistent rasterisers
-  uint32_t *queue = nullptr;     // work-queue heads of the forward / backward rasterisers
   unsigned long long *req_time = nullptr;  // [1 + 2 R]: batch start, per-request fwd / bwd ends
   // scalars
-  uint64_t *d_pairs = nullptr;   // device pair count M
-  uint64_t *h_pairs = nullptr;   // pinned host mirror
-  int32_t *d_status = nullptr;
-  // request / view tables: device copies and a pinned host staging area
+  ddgs::RenderHead *head = nullptr;  // device
+  uint64_t *h_head = nullptr;    // pinned host mirror: the status word, the pair count, a staging word
+  // request / view tables (one device allocation with req_time) and
+  // a pinned host staging area
+  unsigned char *tab = nullptr;
   ddgs::ReqTab *d_req = nullptr;
   ddgs::ViewTab *d_view = nullptr;
   unsigned char *h_tab = nullptr;
@@ -419,7 +486,7 @@ namespace ddgs {
 
 // Kernel ids of the launch counter and profiler (api.cu).
 enum KernelId : int {
-  KID_PREPROCESS_FWD = 0, KID_SCAN_BLOCKS, KID_BIN_COUNT, KID_BIN_OFFSETS, KID_BIN_SCATTER,
+  KID_PREPROCESS_FWD = 0, KID_BIN_COUNT, KID_BIN_OFFSETS, KID_BIN_SCATTER,
   KID_BIN_SORT, KID_BIN_MERGE, KID_RASTER_FWD, KID_L1_LOSS, KID_RASTER_BWD,
   KID_PREPROCESS_BWD, KID_DEBUG, KID_TILE_ORDER, KID_RADS_MINMAX, KID_RADS_COUNT, KID_RADS_SCAN,
   KID_RADS_EMIT, KID_RADS_SELECT, KID_RADS_DRAW, KID_RADS_KNN, KID_COUNT
@@ -439,13 +506,13 @@ struct LaunchScope {
 
 // preprocess.cu
 void launch_preprocess_fwd(const ddgs_gaussians &g, const ddgs_views &v, const ddgs_config &c,
-                           const RenderShape &s, ddgs_workspace &ws, cudaStream_t st);
+                           const RenderShape &s, ddgs_workspace &ws, const ZeroList &zero,
+                           cudaStream_t st);
 void launch_preprocess_bwd(const ddgs_gaussians &g, const ddgs_views &v, const ddgs_config &c,
                            const RenderShape &s, ddgs_workspace &ws, const ddgs_grads &out,
                            cudaStream_t st);
 
 // bin.cu
-void launch_scan_blocks(int64_t nblk, ddgs_workspace &ws, cudaStream_t st);
 // Tile lists of the render: ranges[tile] and vals, from the records' tile
 // rectangles and depths (ws.rect); pair_bound > 0 once pairs exist.
 void launch_binning(const RenderShape &s, uint64_t pair_bound, ddgs_workspace &ws,
@@ -468,7 +535,7 @@ void launch_raster_fwd(const RenderShape &s, const RasterParams &p, ddgs_workspa
                        cudaStream_t st);
 void launch_raster_bwd(const RenderShape &s, const RasterParams &p, ddgs_workspace &ws,
                        const float *dL_dimage, const float *t_final, const uint32_t *n_last,
-                       const PixelRays *pr, cudaStream_t st);
+                       const PixelRays *pr, const ZeroList &zero, cudaStream_t st);
 
 int device_sms();  // streaming multiprocessors of the current device (raster.cu)
 cudaError_t prepare_raster_kernels();  // once per device, before any capture (raster.cu)

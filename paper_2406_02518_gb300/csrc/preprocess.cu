@@ -370,8 +370,9 @@ struct PreArgs {
   int vec;           // features in vectors of four (generic kernels)
   float4 *rec, *rec2;  // rec: two float4 per record
   uint4 *bin_info;  // (rect lo, rect hi, depth bits, tiles touched)
-  uint32_t *blk_total;
-  unsigned long long *t0;  // batch start (min over blocks of %globaltimer), or null
+  unsigned long long *pairs;  // pair count of the render, cleared
+  ZeroList zero;           // for the binning and the rasterisers
+  unsigned long long *t0;  // batch start (%globaltimer of the first block), or null
   int32_t *status;         // device status word: ST_NONFINITE is or-ed in
 };
 
@@ -431,14 +432,16 @@ __global__ void __launch_bounds__(PRE_THREADS, GEN ? 1 : 4) preprocess_fwd_kerne
   __shared__ uint32_t s_red[PRE_THREADS / 32];
   const int tid = threadIdx.x;
   const RenderShape &s = a.s;
+  after_previous();
+  a.zero.clear();
   const BlockReq br(s);
   const ReqTab &rq = br.rq;
   const bool live = br.live;
   const int64_t i = rq.g_off + br.l;  // index into the parameter arrays
-  if (tid == 0 && a.t0) {
+  if (tid == 0 && blockIdx.x == 0 && a.t0) {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    atomicMin(a.t0, t);
+    *a.t0 = t;
   }
   bool bad = false;  // a non-finite input seen by this thread
   for (int e = tid; e < Kr; e += PRE_THREADS) {
@@ -573,7 +576,7 @@ __global__ void __launch_bounds__(PRE_THREADS, GEN ? 1 : 4) preprocess_fwd_kerne
   }
   flag_nonfinite(bad, a.status);
   uint32_t bt = block_sum_u32(total, s_red);
-  if (tid == 0) a.blk_total[blockIdx.x] = bt;
+  if (tid == 0 && bt) atomicAdd(a.pairs, (unsigned long long)bt);
 }
 
 // ---------------------------------------------------------------------------
@@ -605,6 +608,7 @@ struct PreBwdArgs {
   float4 *grad_h;        // per_pixel: dL/dh summed over pixels (cleared the same way)
   ddgs_grads out;
   int want_param, want_basis, want_pose;
+  uint32_t *queue;       // the backward rasteriser's queue head: back to zero for the next pass
 };
 
 // Sum 16 per-lane values over the warp with 15 shuffles; returns the
@@ -659,6 +663,8 @@ __global__ void __launch_bounds__(PRE_THREADS, GEN ? 2 : 3) preprocess_bwd_kerne
   __shared__ float s_b[KS], s_B[KLS * KS], s_basis[GEN ? 1 : (1 + KLS) * KS];
   const int tid = threadIdx.x, lane = tid & 31;
   const RenderShape &s = a.s;
+  after_previous();
+  if (blockIdx.x == 0 && tid == 0) *a.queue = 0u;
   const BlockReq br(s);
   const ReqTab &rq = br.rq;
   const bool live = br.live;
@@ -1093,7 +1099,8 @@ __global__ void __launch_bounds__(PRE_THREADS, GEN ? 2 : 3) preprocess_bwd_kerne
 }  // namespace
 
 void launch_preprocess_fwd(const ddgs_gaussians &g, const ddgs_views &v, const ddgs_config &c,
-                           const RenderShape &s, ddgs_workspace &ws, cudaStream_t st) {
+                           const RenderShape &s, ddgs_workspace &ws, const ZeroList &zero,
+                           cudaStream_t st) {
   PreArgs a;
   a.means = g.means; a.log_scales = g.log_scales; a.quats = g.quats; a.logits = g.opacity_logits;
   a.feat_iso = g.feat_iso; a.feat_dir = g.feat_dir; a.feat_dir_bf16 = g.feat_dir_bf16;
@@ -1107,16 +1114,17 @@ void launch_preprocess_fwd(const ddgs_gaussians &g, const ddgs_views &v, const d
   a.s = s;
   a.rec = ws.rec; a.rec2 = ws.rec2;
   a.bin_info = reinterpret_cast<uint4 *>(ws.rect);
-  a.blk_total = ws.blk_total;
+  a.pairs = &ws.head->pairs;
+  a.zero = zero;
   a.t0 = ws.req_time;
-  a.status = ws.d_status;
+  a.status = &ws.head->status;
   if (s.n_blocks > 0) {
     LaunchScope ls(KID_PREPROCESS_FWD, st);
     const bool fast = a.K == K && a.L == 1 && !a.entangled && !a.per_pixel;
     auto k = fast ? preprocess_fwd_kernel<0>
                   : (a.L == 1 ? preprocess_fwd_kernel<1>
                               : (a.L == 2 ? preprocess_fwd_kernel<2> : preprocess_fwd_kernel<3>));
-    k<<<(unsigned)s.n_blocks, PRE_THREADS, 0, st>>>(a);
+    launch_next(k, (unsigned)s.n_blocks, PRE_THREADS, 0, st, a);
   }
 }
 
@@ -1136,6 +1144,7 @@ void launch_preprocess_bwd(const ddgs_gaussians &g, const ddgs_views &v, const d
   a.s = s;
   a.grad2d = ws.grad2d;
   a.grad_h = ws.grad_h;
+  a.queue = &ws.head->queue[1];
   a.out = out;
   a.want_param = (out.means || out.log_scales || out.quats || out.opacity_logits || out.feat_iso ||
                   out.feat_dir) ? 1 : 0;
@@ -1150,7 +1159,7 @@ void launch_preprocess_bwd(const ddgs_gaussians &g, const ddgs_views &v, const d
                    : (a.L == 2 ? preprocess_bwd_kernel<2> : preprocess_bwd_kernel<3>);
     else if (a.want_param || a.want_basis)
       k = preprocess_bwd_kernel<0>;
-    k<<<(unsigned)s.n_blocks, PRE_THREADS, 0, st>>>(a);
+    launch_kernel(false, k, (unsigned)s.n_blocks, PRE_THREADS, 0, st, a);
   }
 }
 

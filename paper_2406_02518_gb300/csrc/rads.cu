@@ -98,6 +98,7 @@ __device__ __forceinline__ Tv warp_incl_scan(Tv x) {
 // thread and packed 16-bit min / max, two voxels an instruction (512^3: 64 ->
 // 57 us, 4.7 TB/s).
 __global__ void __launch_bounds__(RT) rads_minmax_kernel(Vol v, RadsState *st) {
+  after_previous();
   const int64_t n8 = v.nvox / 8, stride = (int64_t)gridDim.x * blockDim.x;
   const uint4 *p = reinterpret_cast<const uint4 *>(v.hu);  // 8 voxels, little-endian
   uint32_t lo2 = 0x7fff7fffu, hi2 = 0x80008000u;
@@ -286,6 +287,7 @@ struct GroupCross {
 template <bool VEC>
 __global__ void __launch_bounds__(RT) rads_count_kernel(Vol vol, const RadsState *st, uint32_t *csub,
                                                         uint64_t *wsub) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const int mn = st->hu_min, lam2 = st->hu_min + st->hu_max;
   const uint32_t kc2 = above_carry(lam2);
@@ -341,6 +343,7 @@ __device__ __forceinline__ uint64_t block_excl_scan64(uint64_t x, uint64_t *s_w,
 __global__ void __launch_bounds__(SCAN_T) rads_scan_local_kernel(const uint32_t *a, const uint64_t *b, int per,
                                                                  int64_t n, uint64_t *ao, uint64_t *bo,
                                                                  uint64_t *tops) {
+  after_previous();
   __shared__ uint64_t s_w[32];
   const int64_t i = (int64_t)blockIdx.x * SCAN_T + threadIdx.x;
   uint64_t ta, tb;
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(SCAN_T) rads_scan_local_kernel(const uint32_t 
 // the grand totals.
 __global__ void __launch_bounds__(SCAN_T) rads_scan_add_kernel(const uint64_t *tops, int64_t n,
                                                                uint64_t *ao, uint64_t *bo) {
+  after_previous();
   __shared__ uint64_t s_a[32], s_b[32];
   const int t = threadIdx.x;  // gridDim.x <= SCAN_T
   const bool before = t < (int)blockIdx.x;
@@ -404,6 +408,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(RT) rads_emit_kernel(Vol vol, const RadsState *st,
                                                        const uint64_t *coff, const uint32_t *csub,
                                                        uint64_t seed, uint64_t *keys, uint64_t cap) {
+  after_previous();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t cs = lane < NSUB ? csub[(int64_t)blockIdx.x * NSUB + lane] : 0u;
   if (__shfl_sync(0xffffffffu, cs, wid) == 0) return;  // nothing for this warp to write
@@ -462,6 +467,7 @@ __global__ void __launch_bounds__(RT) rads_emit_kernel(Vol vol, const RadsState 
 constexpr int SEL_T = 1024;
 __global__ void __launch_bounds__(SEL_T) rads_select_pass_kernel(const uint64_t *keys, int64_t m,
                                                                  RadsState *st, int shift, int64_t rank0) {
+  after_previous();
   __shared__ uint32_t h[SEL_BINS];
   __shared__ uint32_t s_w[32];
   __shared__ bool s_last;
@@ -514,6 +520,7 @@ __global__ void __launch_bounds__(SEL_T) rads_select_pass_kernel(const uint64_t 
 // again from the list by the last block, one pass per bit.
 __global__ void __launch_bounds__(1024) rads_select_last_kernel(const uint64_t *keys, int64_t m,
                                                                 RadsState *st, int shift, uint64_t *cand) {
+  after_previous();
   __shared__ uint32_t s_n;
   __shared__ bool s_last;
   __shared__ uint64_t s_key[SEL_CAND];
@@ -575,6 +582,7 @@ __global__ void __launch_bounds__(1024) rads_select_last_kernel(const uint64_t *
 __global__ void __launch_bounds__(RT) rads_keep_count_kernel(const uint64_t *keys, int64_t m,
                                                              const RadsState *st, int all,
                                                              uint32_t *cnt) {
+  after_previous();
   __shared__ uint32_t s_c[RT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint64_t limit = all ? ~0ull : st->prefix;
@@ -605,6 +613,7 @@ __global__ void __launch_bounds__(RT) rads_keep_emit_kernel(Vol vol, const uint6
                                                             const uint64_t *off, int64_t n_out, float *means,
                                                             int64_t *kept_edges, KnnGrid grid,
                                                             uint32_t *cells, uint32_t *place) {
+  after_previous();
   __shared__ uint32_t s_c[RT / 32];
   __shared__ uint64_t s_b[RT / 32];
   uint64_t before = 0;
@@ -666,6 +675,7 @@ __global__ void __launch_bounds__(RT) rads_draw_kernel(Vol vol, const RadsState 
                                                        int64_t row0, float *means,
                                                        int64_t *draw_voxels, KnnGrid grid,
                                                        uint32_t *cells, uint32_t *place) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const int64_t j = (int64_t)blockIdx.x * (RT / 32) + (threadIdx.x >> 5);
   if (j >= n2) return;  // warp-uniform
@@ -767,6 +777,7 @@ __device__ __forceinline__ void insert4(float d2, float &b0, float &b1, float &b
 
 // Cell counts to cell starts (one block).
 __global__ void __launch_bounds__(1024) rads_knn_scan_kernel(uint32_t *cells, int n_cells) {  // cells: 16-byte aligned
+  after_previous();
   __shared__ uint32_t s_w[32];
   constexpr int PER = KNN_CELLS / 1024;
   static_assert(PER % 4 == 0, "cells in vectors of four");
@@ -804,6 +815,7 @@ __global__ void __launch_bounds__(1024) rads_knn_scan_kernel(uint32_t *cells, in
 
 __global__ void rads_knn_sort_kernel(const float *means, int64_t n, KnnGrid grid, const uint32_t *cells,
                                      const uint32_t *place, float4 *pts) {
+  after_previous();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float x = means[3 * i], y = means[3 * i + 1], z = means[3 * i + 2];
@@ -836,6 +848,7 @@ template <int LANES, bool FAR>
 __global__ void __launch_bounds__(256) rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid,
                                                        const uint32_t *cells, RadsState *st, uint32_t *far,
                                                        float *log_scales) {
+  after_previous();
   const int sub = threadIdx.x & (LANES - 1);
   const uint32_t group = LANES == 32 ? 0xffffffffu
                                      : ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) / LANES * LANES);
@@ -956,11 +969,11 @@ void scan_chunks(const uint32_t *a, const uint64_t *b, int per, int64_t n, uint6
   const int64_t nt = (n + SCAN_T - 1) / SCAN_T;
   {
     LaunchScope ls(KID_RADS_SCAN, st);
-    rads_scan_local_kernel<<<(unsigned)nt, SCAN_T, 0, st>>>(a, b, per, n, ao, bo, tops);
+    launch_next(rads_scan_local_kernel, (unsigned)nt, SCAN_T, 0, st, a, b, per, n, ao, bo, tops);
   }
   {
     LaunchScope ls(KID_RADS_SCAN, st);
-    rads_scan_add_kernel<<<(unsigned)nt, SCAN_T, 0, st>>>(tops, n, ao, bo);
+    launch_next(rads_scan_add_kernel, (unsigned)nt, SCAN_T, 0, st, tops, n, ao, bo);
   }
 }
 
@@ -1055,13 +1068,13 @@ extern "C" ddgs_status ddgs_rads(const ddgs_volume *vol, int32_t n1, int32_t n2,
   {
     LaunchScope ls(KID_RADS_MINMAX, st);
     const int64_t want = (nvox / 8 + RT - 1) / RT;
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 8 * device_sms()));
-    rads_minmax_kernel<<<grid, RT, 0, st>>>(v, state);
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 8 * device_sms()));
+    launch_next(rads_minmax_kernel, blocks, RT, 0, st, v, state);
   }
   {
     LaunchScope ls(KID_RADS_COUNT, st);
     auto k = vec ? rads_count_kernel<true> : rads_count_kernel<false>;
-    k<<<(unsigned)nblk, RT, 0, st>>>(v, state, csub, wsub);
+    launch_next(k, (unsigned)nblk, RT, 0, st, v, state, csub, wsub);
   }
   scan_chunks(csub, wsub, NSUB, nblk, coff, woff, tops, st);
   RCK(cudaGetLastError());
@@ -1085,7 +1098,7 @@ extern "C" ddgs_status ddgs_rads(const ddgs_volume *vol, int32_t n1, int32_t n2,
     {
       LaunchScope ls(KID_RADS_EMIT, st);
       auto k = vec ? rads_emit_kernel<true> : rads_emit_kernel<false>;
-      k<<<(unsigned)nblk, RT, 0, st>>>(v, state, coff, csub, seed, keys, (uint64_t)M);
+      launch_next(k, (unsigned)nblk, RT, 0, st, v, state, coff, csub, seed, keys, (uint64_t)M);
     }
     const int all = M <= n1 ? 1 : 0;
     if (!all) {
@@ -1094,21 +1107,21 @@ extern "C" ddgs_status ddgs_rads(const ddgs_volume *vol, int32_t n1, int32_t n2,
       do {
         shift -= SEL_BITS;
         LaunchScope ls(KID_RADS_SELECT, st);
-        rads_select_pass_kernel<<<hg, SEL_T, 0, st>>>(keys, M, state, shift,
-                                                      shift == 64 - SEL_BITS ? (int64_t)n1 - 1 : -1);
+        launch_next(rads_select_pass_kernel, hg, SEL_T, 0, st, keys, M, state, shift,
+                    shift == 64 - SEL_BITS ? (int64_t)n1 - 1 : (int64_t)-1);
       } while ((M >> (64 - shift)) > SEL_CAND / 2 && shift > SEL_BITS);
       LaunchScope ls(KID_RADS_SELECT, st);
-      rads_select_last_kernel<<<hg, SEL_T, 0, st>>>(keys, M, state, shift, cand);
+      launch_next(rads_select_last_kernel, hg, SEL_T, 0, st, keys, M, state, shift, cand);
     }
     {
       LaunchScope ls(KID_RADS_SELECT, st);
-      rads_keep_count_kernel<<<(unsigned)nkb, RT, 0, st>>>(keys, M, state, all, kcnt);
+      launch_next(rads_keep_count_kernel, (unsigned)nkb, RT, 0, st, keys, M, state, all, kcnt);
     }
     if (koff) scan_chunks(kcnt, nullptr, 1, nkb, koff, nullptr, tops, st);
     {
       LaunchScope ls(KID_RADS_SELECT, st);
-      rads_keep_emit_kernel<<<(unsigned)nkb, RT, 0, st>>>(v, keys, M, state, all, kcnt, koff, m1, means,
-                                                          kept_edges, grid, cells, place);
+      launch_next(rads_keep_emit_kernel, (unsigned)nkb, RT, 0, st, v, keys, M, state, all, kcnt, koff, m1, means,
+                  kept_edges, grid, cells, place);
     }
     RCK(cudaGetLastError());
   }
@@ -1116,29 +1129,29 @@ extern "C" ddgs_status ddgs_rads(const ddgs_volume *vol, int32_t n1, int32_t n2,
     LaunchScope ls(KID_RADS_DRAW, st);
     const unsigned g = (unsigned)((m2 + RT / 32 - 1) / (RT / 32));
     auto k = vec ? rads_draw_kernel<true> : rads_draw_kernel<false>;
-    k<<<g, RT, 0, st>>>(v, state, woff, wsub, nblk, (int32_t)m2, seed, m1, means, draw_voxels, grid, cells,
-                        place);
+    launch_next(k, g, RT, 0, st, v, state, woff, wsub, nblk, (int32_t)m2, seed, m1, means, draw_voxels, grid, cells,
+                place);
     RCK(cudaGetLastError());
   }
   const int64_t n = m1 + m2;
   if (n > 0) {
     {
       LaunchScope ls(KID_RADS_KNN, st);
-      rads_knn_scan_kernel<<<1, 1024, 0, st>>>(cells, n_cells);
+      launch_next(rads_knn_scan_kernel, 1u, 1024u, 0, st, cells, n_cells);
     }
     {
       LaunchScope ls(KID_RADS_KNN, st);
-      rads_knn_sort_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(means, n, grid, cells, place, pts);
+      launch_next(rads_knn_sort_kernel, (unsigned)((n + 255) / 256), 256u, 0, st, means, n, grid, cells, place, pts);
     }
     {
       LaunchScope ls(KID_RADS_KNN, st);
-      rads_knn_kernel<8, false><<<(unsigned)((n * 8 + 255) / 256), 256, 0, st>>>(pts, n, grid, cells, state,
-                                                                                far, log_scales);
+      launch_next(rads_knn_kernel<8, false>, (unsigned)((n * 8 + 255) / 256), 256u, 0, st, pts, n, grid, cells, state,
+                  far, log_scales);
     }
     {
       LaunchScope ls(KID_RADS_KNN, st);
       const unsigned g = (unsigned)std::min<int64_t>((n * 32 + 255) / 256, 8 * device_sms());
-      rads_knn_kernel<32, true><<<g, 256, 0, st>>>(pts, n, grid, cells, state, far, log_scales);
+      launch_next(rads_knn_kernel<32, true>, g, 256u, 0, st, pts, n, grid, cells, state, far, log_scales);
     }
     RCK(cudaGetLastError());
   }

@@ -65,6 +65,7 @@ struct RasterArgs {
   float4 *grad_h;            // dL/dh per record
   const float *world_to_cam, *detector;
   float *pose_grad;          // [V][12] or null
+  ZeroList zero;             // backward: the summed gradients that the next kernel adds to
 };
 
 __device__ __forceinline__ float sigmoid_r(float x) { return rcp_approx(1.f + __expf(-x)); }
@@ -363,6 +364,7 @@ __global__ void __launch_bounds__(WARPS * 32, 5) raster_fwd_lane_kernel(RasterAr
   const uint32_t nw = (uint32_t)(a.s.tile * a.s.tile / 32);
   __shared__ LaneFwdSmem sm[WARPS];
   const uint64_t n_items = (uint64_t)a.s.total_tiles * nw;
+  after_previous();
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
@@ -536,6 +538,8 @@ __global__ void __launch_bounds__(LANE_WARPS * 32, 3) raster_bwd_lane_kernel(Ras
   extern __shared__ __align__(16) unsigned char lane_smem[];
   LaneBwdSmem &sm = reinterpret_cast<LaneBwdSmem *>(lane_smem)[threadIdx.x >> 5];
   const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
+  after_previous();
+  a.zero.clear();
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
@@ -785,6 +789,7 @@ raster_fwd_pair_kernel(RasterArgs a) {
   constexpr int NW = T * T / 64;
   __shared__ PairFwdSmem<PIX> sm[PAIR_FWD_WARPS];
   const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
+  after_previous();
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
@@ -1059,6 +1064,8 @@ __global__ void __launch_bounds__(PairBwd<PIX>::WARPS * 32, PairBwd<PIX>::BLOCKS
   extern __shared__ __align__(16) unsigned char lane_smem[];
   PairBwdSmem<PIX> &sm = reinterpret_cast<PairBwdSmem<PIX> *>(lane_smem)[threadIdx.x >> 5];
   const uint64_t n_items = (uint64_t)a.s.total_tiles * NW;
+  after_previous();
+  a.zero.clear();
   for (;;) {
     const uint32_t item = warp_next_item(a.counter);
     if (item >= n_items) break;
@@ -1084,6 +1091,7 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(int64_t n_tiles, const
   static_assert(LPT_BUCKETS <= 1024, "one thread per bucket");
   const int t = threadIdx.x, lane = t & 31;
   const int64_t gt = (int64_t)blockIdx.x * 1024 + t;
+  after_previous();
   if (t < LPT_BUCKETS) s_cnt[t] = 0;
   // longer buckets come first: thread t has bucket LPT_BUCKETS - 1 - t
   const int b = LPT_BUCKETS - 1 - t;
@@ -1153,7 +1161,7 @@ void launch_items(Kernel k, int kid, const RasterArgs &a, int regions, int warps
   const int64_t need = (a.s.total_tiles * regions + warps - 1) / warps;
   const int64_t grid = std::min<int64_t>((int64_t)blocks_per_sm(k, warps * 32, dyn) * device_sms(), need);
   LaunchScope ls((KernelId)kid, st);
-  k<<<(unsigned)grid, warps * 32, dyn, st>>>(a);
+  launch_next(k, (unsigned)grid, (unsigned)warps * 32, dyn, st, a);
 }
 
 template <int T, bool PIX>
@@ -1201,8 +1209,8 @@ void bwd_dispatch(const RasterArgs &a, int tile, cudaStream_t st) {
 void launch_tile_order(const RenderShape &s, ddgs_workspace &ws, cudaStream_t st) {
   if (s.total_tiles <= 0) return;
   LaunchScope ls(KID_TILE_ORDER, st);
-  tile_order_kernel<<<(unsigned)((s.total_tiles + 1023) / 1024), 1024, 0, st>>>(
-      s.total_tiles, ws.ranges, ws.list_count + LIST_CLASSES, ws.order);
+  launch_next(tile_order_kernel, (unsigned)((s.total_tiles + 1023) / 1024), 1024u, 0, st, s.total_tiles, ws.ranges,
+              ws.head->counters + LIST_CLASSES, ws.order);
 }
 
 void launch_raster_fwd(const RenderShape &s, const RasterParams &p, ddgs_workspace &ws,
@@ -1218,9 +1226,8 @@ void launch_raster_fwd(const RenderShape &s, const RasterParams &p, ddgs_workspa
   a.t_final = t_final;
   a.n_last = n_last;
   a.order = ws.order;
-  a.counter = ws.queue;
+  a.counter = &ws.head->queue[0];
   a.req_end = ws.req_time ? ws.req_time + 1 : nullptr;
-  cudaMemsetAsync(ws.queue, 0, sizeof(uint32_t), st);
   if (pr) {  // per-pixel ray angles
     a.rec2 = ws.rec2;
     a.world_to_cam = pr->world_to_cam;
@@ -1233,7 +1240,7 @@ void launch_raster_fwd(const RenderShape &s, const RasterParams &p, ddgs_workspa
 
 void launch_raster_bwd(const RenderShape &s, const RasterParams &p, ddgs_workspace &ws,
                        const float *dL_dimage, const float *t_final, const uint32_t *n_last,
-                       const PixelRays *pr, cudaStream_t st) {
+                       const PixelRays *pr, const ZeroList &zero, cudaStream_t st) {
   RasterArgs a{};
   a.s = s;
   a.P = p;
@@ -1245,9 +1252,9 @@ void launch_raster_bwd(const RenderShape &s, const RasterParams &p, ddgs_workspa
   a.t_final_in = t_final;
   a.n_last_in = n_last;
   a.order = ws.order;
-  a.counter = ws.queue + 1;
+  a.counter = &ws.head->queue[1];
+  a.zero = zero;
   a.req_end = ws.req_time ? ws.req_time + 1 + s.R : nullptr;
-  cudaMemsetAsync(ws.queue + 1, 0, sizeof(uint32_t), st);
   if (pr) {  // per-pixel ray angles
     a.rec2 = ws.rec2;
     a.grad_h = ws.grad_h;

@@ -25,10 +25,9 @@ constexpr int64_t kMaxRecords = int64_t(1) << 18;  // views x Gaussians
 constexpr int64_t kMaxPairs = int64_t(1) << 20;    // (Gaussian, tile) pairs
 constexpr int64_t kMaxTiles = int64_t(1) << 16;    // views x tiles per view
 constexpr int64_t kMaxViews = 1024;                // views per call
-constexpr int64_t kMaxBlocks = kMaxRecords / ddgs::PRE_THREADS + 1;
 constexpr int64_t kSlotBudget = int64_t(1) << 18;  // tile counters of the binning blocks
 constexpr int64_t kMaxSlots = 2 * (kMaxTiles > kSlotBudget ? kMaxTiles : kSlotBudget);
-constexpr int64_t kMaxParts = 2 * ((kMaxTiles + 1023) / 1024) + 2;
+constexpr int64_t kMaxParts = (kMaxTiles + 1023) / 1024 + 1;
 constexpr int64_t kMaxListItems = ddgs::LIST_CLASSES * kMaxTiles + kMaxPairs / ddgs::BIN_LIST_LONG + 64;
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -38,20 +37,16 @@ constexpr size_t kOffRec1 = align256(kOffRec0 + kMaxRecords * sizeof(float4));
 constexpr size_t kOffInfo = align256(kOffRec1 + kMaxRecords * sizeof(float4));
 static_assert(kOffRec1 == kOffRec0 + kMaxRecords * sizeof(float4),
               "the records are one interleaved array over both regions");
-constexpr size_t kOffBlkTotal = align256(kOffInfo + kMaxRecords * sizeof(uint4));
-constexpr size_t kOffKeys0 = align256(kOffBlkTotal + kMaxBlocks * sizeof(uint32_t));
+constexpr size_t kOffKeys0 = align256(kOffInfo + kMaxRecords * sizeof(uint4));
 constexpr size_t kOffKeys1 = align256(kOffKeys0 + kMaxPairs * sizeof(uint64_t));
 constexpr size_t kOffVals = align256(kOffKeys1 + kMaxPairs * sizeof(uint64_t));
 constexpr size_t kOffHist = align256(kOffVals + kMaxPairs * sizeof(uint32_t));
 constexpr size_t kOffPart = align256(kOffHist + kMaxSlots * sizeof(uint32_t));
 constexpr size_t kOffLists = align256(kOffPart + kMaxParts * sizeof(uint64_t));
-constexpr size_t kOffListCount = align256(kOffLists + kMaxListItems * sizeof(uint64_t));
-constexpr size_t kOffRanges = align256(kOffListCount + ddgs::BIN_COUNTERS * sizeof(uint32_t));
-constexpr size_t kOffPairs = align256(kOffRanges + kMaxTiles * sizeof(uint2));
-constexpr size_t kOffStatus = align256(kOffPairs + sizeof(uint64_t));
-constexpr size_t kOffOrder = align256(kOffStatus + sizeof(int32_t));
-constexpr size_t kOffQueue = align256(kOffOrder + kMaxTiles * sizeof(uint32_t));
-constexpr size_t kOffReq = align256(kOffQueue + 2 * sizeof(uint32_t));
+constexpr size_t kOffRanges = align256(kOffLists + kMaxListItems * sizeof(uint64_t));
+constexpr size_t kOffHead = align256(kOffRanges + kMaxTiles * sizeof(uint2));
+constexpr size_t kOffOrder = align256(kOffHead + sizeof(ddgs::RenderHead));
+constexpr size_t kOffReq = align256(kOffOrder + kMaxTiles * sizeof(uint32_t));
 constexpr size_t kOffView = align256(kOffReq + 2 * sizeof(ddgs::ReqTab));
 constexpr size_t kScratchBytes = align256(kOffView + (kMaxViews + 1) * sizeof(ddgs::ViewTab));
 
@@ -162,24 +157,19 @@ extern "C" ddgs_status ddgs_render_static(const ddgs_gaussians *g, const ddgs_vi
   ws.rec_cap = kMaxRecords;
   ws.pair_cap = kMaxPairs;
   ws.tile_cap = kMaxTiles;
-  ws.blk_cap = kMaxBlocks;
   ws.hist_cap = kMaxSlots;
   ws.list_cap = kMaxListItems;
   ws.rec = reinterpret_cast<float4 *>(base + kOffRec0);  // rec0 and rec1 regions, contiguous
   ws.rect = reinterpret_cast<uint2 *>(base + kOffInfo);
-  ws.blk_total = reinterpret_cast<uint32_t *>(base + kOffBlkTotal);
   ws.keys[0] = reinterpret_cast<uint64_t *>(base + kOffKeys0);
   ws.keys[1] = reinterpret_cast<uint64_t *>(base + kOffKeys1);
   ws.vals = reinterpret_cast<uint32_t *>(base + kOffVals);
   ws.hist = reinterpret_cast<uint32_t *>(base + kOffHist);
   ws.part = reinterpret_cast<uint64_t *>(base + kOffPart);
   ws.lists = reinterpret_cast<uint64_t *>(base + kOffLists);
-  ws.list_count = reinterpret_cast<uint32_t *>(base + kOffListCount);
   ws.ranges = reinterpret_cast<uint2 *>(base + kOffRanges);
-  ws.d_pairs = reinterpret_cast<uint64_t *>(base + kOffPairs);
-  ws.d_status = reinterpret_cast<int32_t *>(base + kOffStatus);
+  ws.head = reinterpret_cast<ddgs::RenderHead *>(base + kOffHead);
   ws.order = reinterpret_cast<uint32_t *>(base + kOffOrder);
-  ws.queue = reinterpret_cast<uint32_t *>(base + kOffQueue);
   ws.req_time = nullptr;
   ddgs::ReqTab *d_req = reinterpret_cast<ddgs::ReqTab *>(base + kOffReq);
   ddgs::ViewTab *d_view = reinterpret_cast<ddgs::ViewTab *>(base + kOffView);
@@ -191,15 +181,14 @@ extern "C" ddgs_status ddgs_render_static(const ddgs_gaussians *g, const ddgs_vi
                             cudaMemcpyHostToDevice, cs));
 
   // counters left by the previous call start again from zero
-  CK_STATIC(cudaMemsetAsync(ws.d_status, 0, sizeof(int32_t), cs));
-  CK_STATIC(cudaMemsetAsync(ws.d_pairs, 0, sizeof(uint64_t), cs));
+  CK_STATIC(cudaMemsetAsync(ws.head, 0, sizeof(ddgs::RenderHead), cs));
+  CK_STATIC(cudaMemsetAsync(ws.part, 0, kMaxParts * sizeof(uint64_t), cs));
   uint64_t pairs = 0;
   if (s.records > 0) {
-    ddgs::launch_preprocess_fwd(*g, *v, *c, s, ws, cs);
-    ddgs::launch_scan_blocks(s.n_blocks, ws, cs);
+    ddgs::launch_preprocess_fwd(*g, *v, *c, s, ws, ddgs::ZeroList{}, cs);
     CK_STATIC(cudaGetLastError());
     // the pair count decides the sort's size: read it (no allocation)
-    CK_STATIC(cudaMemcpyAsync(&pairs, ws.d_pairs, sizeof(uint64_t), cudaMemcpyDeviceToHost, cs));
+    CK_STATIC(cudaMemcpyAsync(&pairs, &ws.head->pairs, sizeof(uint64_t), cudaMemcpyDeviceToHost, cs));
     CK_STATIC(cudaStreamSynchronize(cs));
     if (pairs > (uint64_t)kMaxPairs) return DDGS_ERR_CAPACITY;
   }

@@ -152,3 +152,27 @@ def test_picked_batches(shape, tile, per_pixel, ws):
     scene = dataclasses.replace(scene, per_pixel=per_pixel)
     views = _views([syn.pose_matrix(syn.rot_y(0.2), np.array([0.0, 0.1, 2.0]))], 4.0, 4.0 / W, H, W)
     _sampled_check(scene, views, syn.Settings(near_plane=0.2, tile=tile), ws, [0], 1500, 7, B.GRAD_FIELDS)
+
+
+def test_no_sync_render_without_room_for_slices(ws):
+    """A workspace sized by a synchronising render of many tiles takes a no-sync
+    render of a crowded view that fits its records, pairs and tiles, although
+    it was never reserved for depth slices; a synchronising render of the same
+    layout after it uses them again, and the backward of either is accepted."""
+    scene = _column(30000, 95, None, 0.3)
+    st = syn.Settings(near_plane=0.2, tile=8)
+    pose = [syn.pose_matrix(np.eye(3), np.array([0.0, 0.0, 2.0]))]
+    large, small = _views(pose, 4.0, 1.2 / 200, 200, 200), _views(pose, 4.0, 1.2 / 16, 16, 16)
+    cloud = B.cloud_from_arrays(scene)
+    w2 = B.Workspace()
+    B.render(cloud, B.views_from_arrays(large), B.config_from_settings(st), w2)
+    gv = B.views_from_arrays(small)
+    ref = oracle.bin32(scene, small, st)
+    for no_sync in (True, False, True):
+        cfg = B.config_from_settings(st, no_sync=no_sync)
+        img, tf, nl = B.render(cloud, gv, cfg, w2)
+        g = B.render_backward(cloud, gv, cfg, w2, torch.ones_like(img), tf, nl)
+        assert w2.sync_status() == 0
+        compare_binning(_bins(w2, scene, small, st), ref)
+        assert float(g["means"].abs().max()) > 0
+    w2.close()
