@@ -807,21 +807,33 @@ raster_fwd_pair_kernel(RasterArgs a) {
 // from sums over pairs: sum A = sum S, A x = S x, A y = S y + D, A x^2 = S x^2,
 // A x y = (S y + D) x, A y^2 = S y^2 + D (2 y + 1). With per-pixel rays the
 // table holds dL/dz of both pixels instead, for the sums of dL/dz and dL/dz Y.
+//
+// A pair adds few of a batch's 32 entries (4.4 in a regular view of 500k
+// Gaussians, 11.2 in a dense fit). With per-pixel rays, whose table is twice as
+// wide, a lane therefore keeps what it stores one after the other, PAIR_KEEP
+// entries at most: entry e of pair p is the popc of the pair's added entries
+// below e, and a longer walk is done in stretches, each with its own sums. So
+// sixteen warps fit per SM, not ten (200k Gaussians on 8 views of 256^2:
+// raster_bwd 347 -> 297 us; keeping 12 gives the same, 8 is 7 % slower). Without rays the [pair][entry] table stays: the
+// look-ups and the second set of atomics cost more than the warps give (64 views
+// of 256^2 2168 -> 2278 us, 100k Gaussians on one 512^2 view 88 -> 119).
+constexpr int PAIR_KEEP = 16;
 template <bool PIX>
 struct PairBwdSmem {
   PairSlot slot[33];  // entry 32: a sentinel that no pixel adds
   float4 z[PIX ? 33 : 1];   // (a, h_0, h_1, h_2)
   float4 y[PIX ? 64 : 1];   // Y_1 of the rays of the upper and of the lower pixels
+  uint32_t used[PIX ? 32 : 1];  // the entries that each pair added
   uint32_t id[32], cover[32], j[32];
-  float2 sd[32 * 32];  // [pair][entry ^ pair]: (S, D)
-  float2 dz[PIX ? 32 * 32 : 1];  // the same: dL/dz of the two pixels
-  float nb[PIX ? 1 : 32 * 32];   // the same: -sum of dL/dc
+  static constexpr int KEEP = PIX ? PAIR_KEEP : 32;  // a lane's entries in the tables
+  float2 sd[KEEP * 32];  // [pair][entry ^ pair], with rays [stored][pair]: (S, D)
+  float2 dz[PIX ? KEEP * 32 : 1];  // the same: dL/dz of the two pixels
+  float nb[PIX ? 1 : KEEP * 32];   // the same: -sum of dL/dc
 };
-// Blocks of four warps and 57 KB, sixteen warps per SM; with per-pixel rays
-// blocks of two and 40 KB, ten warps.
+// Blocks of four warps and 57 KB (49 KB with rays), sixteen warps per SM.
 template <bool PIX>
 struct PairBwd {
-  static constexpr int WARPS = PIX ? 2 : 4, BLOCKS = PIX ? 5 : 4;
+  static constexpr int WARPS = 4, BLOCKS = 4;
   static constexpr size_t SMEM = WARPS * sizeof(PairBwdSmem<PIX>);
 };
 
@@ -893,134 +905,143 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
     }
     const int skip = min(skip0, skip1);
     mine &= skip >= 32 ? 0u : (0xffffffffu << skip);
-    uint32_t used = 0;
-    const int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mine));
+    int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mine));
     uint32_t bn = mine & (0u - mine);  // the next entry's bit (0 past the last)
     int kn = __popc(bn - 1u);          // its index: 32, the sentinel, past the last
     PairSlot sn = sm.slot[kn];
-    for (int t = 0; t < trips; ++t) {
-      const int k = kn;
-      const uint32_t bit = bn;
-      const PairSlot s = sn;
-      mine ^= bit;
-      bn = mine & (0u - mine);
-      kn = __popc(bn - 1u);
-      sn = sm.slot[kn];
-      const float2 qf = unpack2(pair_q(s, px, npy));
-      const uint64_t G = pack2(exp2_approx(qf.x), exp2_approx(qf.y));
-      const float2 ng = unpack2(mul2(s.c.x, G));
-      const float ns0 = fmaxf(namax, ng.x), ns1 = fmaxf(namax, ng.y);  // -sigma
-      const bool ok0 = !(qf.x < a.P.q_lim || qf.x > 0.f) && ns0 <= namin && k >= skip0;
-      const bool ok1 = !(qf.y < a.P.q_lim || qf.y > 0.f) && ns1 <= namin && k >= skip1;
-      const uint64_t ns = pack2(ns0, ns1);
-      // 1 / (1 - sigma) with sigma <= alpha_max < 1: the fast reciprocal's
-      // relative error (~1 ulp) is far inside the gradient tolerance
-      const float2 om = unpack2(add2(one, ns));
-      const uint64_t inv = pack2(rcp_approx(om.x), rcp_approx(om.y));
-      const uint64_t Tn = mul2(Tr, inv);
-      uint64_t col = s.c.y;
-      float4 z;
-      float2 cf;
-      if (PIX) {
-        z = sm.z[k];
-        cf = make_float2(pixel_colour(ray0, z), pixel_colour(ray1, z));
-        col = pack2(cf.x, cf.y);
-      }
-      const uint64_t gdC = fma2(col, Tn, mul2(nS, inv));  // g dC/dsigma
-      const uint64_t nsT = mul2(ns, Tn);                  // -g dC/dc
-      const uint64_t nSn = fma2(col, nsT, nS);
-      const float2 gA = unpack2(mul2(gdC, G)), nb = unpack2(nsT);
-      const float A0 = ok0 && !(ng.x < namax) ? gA.x : 0.f, A1 = ok1 && !(ng.y < namax) ? gA.y : 0.f;
-      const float b0_ = ok0 ? nb.x : 0.f, b1_ = ok1 ? nb.y : 0.f;
-      if (ok0 || ok1) {
-        const int at = lane * 32 + (k ^ lane);
-        sm.sd[at] = make_float2(A0 + A1, A1);
+    while (trips > 0) {
+      uint32_t used = 0;
+      int next = lane;  // with rays: where the next stored entry goes
+      for (int t = PIX ? min(trips, sm.KEEP) : trips; t > 0; --t) {
+        const int k = kn;
+        const uint32_t bit = bn;
+        const PairSlot s = sn;
+        mine ^= bit;
+        bn = mine & (0u - mine);
+        kn = __popc(bn - 1u);
+        sn = sm.slot[kn];
+        const float2 qf = unpack2(pair_q(s, px, npy));
+        const uint64_t G = pack2(exp2_approx(qf.x), exp2_approx(qf.y));
+        const float2 ng = unpack2(mul2(s.c.x, G));
+        const float ns0 = fmaxf(namax, ng.x), ns1 = fmaxf(namax, ng.y);  // -sigma
+        const bool ok0 = !(qf.x < a.P.q_lim || qf.x > 0.f) && ns0 <= namin && k >= skip0;
+        const bool ok1 = !(qf.y < a.P.q_lim || qf.y > 0.f) && ns1 <= namin && k >= skip1;
+        const uint64_t ns = pack2(ns0, ns1);
+        // 1 / (1 - sigma) with sigma <= alpha_max < 1: the fast reciprocal's
+        // relative error (~1 ulp) is far inside the gradient tolerance
+        const float2 om = unpack2(add2(one, ns));
+        const uint64_t inv = pack2(rcp_approx(om.x), rcp_approx(om.y));
+        const uint64_t Tn = mul2(Tr, inv);
+        uint64_t col = s.c.y;
+        float4 z;
+        float2 cf;
         if (PIX) {
-          const float z0 = -b0_ * cf.x * (1.f - cf.x), z1 = -b1_ * cf.y * (1.f - cf.y);
-          sm.dz[at] = make_float2(ok0 ? z0 : 0.f, ok1 ? z1 : 0.f);
-          if (ok0) {
-            gY0[0] = fmaf(z0, z.y, gY0[0]);
-            gY0[1] = fmaf(z0, z.z, gY0[1]);
-            gY0[2] = fmaf(z0, z.w, gY0[2]);
-          }
-          if (ok1) {
-            gY1[0] = fmaf(z1, z.y, gY1[0]);
-            gY1[1] = fmaf(z1, z.z, gY1[1]);
-            gY1[2] = fmaf(z1, z.w, gY1[2]);
-          }
-        } else {
-          sm.nb[at] = b0_ + b1_;
+          z = sm.z[k];
+          cf = make_float2(pixel_colour(ray0, z), pixel_colour(ray1, z));
+          col = pack2(cf.x, cf.y);
         }
-        used |= bit;
+        const uint64_t gdC = fma2(col, Tn, mul2(nS, inv));  // g dC/dsigma
+        const uint64_t nsT = mul2(ns, Tn);                  // -g dC/dc
+        const uint64_t nSn = fma2(col, nsT, nS);
+        const float2 gA = unpack2(mul2(gdC, G)), nb = unpack2(nsT);
+        const float A0 = ok0 && !(ng.x < namax) ? gA.x : 0.f, A1 = ok1 && !(ng.y < namax) ? gA.y : 0.f;
+        const float b0_ = ok0 ? nb.x : 0.f, b1_ = ok1 ? nb.y : 0.f;
+        if (ok0 || ok1) {
+          const int at = PIX ? next : lane * 32 + (k ^ lane);
+          sm.sd[at] = make_float2(A0 + A1, A1);
+          if (PIX) {
+            const float z0 = -b0_ * cf.x * (1.f - cf.x), z1 = -b1_ * cf.y * (1.f - cf.y);
+            sm.dz[at] = make_float2(ok0 ? z0 : 0.f, ok1 ? z1 : 0.f);
+            if (ok0) {
+              gY0[0] = fmaf(z0, z.y, gY0[0]);
+              gY0[1] = fmaf(z0, z.z, gY0[1]);
+              gY0[2] = fmaf(z0, z.w, gY0[2]);
+            }
+            if (ok1) {
+              gY1[0] = fmaf(z1, z.y, gY1[0]);
+              gY1[1] = fmaf(z1, z.z, gY1[1]);
+              gY1[2] = fmaf(z1, z.w, gY1[2]);
+            }
+          } else {
+            sm.nb[at] = b0_ + b1_;
+          }
+          used |= bit;
+          next += 32;
+        }
+        const float2 To = unpack2(Tr), Tv = unpack2(Tn), So = unpack2(nS), Sv = unpack2(nSn);
+        Tr = pack2(ok0 ? Tv.x : To.x, ok1 ? Tv.y : To.y);
+        nS = pack2(ok0 ? Sv.x : So.x, ok1 ? Sv.y : So.y);
       }
-      const float2 To = unpack2(Tr), Tv = unpack2(Tn), So = unpack2(nS), Sv = unpack2(nSn);
-      Tr = pack2(ok0 ? Tv.x : To.x, ok1 ? Tv.y : To.y);
-      nS = pack2(ok0 ? Sv.x : So.x, ok1 ? Sv.y : So.y);
+      trips = PIX ? trips - sm.KEEP : 0;
+      if (PIX) sm.used[lane] = used;
+      __syncwarp();
+      uint32_t pm = transpose32(used);  // lane e: the pairs that added entry e
+      const uint32_t below = (1u << lane) - 1u;
+      if (pm) {
+        uint64_t sd = 0, sdx = 0, sdy = 0;  // sums of (S, D), (S, D) x, (S, D) y
+        float sxx = 0.f, sxy = 0.f, syy = 0.f, sb = 0.f, sh[3] = {0.f, 0.f, 0.f};
+        do {  // two pairs per trip: half the loop overhead, two loads in flight
+          const int p = __ffs(pm) - 1;
+          pm &= pm - 1;
+          const bool two = pm != 0;
+          const int q = two ? __ffs(pm) - 1 : p;
+          pm &= pm - 1;
+          const int ip = PIX ? p + 32 * __popc(sm.used[p] & below) : p * 32 + (lane ^ p);
+          const int iq = PIX ? q + 32 * __popc(sm.used[q] & below) : q * 32 + (lane ^ q);
+          const float2 u = sm.sd[ip];
+          float2 v = sm.sd[iq];
+          if (!two) v = make_float2(0.f, 0.f);
+          if (PIX) {
+            const float2 zu = sm.dz[ip];
+            float2 zv = sm.dz[iq];
+            if (!two) zv = make_float2(0.f, 0.f);
+            sb += (zu.x + zu.y) + (zv.x + zv.y);
+            const float4 yu0 = sm.y[p], yu1 = sm.y[32 + p], yv0 = sm.y[q], yv1 = sm.y[32 + q];
+            sh[0] = fmaf(zu.x, yu0.x, fmaf(zu.y, yu1.x, fmaf(zv.x, yv0.x, fmaf(zv.y, yv1.x, sh[0]))));
+            sh[1] = fmaf(zu.x, yu0.y, fmaf(zu.y, yu1.y, fmaf(zv.x, yv0.y, fmaf(zv.y, yv1.y, sh[1]))));
+            sh[2] = fmaf(zu.x, yu0.z, fmaf(zu.y, yu1.z, fmaf(zv.x, yv0.z, fmaf(zv.y, yv1.z, sh[2]))));
+          } else {
+            const float ub = sm.nb[ip], vb = sm.nb[iq];
+            sb -= ub + (two ? vb : 0.f);
+          }
+          const float x = (float)(p & 7), y = (float)((p >> 2) & 6);
+          const float x2 = (float)(q & 7), y2 = (float)((q >> 2) & 6);
+          const uint64_t up = pack2(u.x, u.y), vp = pack2(v.x, v.y);
+          sd = add2(sd, add2(up, vp));
+          sdx = fma2(up, pack2(x, x), fma2(vp, pack2(x2, x2), sdx));
+          sdy = fma2(up, pack2(y, y), fma2(vp, pack2(y2, y2), sdy));
+          const float ax = u.x * x, ax2 = v.x * x2;
+          sxx = fmaf(ax, x, fmaf(ax2, x2, sxx));
+          sxy = fmaf(ax, y, fmaf(ax2, y2, sxy));
+          syy = fmaf(u.x * y, y, fmaf(v.x * y2, y2, syy));
+        } while (pm);
+        const float2 fd = unpack2(sd), fx = unpack2(sdx), fy = unpack2(sdy);
+        const float s0 = fd.x, s1 = fx.x, s2 = fy.x + fd.y, s4 = sxy + fx.y,
+                    s5 = syy + fmaf(2.f, fy.y, fd.y);
+        const PairSlot sl = sm.slot[lane];
+        const float2 ua = unpack2(sl.g.x);
+        const float ca = ua.y, cb2 = unpack2(sl.k.x).x, cc = unpack2(sl.k.y).x;
+        const float u = ua.x - cx, v = unpack2(sl.g.y).x - cy;  // mean relative to pixel (0, 0)
+        // sums over the entry's pixels of A dx, A dy, A dx^2, A dx dy, A dy^2
+        const float sdx1 = fmaf(u, s0, -s1), sdy1 = fmaf(v, s0, -s2);
+        const float gxx = fmaf(u, fmaf(u, s0, -2.f * s1), sxx);
+        const float gxy = fmaf(u, fmaf(v, s0, -s2), fmaf(-v, s1, s4));
+        const float gyy = fmaf(v, fmaf(v, s0, -2.f * s2), s5);
+        const float hq = 0.5f * unpack2(sl.c.x).x;  // dL/dq = -alpha A / 2
+        // dq/du = 2 (a dx + b dy), dq/dv = 2 (b dx + c dy), dq/db = 2 dx dy;
+        // the record holds (a', 2b', c') = CONIC_SCALE (a, 2b, c)
+        const float hk = hq * INV_CONIC_SCALE;
+        const float gx = hk * sdx1, gy = hk * sdy1;
+        const float du = fmaf(2.f * ca, gx, cb2 * gy);
+        const float dv = fmaf(cb2, gx, 2.f * cc * gy);
+        const int64_t r = rg.rec_base + sm.id[lane];
+        atomicAdd(a.grad2d + 2 * r, make_float4(du, dv, hq * gxx, 2.f * hq * gxy));
+        atomicAdd(a.grad2d + 2 * r + 1, make_float4(hq * gyy, s0, sb, 0.f));
+        if (PIX) atomicAdd(a.grad_h + r, make_float4(sh[0], sh[1], sh[2], 0.f));
+      }
+      __syncwarp();  // the sums of the next stretch use the same table
     }
-    __syncwarp();
-    uint32_t pm = transpose32(used);  // lane e: the pairs that added entry e
-    if (pm) {
-      uint64_t sd = 0, sdx = 0, sdy = 0;  // sums of (S, D), (S, D) x, (S, D) y
-      float sxx = 0.f, sxy = 0.f, syy = 0.f, sb = 0.f, sh[3] = {0.f, 0.f, 0.f};
-      do {  // two pairs per trip: half the loop overhead, two loads in flight
-        const int p = __ffs(pm) - 1;
-        pm &= pm - 1;
-        const bool two = pm != 0;
-        const int q = two ? __ffs(pm) - 1 : p;
-        pm &= pm - 1;
-        const int ip = p * 32 + (lane ^ p), iq = q * 32 + (lane ^ q);
-        const float2 u = sm.sd[ip];
-        float2 v = sm.sd[iq];
-        if (!two) v = make_float2(0.f, 0.f);
-        if (PIX) {
-          const float2 zu = sm.dz[ip];
-          float2 zv = sm.dz[iq];
-          if (!two) zv = make_float2(0.f, 0.f);
-          sb += (zu.x + zu.y) + (zv.x + zv.y);
-          const float4 yu0 = sm.y[p], yu1 = sm.y[32 + p], yv0 = sm.y[q], yv1 = sm.y[32 + q];
-          sh[0] = fmaf(zu.x, yu0.x, fmaf(zu.y, yu1.x, fmaf(zv.x, yv0.x, fmaf(zv.y, yv1.x, sh[0]))));
-          sh[1] = fmaf(zu.x, yu0.y, fmaf(zu.y, yu1.y, fmaf(zv.x, yv0.y, fmaf(zv.y, yv1.y, sh[1]))));
-          sh[2] = fmaf(zu.x, yu0.z, fmaf(zu.y, yu1.z, fmaf(zv.x, yv0.z, fmaf(zv.y, yv1.z, sh[2]))));
-        } else {
-          const float ub = sm.nb[ip], vb = sm.nb[iq];
-          sb -= ub + (two ? vb : 0.f);
-        }
-        const float x = (float)(p & 7), y = (float)((p >> 2) & 6);
-        const float x2 = (float)(q & 7), y2 = (float)((q >> 2) & 6);
-        const uint64_t up = pack2(u.x, u.y), vp = pack2(v.x, v.y);
-        sd = add2(sd, add2(up, vp));
-        sdx = fma2(up, pack2(x, x), fma2(vp, pack2(x2, x2), sdx));
-        sdy = fma2(up, pack2(y, y), fma2(vp, pack2(y2, y2), sdy));
-        const float ax = u.x * x, ax2 = v.x * x2;
-        sxx = fmaf(ax, x, fmaf(ax2, x2, sxx));
-        sxy = fmaf(ax, y, fmaf(ax2, y2, sxy));
-        syy = fmaf(u.x * y, y, fmaf(v.x * y2, y2, syy));
-      } while (pm);
-      const float2 fd = unpack2(sd), fx = unpack2(sdx), fy = unpack2(sdy);
-      const float s0 = fd.x, s1 = fx.x, s2 = fy.x + fd.y, s4 = sxy + fx.y,
-                  s5 = syy + fmaf(2.f, fy.y, fd.y);
-      const PairSlot sl = sm.slot[lane];
-      const float2 ua = unpack2(sl.g.x);
-      const float ca = ua.y, cb2 = unpack2(sl.k.x).x, cc = unpack2(sl.k.y).x;
-      const float u = ua.x - cx, v = unpack2(sl.g.y).x - cy;  // mean relative to pixel (0, 0)
-      // sums over the entry's pixels of A dx, A dy, A dx^2, A dx dy, A dy^2
-      const float sdx1 = fmaf(u, s0, -s1), sdy1 = fmaf(v, s0, -s2);
-      const float gxx = fmaf(u, fmaf(u, s0, -2.f * s1), sxx);
-      const float gxy = fmaf(u, fmaf(v, s0, -s2), fmaf(-v, s1, s4));
-      const float gyy = fmaf(v, fmaf(v, s0, -2.f * s2), s5);
-      const float hq = 0.5f * unpack2(sl.c.x).x;  // dL/dq = -alpha A / 2
-      // dq/du = 2 (a dx + b dy), dq/dv = 2 (b dx + c dy), dq/db = 2 dx dy;
-      // the record holds (a', 2b', c') = CONIC_SCALE (a, 2b, c)
-      const float hk = hq * INV_CONIC_SCALE;
-      const float gx = hk * sdx1, gy = hk * sdy1;
-      const float du = fmaf(2.f * ca, gx, cb2 * gy);
-      const float dv = fmaf(cb2, gx, 2.f * cc * gy);
-      const int64_t r = rg.rec_base + sm.id[lane];
-      atomicAdd(a.grad2d + 2 * r, make_float4(du, dv, hq * gxx, 2.f * hq * gxy));
-      atomicAdd(a.grad2d + 2 * r + 1, make_float4(hq * gyy, s0, sb, 0.f));
-      if (PIX) atomicAdd(a.grad_h + r, make_float4(sh[0], sh[1], sh[2], 0.f));
-    }
-    __syncwarp();  // the slice is rewritten by the next batch
+    __syncwarp();  // the slice is rewritten by the next batch, also after one without a trip
   }
   if (PIX && a.pose_grad) {
     // Y_1(d / |d|), d = W^T rc: dL/dW[r][c] = rc[r] dL/dd[c], summed over the warp

@@ -154,6 +154,18 @@ def test_picked_batches(shape, tile, per_pixel, ws):
     _sampled_check(scene, views, syn.Settings(near_plane=0.2, tile=tile), ws, [0], 1500, 7, B.GRAD_FIELDS)
 
 
+@pytest.mark.parametrize("n,tile", [(16, 8), (17, 8), (32, 16), (33, 8), (70, 16)])
+def test_pixel_ray_stretches(n, tile, ws):
+    """Faint Gaussians over the whole detector: every pair of pixels adds every
+    entry of a batch, so the backward's walks fill one stretch of its table
+    (16 entries), one and an entry, and both halves of whole batches."""
+    scene = syn.uniform_cloud(n, seed=51 + n, dir_frac=0.5, dir_std=1.0, extent=0.2, log_scale_range=(-0.9, -0.5),
+                              alpha_range=(0.02, 0.06))
+    scene = dataclasses.replace(scene, per_pixel=True)
+    st = syn.Settings(near_plane=0.2, tile=tile)
+    _check(scene, _two_views(45, 60, 1.0 / 56), st, B.cloud_from_arrays(scene), B.config_from_settings(st), ws)
+
+
 def test_no_sync_render_without_room_for_slices(ws):
     """A workspace sized by a synchronising render of many tiles takes a no-sync
     render of a crowded view that fits its records, pairs and tiles, although
