@@ -561,8 +561,7 @@ constexpr size_t LANE_BWD_SMEM = LANE_WARPS * sizeof(LaneBwdSmem);
 // took 14.5 (CPU count over the benchmark's lists). The two pixels' chains are
 // independent, and most of their arithmetic is done on binary32 pairs (add,
 // mul and fma .rn.f32x2: one instruction, each half rounded as the scalar
-// operation is), with the entry's values staged in duplicate so that they load
-// as pairs. sigma is carried negated (max(-alpha_max, -alpha G)), which turns
+// operation is). sigma is carried negated (max(-alpha_max, -alpha G)), which turns
 // 1 - sigma and T (1 - sigma) into an add and an fma; every decision is the
 // one eval_pair takes, bit for bit.
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
@@ -591,25 +590,41 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 
-// A staged entry: (u, a'), (v, v) | (2b', 2b'), (c', c') | (-alpha, -alpha),
-// (colour, colour).
-struct PairSlot {
-  ulonglong2 g, k, c;
+// A staged entry: mean, a', 2b', c', -alpha, colour. Shared memory bounds the
+// pair kernels (its pipe was busy 84 % forward, 86 % backward when each lane
+// loaded 48 bytes a trip, the values duplicated for the packed units), so an
+// entry is two 16-byte pieces, in arrays of their own so that eight consecutive
+// entries meet no bank conflict; duplicating in registers is cheaper (raster_fwd
+// and raster_bwd at 64 views of 256^2: 1068 -> 1008 and 2168 -> 2078 us, 2M
+// Gaussians on 8 of 1024^2 1418 -> 1310 and 2950 -> 2834). Smaller pieces take
+// fewer cycles of the pipe but more instructions (8 bytes 1018 and 2082, 4 bytes
+// 1020 and 2106), and so does q' in scalar operations (1044 and 2105).
+struct PairEntry {
+  float u, v, a, b, c, na, col;
+};
+template <int N>
+struct PairSlots {
+  float4 f[2][N];
+  __device__ __forceinline__ void put(int k, const PairEntry &e) {
+    f[0][k] = make_float4(e.u, e.v, e.a, e.b);
+    f[1][k] = make_float4(e.c, e.na, e.col, 0.f);
+  }
+  __device__ __forceinline__ PairEntry get(int k) const {
+    const float4 x = f[0][k], y = f[1][k];
+    return {x.x, x.y, x.z, x.w, y.x, y.y, y.z};
+  }
 };
 
-__device__ __forceinline__ void stage_pair(PairSlot &s, float4 r0, float4 r1) {
-  s.g = make_ulonglong2(pack2(r0.x, r0.z), pack2(r0.y, r0.y));
-  s.k = make_ulonglong2(pack2(r0.w, r0.w), pack2(r1.x, r1.x));
-  s.c = make_ulonglong2(pack2(-r1.y, -r1.y), pack2(r1.z, r1.z));
+__device__ __forceinline__ PairEntry pair_entry(float4 r0, float4 r1) {
+  return {r0.x, r0.y, r0.z, r0.w, r1.x, -r1.y, r1.z};
 }
 
 // q' at both pixels (eval_pair's operations); npy = (-py, -(py + 1)).
-__device__ __forceinline__ uint64_t pair_q(const PairSlot &s, float px, uint64_t npy) {
-  const float2 ua = unpack2(s.g.x);
-  const float dx = __fsub_rn(ua.x, px), m = __fmul_rn(ua.y, dx);
-  const uint64_t dy = add2(s.g.y, npy);
-  const uint64_t t = fma2(s.k.x, dy, pack2(m, m));
-  return fma2(mul2(s.k.y, dy), dy, mul2(pack2(dx, dx), t));
+__device__ __forceinline__ uint64_t pair_q(const PairEntry &s, float px, uint64_t npy) {
+  const float dx = __fsub_rn(s.u, px), m = __fmul_rn(s.a, dx);
+  const uint64_t dy = add2(pack2(s.v, s.v), npy);
+  const uint64_t t = fma2(pack2(s.b, s.b), dy, pack2(m, m));
+  return fma2(mul2(pack2(s.c, s.c), dy), dy, mul2(pack2(dx, dx), t));
 }
 
 // The 8 x 8 pixel region of a work item.
@@ -658,7 +673,7 @@ __device__ __forceinline__ uint32_t pair_cover(float4 b, float cx, float cy) {
 // below t_min), and from the start outside the image.
 template <bool PIX>
 struct PairFwdSmem {
-  PairSlot slot[64];
+  PairSlots<64> slot;
   uint32_t j[64], cover[32];
   float4 z[PIX ? 64 : 1];  // (a, h_0, h_1, h_2)
 };
@@ -700,7 +715,7 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
       pk.fill(st, sm.cover, sm.j + half,
               [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
               [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) {
-                stage_pair(sm.slot[half + k], r0, r1);
+                sm.slot.put(half + k, pair_entry(r0, r1));
                 if (PIX) sm.z[half + k] = a.rec2[rg.rec_base + id];
               },
               cover);
@@ -720,11 +735,10 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
       if (m == 0) continue;
       const uint32_t k = (uint32_t)__ffs(m) - 1u;
       m &= m - 1;
-      const PairSlot &s = sm.slot[slot + k];
+      const PairEntry s = sm.slot.get(slot + k);
       const uint64_t q = pair_q(s, px, npy);
       const float2 qf = unpack2(q);
-      const uint64_t naG = mul2(s.c.x, pack2(exp2_approx(qf.x), exp2_approx(qf.y)));
-      const float2 ng = unpack2(naG);
+      const float2 ng = make_float2(__fmul_rn(s.na, exp2_approx(qf.x)), __fmul_rn(s.na, exp2_approx(qf.y)));
       const float ns0 = fmaxf(namax, ng.x), ns1 = fmaxf(namax, ng.y);  // -sigma
       const bool ok0 = !(qf.x < a.P.q_lim || qf.x > 0.f) && ns0 <= namin;
       const bool ok1 = !(qf.y < a.P.q_lim || qf.y > 0.f) && ns1 <= namin;
@@ -732,12 +746,12 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
       const float2 Tn = unpack2(fma2(Tr, ns, Tr));  // T (1 - sigma)
       const bool st0 = ok0 && Tn.x < a.P.t_min, st1 = ok1 && Tn.y < a.P.t_min;
       // C - (colour (-sigma)) T
-      uint64_t col = s.c.y;
+      float2 col = make_float2(s.col, s.col);
       if (PIX && (ok0 || ok1)) {
         const float4 z = sm.z[slot + k];
-        col = pack2(pixel_colour(ray0, z), pixel_colour(ray1, z));
+        col = make_float2(pixel_colour(ray0, z), pixel_colour(ray1, z));
       }
-      const float2 w = unpack2(mul2(col, ns));
+      const float2 w = make_float2(__fmul_rn(col.x, ns0), __fmul_rn(col.y, ns1));
       const uint32_t p = PICK ? slot + k + 1u : pos + k;
       if (ok0 && !st0) {
         C0 = fmaf(-w.x, T0, C0);
@@ -820,7 +834,7 @@ raster_fwd_pair_kernel(RasterArgs a) {
 constexpr int PAIR_KEEP = 16;
 template <bool PIX>
 struct PairBwdSmem {
-  PairSlot slot[33];  // entry 32: a sentinel that no pixel adds
+  PairSlots<33> slot;  // entry 32: a sentinel that no pixel adds
   float4 z[PIX ? 33 : 1];   // (a, h_0, h_1, h_2)
   float4 y[PIX ? 64 : 1];   // Y_1 of the rays of the upper and of the lower pixels
   uint32_t used[PIX ? 32 : 1];  // the entries that each pair added
@@ -870,9 +884,7 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
     sm.y[32 + lane] = make_float4(ray1.Y[0], ray1.Y[1], ray1.Y[2], 0.f);
   }
   if (lane == 0) {  // q' = -inf at every pixel
-    sm.slot[32].g = make_ulonglong2(pack2(3.0e38f, -1.f), pack2(3.0e38f, 3.0e38f));
-    sm.slot[32].k = make_ulonglong2(pack2(0.f, 0.f), pack2(-1.f, -1.f));
-    sm.slot[32].c = make_ulonglong2(0ull, 0ull);
+    sm.slot.put(32, {3.0e38f, 3.0e38f, -1.f, 0.f, -1.f, 0.f, 0.f});
     if (PIX) sm.z[32] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   const uint32_t max_last = __reduce_max_sync(0xffffffffu, max(last0, last1));
@@ -888,7 +900,7 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
         st, sm.cover, sm.j,
         [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
         [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) {
-          stage_pair(sm.slot[k], r0, r1);
+          sm.slot.put(k, pair_entry(r0, r1));
           sm.id[k] = id;
           if (PIX) sm.z[k] = a.rec2[rg.rec_base + id];
         },
@@ -908,21 +920,22 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
     int trips = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(mine));
     uint32_t bn = mine & (0u - mine);  // the next entry's bit (0 past the last)
     int kn = __popc(bn - 1u);          // its index: 32, the sentinel, past the last
-    PairSlot sn = sm.slot[kn];
+    PairEntry sn = sm.slot.get(kn);
     while (trips > 0) {
       uint32_t used = 0;
       int next = lane;  // with rays: where the next stored entry goes
       for (int t = PIX ? min(trips, sm.KEEP) : trips; t > 0; --t) {
         const int k = kn;
         const uint32_t bit = bn;
-        const PairSlot s = sn;
+        const PairEntry s = sn;
         mine ^= bit;
         bn = mine & (0u - mine);
         kn = __popc(bn - 1u);
-        sn = sm.slot[kn];
+        sn = sm.slot.get(kn);
         const float2 qf = unpack2(pair_q(s, px, npy));
-        const uint64_t G = pack2(exp2_approx(qf.x), exp2_approx(qf.y));
-        const float2 ng = unpack2(mul2(s.c.x, G));
+        const float g0 = exp2_approx(qf.x), g1 = exp2_approx(qf.y);
+        const uint64_t G = pack2(g0, g1);
+        const float2 ng = make_float2(__fmul_rn(s.na, g0), __fmul_rn(s.na, g1));
         const float ns0 = fmaxf(namax, ng.x), ns1 = fmaxf(namax, ng.y);  // -sigma
         const bool ok0 = !(qf.x < a.P.q_lim || qf.x > 0.f) && ns0 <= namin && k >= skip0;
         const bool ok1 = !(qf.y < a.P.q_lim || qf.y > 0.f) && ns1 <= namin && k >= skip1;
@@ -932,7 +945,7 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
         const float2 om = unpack2(add2(one, ns));
         const uint64_t inv = pack2(rcp_approx(om.x), rcp_approx(om.y));
         const uint64_t Tn = mul2(Tr, inv);
-        uint64_t col = s.c.y;
+        uint64_t col = pack2(s.col, s.col);
         float4 z;
         float2 cf;
         if (PIX) {
@@ -1018,16 +1031,15 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
         const float2 fd = unpack2(sd), fx = unpack2(sdx), fy = unpack2(sdy);
         const float s0 = fd.x, s1 = fx.x, s2 = fy.x + fd.y, s4 = sxy + fx.y,
                     s5 = syy + fmaf(2.f, fy.y, fd.y);
-        const PairSlot sl = sm.slot[lane];
-        const float2 ua = unpack2(sl.g.x);
-        const float ca = ua.y, cb2 = unpack2(sl.k.x).x, cc = unpack2(sl.k.y).x;
-        const float u = ua.x - cx, v = unpack2(sl.g.y).x - cy;  // mean relative to pixel (0, 0)
+        const PairEntry sl = sm.slot.get(lane);
+        const float ca = sl.a, cb2 = sl.b, cc = sl.c;
+        const float u = sl.u - cx, v = sl.v - cy;  // mean relative to pixel (0, 0)
         // sums over the entry's pixels of A dx, A dy, A dx^2, A dx dy, A dy^2
         const float sdx1 = fmaf(u, s0, -s1), sdy1 = fmaf(v, s0, -s2);
         const float gxx = fmaf(u, fmaf(u, s0, -2.f * s1), sxx);
         const float gxy = fmaf(u, fmaf(v, s0, -s2), fmaf(-v, s1, s4));
         const float gyy = fmaf(v, fmaf(v, s0, -2.f * s2), s5);
-        const float hq = 0.5f * unpack2(sl.c.x).x;  // dL/dq = -alpha A / 2
+        const float hq = 0.5f * sl.na;  // dL/dq = -alpha A / 2
         // dq/du = 2 (a dx + b dy), dq/dv = 2 (b dx + c dy), dq/db = 2 dx dy;
         // the record holds (a', 2b', c') = CONIC_SCALE (a, 2b, c)
         const float hk = hq * INV_CONIC_SCALE;
