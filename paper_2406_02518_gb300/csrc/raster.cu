@@ -844,7 +844,7 @@ struct PairBwdSmem {
   float2 dz[PIX ? KEEP * 32 : 1];  // the same: dL/dz of the two pixels
   float nb[PIX ? 1 : KEEP * 32];   // the same: -sum of dL/dc
 };
-// Blocks of four warps and 57 KB (49 KB with rays), sixteen warps per SM.
+// Blocks of four warps and 55 KB (45 KB with rays), sixteen warps per SM.
 template <bool PIX>
 struct PairBwd {
   static constexpr int WARPS = 4, BLOCKS = 4;
