@@ -1048,8 +1048,10 @@ __global__ void __launch_bounds__(PRE_THREADS, GEN ? 2 : 3) preprocess_bwd_kerne
 #pragma unroll
         for (int g = 0; g < PRE_THREADS; g += 32) {
           const float w = s_w[m * PRE_THREADS + g + lane];
+          if (w != 0.f) {  // a Gaussian of weight zero adds nothing, whatever its features are
 #pragma unroll
-          for (int j = 0; j < 8; ++j) acc[j] = fmaf(w, s_f[j * PRE_THREADS + g + lane], acc[j]);
+            for (int j = 0; j < 8; ++j) acc[j] = fmaf(w, s_f[j * PRE_THREADS + g + lane], acc[j]);
+          }
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
