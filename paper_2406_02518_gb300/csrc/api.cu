@@ -202,6 +202,7 @@ ddgs_status upload_layout(ddgs_workspace *ws, Layout &L, bool no_sync, cudaStrea
     CK(cudaMemcpyAsync(ws->d_req, hr, L.req.size() * sizeof(ddgs::ReqTab), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(ws->d_view, hv, L.view.size() * sizeof(ddgs::ViewTab), cudaMemcpyHostToDevice, st));
     ws->last_hash = L.hash;
+    ws->graph_hash = 0;
   }
   L.shape.req = ws->d_req;
   L.shape.view = ws->d_view;
@@ -272,15 +273,16 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
   return ensure_lists(ws);
 }
 
-// A no-sync render on a workspace without room for its depth slices (made for
-// another layout, never reserved for this one) is binned without them.
-void drop_slices(const ddgs_workspace *ws, Layout &L) {
-  ddgs::RenderShape &s = L.shape;
-  if (!s.sliced || (s.total_vtiles <= ws->vtile_cap && s.total_vtiles <= ws->vrange_cap &&
-                    s.V <= ws->split_cap && s.hist_slots <= ws->hist_cap &&
-                    ddgs::list_capacity(s.total_vtiles, ws->pair_cap) <= ws->list_cap))
-    return;
-  ddgs::plan_binning(L.view.data(), L.V, L.req.data(), s.total_tiles, s.tile, s);
+// Whether the workspace has room for the depth slices of a plan.
+bool slices_fit(const ddgs_workspace *ws, const ddgs::RenderShape &s) {
+  return s.total_vtiles <= ws->vtile_cap && s.total_vtiles <= ws->vrange_cap && s.V <= ws->split_cap &&
+         s.hist_slots <= ws->hist_cap && ddgs::list_capacity(s.total_vtiles, ws->pair_cap) <= ws->list_cap;
+}
+
+// The layout without its depth slices: a no-sync render on a workspace that has
+// no room for them (made for another layout, never reserved for this one).
+void drop_slices(Layout &L) {
+  ddgs::plan_binning(L.view.data(), L.V, L.req.data(), L.shape.total_tiles, L.shape.tile, L.shape);
   L.hash ^= kUnsliced;
 }
 
@@ -503,8 +505,13 @@ ddgs_status render_common(const ddgs_gaussians &g, const ddgs_views &v, const dd
   if (!on_workspace_device(ws)) return DDGS_ERR_INVALID_ARG;
   ddgs_status st;
   ddgs::RenderShape &s = L.shape;
+  // A graph that captured a render without slices replays its kernels on the
+  // tables and buffers of that plan, so later renders of the layout keep it, also
+  // where they could grow the workspace, until another layout's tables take its place.
+  const bool kept = s.sliced && ws->graph_hash == (L.hash ^ kUnsliced);
+  const bool unsliced = kept || (s.sliced && c->no_sync && !slices_fit(ws, s));
+  if (unsliced) drop_slices(L);
   if (c->no_sync) {
-    drop_slices(ws, L);
     if (s.records > ws->rec_cap || s.n_blocks > ws->blk_cap || s.total_tiles > ws->tile_cap ||
         s.total_vtiles > ws->vtile_cap || s.hist_slots > ws->hist_cap || !ws->keys[0] ||
         ddgs::list_capacity(s.total_vtiles, ws->pair_cap) > ws->list_cap)
@@ -520,6 +527,7 @@ ddgs_status render_common(const ddgs_gaussians &g, const ddgs_views &v, const dd
     }
   }
   if ((st = upload_layout(ws, L, c->no_sync != 0, s_))) return st;
+  if (unsliced && !kept && capturing(s_)) ws->graph_hash = L.hash;
   ws->have_render = false;
   CK(cudaMemsetAsync(reinterpret_cast<unsigned char *>(ws->head) + ddgs::HEAD_CLEARED, 0,
                      sizeof(ddgs::RenderHead) - ddgs::HEAD_CLEARED, s_));

@@ -474,7 +474,9 @@ struct ddgs_workspace {
   ddgs::RenderShape shape{};
   bool have_render = false;
   uint64_t pair_bound = 0;       // grid bound used for the pair kernels
-  int64_t last_hash = 0;         // identifies the batch layout of the last render
+  uint64_t last_hash = 0;        // identifies the batch layout of the last render
+  uint64_t graph_hash = 0;       // = last_hash where a stream capture recorded that layout without
+                                 // the depth slices it would have (0 otherwise)
   // initialisation (rads.cu): crossing keys and per-chunk scratch
   uint64_t *rads_keys = nullptr;
   int64_t rads_key_cap = 0;

@@ -1,0 +1,70 @@
+"""What outlives one call on a workspace: a captured graph's tables and buffers."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2406_02518_gb300 import binding as B
+from paper_2406_02518_gb300 import synthetic as syn
+from _parity import compare_binning
+from test_gpu_kernel_paths import _column
+from test_gpu_parity import _bins, _lib, _views  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+POSE = [syn.pose_matrix(np.eye(3), np.array([0.0, 0.0, 2.0]))]
+
+
+def _offset_launches(run):
+    """Launches of the binning's offset kernels in one render: three where tiles
+    are cut into depth slices, two without."""
+    B.profiler_collect()
+    B.profiler_enable(True)
+    try:
+        run()
+        torch.cuda.synchronize()
+        return B.profiler_collect()["bin_offsets"][1]
+    finally:
+        B.profiler_enable(False)
+
+
+@pytest.mark.parametrize("captured", [True, False])
+def test_graph_of_a_render_without_slices(captured):
+    """A workspace without room for a crowded view's depth slices: the no-sync
+    render goes without. Once a graph has captured it, a synchronising render of
+    the same layout must leave the graph's tables and buffers as they are; where
+    none has, it makes room and uses the slices."""
+    scene = _column(30000, 95, None, 0.3)
+    st = syn.Settings(near_plane=0.2, tile=8)
+    large, small = _views(POSE, 4.0, 1.2 / 200, 200, 200), _views(POSE, 4.0, 1.2 / 16, 16, 16)
+    cloud, gv = B.cloud_from_arrays(scene), B.views_from_arrays(small)
+    cfg, cfg_ns = B.config_from_settings(st), B.config_from_settings(st, no_sync=True)
+    ref = oracle.bin32(scene, small, st)
+    w = B.Workspace()
+    B.render(cloud, B.views_from_arrays(large), cfg, w)
+    out = B.render(cloud, gv, cfg_ns, w)
+    dL, grads = torch.ones_like(out[0]), {}
+    B.render_backward(cloud, gv, cfg_ns, w, dL, out[1], out[2])
+    torch.cuda.synchronize()
+    want = [t.clone() for t in out]
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            B.render(cloud, gv, cfg_ns, w, out=out)
+            grads = B.render_backward(cloud, gv, cfg_ns, w, dL, out[1], out[2])
+    assert _offset_launches(lambda: B.render(cloud, gv, cfg, w)) == (2 if captured else 3)
+    if captured:
+        for _ in range(2):
+            for t in out:
+                t.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(out, want))
+            assert float(grads["means"].abs().max()) > 0
+        assert w.sync_status() == 0
+        compare_binning(_bins(w, scene, small, st), ref)
+        # another layout ends the graph's claim: the slices come back
+        B.render(cloud, B.views_from_arrays(large), cfg, w)
+        assert _offset_launches(lambda: B.render(cloud, gv, cfg, w)) == 3
+    compare_binning(_bins(w, scene, small, st), ref)
+    w.close()
