@@ -458,8 +458,8 @@ ddgs_status ddgs_workspace_create(ddgs_workspace **out) {
 ddgs_status ddgs_workspace_destroy(ddgs_workspace *ws) {
   if (!ws) return DDGS_OK;
   void *dev[] = {ws->rec, ws->rect, ws->tiles_touched, ws->grad2d, ws->keys[0], ws->keys[1], ws->vals,
-                 ws->hist, ws->part, ws->lists, ws->ranges, ws->vranges, ws->head, ws->tab, ws->order,
-                 ws->rec2, ws->grad_h, ws->rads_keys, ws->rads_buf};
+                 ws->hist, ws->part, ws->lists, ws->ranges, ws->vranges, ws->splits, ws->head, ws->tab,
+                 ws->order, ws->rec2, ws->grad_h, ws->rads_keys, ws->rads_buf};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (ws->h_head) cudaFreeHost(ws->h_head);

@@ -1,4 +1,5 @@
-"""What outlives one call on a workspace: a captured graph's tables and buffers."""
+"""What outlives one call on a workspace: its memory, and a captured graph's tables
+and buffers."""
 import numpy as np
 import pytest
 import torch
@@ -68,3 +69,24 @@ def test_graph_of_a_render_without_slices(captured):
         assert _offset_launches(lambda: B.render(cloud, gv, cfg, w)) == 3
     compare_binning(_bins(w, scene, small, st), ref)
     w.close()
+
+
+def test_workspaces_return_their_memory():
+    """Create, reserve, render a crowded view and destroy, many times: the free
+    memory comes back. (Reserving for 4 M records makes room for depth slices.)"""
+    scene = _column(2100, 98, None, 0.3)
+    st = syn.Settings(near_plane=0.2, tile=8)
+    cloud, gv = B.cloud_from_arrays(scene), B.views_from_arrays(_views(POSE, 4.0, 1.2 / 8, 8, 8))
+    cfg = B.config_from_settings(st)
+
+    def cycles(n):
+        for _ in range(n):
+            w = B.Workspace()
+            w.reserve(4_000_000, 1 << 20, 4096)
+            B.render(cloud, gv, cfg, w)
+            w.close()
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    before = cycles(4)
+    assert before - cycles(60) < 8 << 20
