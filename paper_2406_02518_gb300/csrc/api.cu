@@ -1,7 +1,6 @@
 // api.cu -- the C ABI: argument checks, workspace management and the order of
 // the kernels of a render and of its backward pass.
 #include <algorithm>
-#include <climits>
 #include <atomic>
 #include <cstdio>
 #include <cstring>
@@ -246,16 +245,11 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
     if ((st = grow(ws->order, ws->tile_cap, cap, sizeof(uint32_t)))) return st;
     ws->tile_cap = cap;
   }
-  if (s.sliced && (s.V > ws->split_cap || !ws->splits)) {
-    const int64_t cap = s.V + s.V / 4 + 64;
-    ddgs_status st = grow(ws->splits, ws->split_cap, cap * ddgs::SLICE_MAX, sizeof(uint32_t));
-    if (st) return st;
-    ws->split_cap = cap;
-  }
   if (s.sliced && (s.total_vtiles > ws->vrange_cap || !ws->vranges)) {
     int64_t cap = s.total_vtiles + s.total_vtiles / 4 + 64;
-    ddgs_status st = grow(ws->vranges, ws->vrange_cap, cap, sizeof(uint2));
-    if (st) return st;
+    ddgs_status st;
+    if ((st = grow(ws->splits, ws->vrange_cap, cap, sizeof(uint32_t)))) return st;
+    if ((st = grow(ws->vranges, ws->vrange_cap, cap, sizeof(uint2)))) return st;
     ws->vrange_cap = cap;
   }
   if (s.total_vtiles > ws->vtile_cap || !ws->part) {  // the part sums follow the lists
@@ -275,8 +269,8 @@ ddgs_status ensure_records(ddgs_workspace *ws, const ddgs::RenderShape &s) {
 
 // Whether the workspace has room for the depth slices of a plan.
 bool slices_fit(const ddgs_workspace *ws, const ddgs::RenderShape &s) {
-  return s.total_vtiles <= ws->vtile_cap && s.total_vtiles <= ws->vrange_cap && s.V <= ws->split_cap &&
-         s.hist_slots <= ws->hist_cap && ddgs::list_capacity(s.total_vtiles, ws->pair_cap) <= ws->list_cap;
+  return s.total_vtiles <= ws->vtile_cap && s.total_vtiles <= ws->vrange_cap && s.hist_slots <= ws->hist_cap &&
+         ddgs::list_capacity(s.total_vtiles, ws->pair_cap) <= ws->list_cap;
 }
 
 // The layout without its depth slices: a no-sync render on a workspace that has
@@ -480,8 +474,7 @@ ddgs_status ddgs_workspace_reserve(ddgs_workspace *ws, int64_t records, int64_t 
   s.n_blocks = records / ddgs::PRE_THREADS + 4096;
   s.total_tiles = tiles;
   s.total_vtiles = ddgs::vtile_bound(tiles, records);
-  s.sliced = 1;  // a sliced view has more than SLICE_FROM records
-  s.V = (int32_t)std::min<int64_t>(records / ddgs::SLICE_FROM + 1, INT32_MAX / 2);
+  s.sliced = 1;
   s.hist_slots = ddgs::hist_slot_bound(s.total_vtiles);
   ddgs_status st = ensure_records(ws, s);
   if (st) return st;

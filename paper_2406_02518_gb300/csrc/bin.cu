@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(SLICE_SAMPLE) bin_slices_kernel(RenderShape s,
       __syncthreads();
     }
   const int slices = 1 << vt.lg_slices;
-  if (t > 0 && t < slices) splits[(int64_t)blockIdx.x * SLICE_MAX + t] = s_d[(int64_t)t * m / slices];
+  if (t > 0 && t < slices) splits[vt.vtile_base + t] = s_d[(int64_t)t * m / slices];
 }
 
 // The part of a record's tile rectangle inside the block's band; false when
@@ -130,11 +130,10 @@ __global__ void __launch_bounds__(BIN_THREADS, 8) bin_count_kernel(RenderShape s
   extern __shared__ uint32_t s_cnt[];
   __shared__ uint32_t s_sp[SLICE_MAX];
   after_previous();
-  const int v = find_item_view(s.view, s.V, blockIdx.x);
-  const ViewTab vt = s.view[v];
+  const ViewTab vt = s.view[find_item_view(s.view, s.V, blockIdx.x)];
   const BinItem it = bin_item(s, vt, blockIdx.x);
   const int area = (it.bw * it.bh) << (SLICED ? it.lg : 0);
-  if (SLICED && it.lg && threadIdx.x < (1 << it.lg)) s_sp[threadIdx.x] = splits[(int64_t)v * SLICE_MAX + threadIdx.x];
+  if (SLICED && it.lg && threadIdx.x < (1 << it.lg)) s_sp[threadIdx.x] = splits[vt.vtile_base + threadIdx.x];
   for (int p = threadIdx.x; p < area; p += BIN_THREADS) s_cnt[p] = 0;
   __syncthreads();
   for (int64_t l0 = it.l0 + threadIdx.x; l0 < it.l1; l0 += BIN_LOADS * BIN_THREADS) {
@@ -437,12 +436,11 @@ __global__ void __launch_bounds__(SCAT_THREADS, 3) bin_scatter_kernel(RenderShap
   after_previous();
   __shared__ uint32_t s_wsum[SCAT_THREADS / 32];
   __shared__ uint32_t s_sp[SLICE_MAX];
-  const int v = find_item_view(s.view, s.V, blockIdx.x);
-  const ViewTab vt = s.view[v];
+  const ViewTab vt = s.view[find_item_view(s.view, s.V, blockIdx.x)];
   const BinItem it = bin_item(s, vt, blockIdx.x);
   const int tiles_y = (vt.H + s.tile - 1) / s.tile;
   const int lg = SLICED ? it.lg : 0, area = (it.bw * it.bh) << lg;
-  if (SLICED && it.lg && threadIdx.x < (1 << it.lg)) s_sp[threadIdx.x] = splits[(int64_t)v * SLICE_MAX + threadIdx.x];
+  if (SLICED && it.lg && threadIdx.x < (1 << it.lg)) s_sp[threadIdx.x] = splits[vt.vtile_base + threadIdx.x];
   constexpr int STAGE = scatter_stage(DIRECT, SLICED);
   uint64_t *s_key = reinterpret_cast<uint64_t *>(scat_smem);  // [STAGE] staged pairs
   uint32_t *s_dst = reinterpret_cast<uint32_t *>(s_key + STAGE);  // [STAGE] their places

@@ -259,9 +259,10 @@ inline void plan_binning(ViewTab *view, int32_t V, const ReqTab *req, int64_t to
 }
 
 // Lists any layout of this many tiles and records can have once plan_slices
-// has cut them: a view that is cut has fewer than 2 n / SLICE_TARGET of them.
+// has cut them: a view that is cut has fewer than 2 n / SLICE_TARGET of them, and
+// the gap that aligns its first list is shorter than a tile's lists.
 inline int64_t vtile_bound(int64_t tiles, int64_t records) {
-  return tiles + 2 * records / SLICE_TARGET;
+  return tiles + 4 * records / SLICE_TARGET;
 }
 
 // Depth slices (host, after plan_binning). A view with more than SLICE_FROM
@@ -456,8 +457,7 @@ struct ddgs_workspace {
   uint2 *ranges = nullptr;       // [tiles]
   uint2 *vranges = nullptr;      // [vrange_cap] the lists' ranges where tiles are sliced by depth
   int64_t vrange_cap = 0;
-  uint32_t *splits = nullptr;    // [split_cap][SLICE_MAX] first depth of each slice of a view
-  int64_t split_cap = 0;         // views
+  uint32_t *splits = nullptr;    // [vrange_cap] first depth of each slice of a view, from its first list on
   uint32_t *order = nullptr;     // [tiles] work order of the persistent rasterisers
   unsigned long long *req_time = nullptr;  // [1 + 2 R]: batch start, per-request fwd / bwd ends
   // scalars

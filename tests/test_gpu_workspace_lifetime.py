@@ -90,3 +90,29 @@ def test_workspaces_return_their_memory():
 
     before = cycles(4)
     assert before - cycles(60) < 8 << 20
+
+
+def test_reserved_batch_of_many_views_keeps_its_slices():
+    """A batch on a workspace reserved by its records, pairs and tiles: the depth
+    slices of its crowded views have room, however many other views there are and
+    however the lists of one view are aligned after another's."""
+    st = syn.Settings(near_plane=0.2, tile=8)
+    tiny, crowded = _column(1, 96, None, 0.1), _column(8193, 97, None, 0.3)
+    view = B.views_from_arrays(_views(POSE, 4.0, 1.2 / 8, 8, 8))  # one tile
+    for clouds in ([tiny, crowded] * 40, [tiny] * 400 + [crowded]):
+        batch = B.Batch([B.cloud_from_arrays(c) for c in clouds], [view] * len(clouds))
+        w = B.Workspace()
+        img, _, _ = B.render_batched(batch, B.config_from_settings(st), w)
+        pairs = w.pairs()
+        w.close()
+        w = B.Workspace()
+        w.reserve(int(batch.n.sum()), pairs, len(clouds))
+        out = [None]
+
+        def run():
+            out[0] = B.render_batched(batch, B.config_from_settings(st, no_sync=True), w)
+
+        assert _offset_launches(run) == 3
+        assert w.sync_status() == 0
+        assert torch.equal(out[0][0], img)
+        w.close()
