@@ -36,6 +36,8 @@ constexpr int SEL_BITS = 11, SEL_BINS = 1 << SEL_BITS;  // radix select: digits 
 constexpr int SEL_CAND = 4096;  // keys that the select's last step orders in one block
 constexpr int KNN_CELLS = 32768;  // most cells of the neighbour search's grid
 constexpr int KNN_NEAR = 1;     // rings of cells searched by eight lanes a point, then by a warp
+constexpr int KNN_T = 256;      // threads per block of the search
+constexpr int CROWD_TILE = 1024;  // points staged at a time for those in crowded cells
 
 // Output number i + 1 of SplitMix64 (Steele, Lea and Flood, OOPSLA 2014)
 // seeded with `seed`: the state after i + 1 golden-gamma steps, finalised.
@@ -53,6 +55,7 @@ struct RadsState {
   uint32_t done;     // blocks finished in the current select pass
   uint32_t n_cand;   // keys sharing the prefix found so far
   uint32_t n_far;    // points whose neighbours lie beyond KNN_NEAR cells
+  uint32_t n_crowd;  // points in crowded cells
   uint32_t hist[SEL_BINS];
 };
 
@@ -833,34 +836,114 @@ __device__ __forceinline__ void merge4(float b[4], const float o[4]) {
   b[3] = fmaxf(h0, h1);
 }
 
+// Squared distance of two points: the brute-force search's, bit for bit.
+__device__ __forceinline__ float distance2(const float4 &c, const float4 &q) {
+  const float dx = c.x - q.x, dy = c.y - q.y, dz = c.z - q.z;
+  return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+}
+
+// The 4 smallest over a group of LANES lanes, each with its own list.
+template <int LANES>
+__device__ __forceinline__ void merge_group(uint32_t group, float m[4]) {
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) {
+    float t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = __shfl_xor_sync(group, m[k], o);
+    merge4(m, t);
+  }
+}
+template <int LANES>
+__device__ __forceinline__ uint32_t lane_group() {
+  return LANES == 32 ? 0xffffffffu : ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) / LANES * LANES);
+}
+
+// log s of sorted point q: b[0] is the point itself (0), the others are the
+// nearest other points.
+__device__ __forceinline__ void knn_scale(const float4 &q, int64_t n, const float b[4], float *log_scales) {
+  const int kk = n - 1 < 3 ? (int)(n - 1) : 3;
+  float m = 0.f;
+  if (kk >= 1) m += b[1];
+  if (kk >= 2) m += b[2];
+  if (kk >= 3) m += b[3];
+  m = kk > 0 ? m / (float)kk : 0.f;
+  const float ls = 0.5f * logf(fmaxf(m, 1e-7f));
+  const int64_t o = __float_as_uint(q.w);
+  log_scales[3 * o] = ls;
+  log_scales[3 * o + 1] = ls;
+  log_scales[3 * o + 2] = ls;
+}
+
+// Points with nearly all others around them (the n_crowd last entries of `far`,
+// backwards): a block compares 32 of them, one a lane, with every point,
+// CROWD_TILE at a time in shared memory, of which each warp takes its share. The
+// grid spares such a point nothing, and its scan costs more a pair (40,216 points
+// in one cell: pass 920 us, with the grid alone 1,410 or more, with a search over
+// all pairs in place of the grid 938; two points a lane 934, eight or sixteen lanes
+// a point 987-1,115). The line lies at seven in eight points because a mixture pays
+// for both searches, one after the other: the 19,600 points of a box of 40^3 voxels
+// take 276 us here, 412 with the line at a third.
+__device__ __forceinline__ void knn_crowded(const float4 *pts, int64_t n, int64_t n_crowd, const uint32_t *far,
+                                            float4 *s_p, float *log_scales) {
+  constexpr int NW = KNN_T / 32;
+  static_assert(NW * 32 <= CROWD_TILE, "the warps' results take the tile's place");
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float inf = __int_as_float(0x7f800000);
+  for (int64_t first = (int64_t)blockIdx.x * 32; first < n_crowd; first += (int64_t)gridDim.x * 32) {
+    const float4 q = pts[far[n - 1 - min(first + lane, n_crowd - 1)]];
+    float b[4] = {inf, inf, inf, inf};
+    for (int64_t t0 = 0; t0 < n; t0 += CROWD_TILE) {
+      const int cnt = (int)min((int64_t)CROWD_TILE, n - t0);
+      __syncthreads();
+      for (int k = threadIdx.x; k < cnt; k += KNN_T) s_p[k] = pts[t0 + k];
+      __syncthreads();
+#pragma unroll 4
+      for (int k = w; k < cnt; k += NW) insert4(distance2(s_p[k], q), b[0], b[1], b[2], b[3]);
+    }
+    __syncthreads();
+    s_p[w * 32 + lane] = make_float4(b[0], b[1], b[2], b[3]);
+    __syncthreads();
+    if (w == 0 && first + lane < n_crowd) {
+      for (int k = 1; k < NW; ++k) {
+        const float4 v = s_p[k * 32 + lane];
+        const float o[4] = {v.x, v.y, v.z, v.w};
+        merge4(b, o);
+      }
+      knn_scale(q, n, b, log_scales);
+    }
+  }
+}
+
 // LANES lanes per point. The cells within r of the point's own form a box;
 // once the 4th smallest distance found in it is no larger than the distance to
 // the box's faces (less a slack for the rounding of the cell assignment), no
 // point outside can be nearer. The rows of cells along x are stretches of
 // consecutive points. Points that need more than KNN_NEAR cells (isolated ones:
 // hundreds of rows, mostly empty) are left to a second launch with a warp for
-// each, which starts again. Distances are the brute-force
-// search's, bit for bit. (Brute force over all pairs: 344 us for the 25,000
+// each, which starts again, and so are those with nearly all points around them
+// (knn_crowded). (Brute force over all pairs: 344 us for the 25,000
 // points of a 512^3 volume; grid and search 57. All rows shared by eight lanes
 // 143, a lane per row from the second ring on 96, KNN_NEAR = 2 and 3 20 and 35
-// more than 1.)
+// more than 1.) A stretch of a crowded cell is long, and its scan waits for its
+// loads: three of them in flight, in place of one, take the 15,400 points of a
+// bright box of 30^3 voxels in a 512^3 volume from 319 to 244 us (two 276, four 237
+// but more registers; spread points 65 and 65).
 template <int LANES, bool FAR>
-__global__ void __launch_bounds__(256) rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid,
-                                                       const uint32_t *cells, RadsState *st, uint32_t *far,
-                                                       float *log_scales) {
+__global__ void __launch_bounds__(KNN_T, 1) rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid,
+                                                         const uint32_t *cells, RadsState *st, uint32_t *far,
+                                                         float *log_scales) {
   after_previous();
   const int sub = threadIdx.x & (LANES - 1);
-  const uint32_t group = LANES == 32 ? 0xffffffffu
-                                     : ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) / LANES * LANES);
+  const uint32_t group = lane_group<LANES>();
   const float inf = __int_as_float(0x7f800000);
   const int64_t count = FAR ? (int64_t)st->n_far : n;
-  for (int64_t item = ((int64_t)blockIdx.x * 256 + threadIdx.x) / LANES; item < count;
-       item += (int64_t)gridDim.x * 256 / LANES) {
+  for (int64_t item = ((int64_t)blockIdx.x * KNN_T + threadIdx.x) / LANES; item < count;
+       item += (int64_t)gridDim.x * KNN_T / LANES) {
     const int64_t i = FAR ? (int64_t)far[item] : item;
     const float4 q = pts[i];
     const int cx = grid.axis(0, q.x), cy = grid.axis(1, q.y), cz = grid.axis(2, q.z);
     float b[4] = {inf, inf, inf, inf};
-    bool found = false, left = false;
+    bool found = false, left = false, crowded = false;
     for (int r = 1; !found; ++r) {
       if (!FAR && r > KNN_NEAR) {
         left = true;
@@ -869,36 +952,56 @@ __global__ void __launch_bounds__(256) rads_knn_kernel(const float4 *pts, int64_
       const int x0 = max(cx - r, 0), x1 = min(cx + r, grid.n[0] - 1), y0 = max(cy - r, 0),
                 y1 = min(cy + r, grid.n[1] - 1), z0 = max(cz - r, 0), z1 = min(cz + r, grid.n[2] - 1);
       float m[4] = {inf, inf, inf, inf};  // this lane's share of the new cells
-      auto scan = [&](int row, int xa, int xb, uint32_t first, uint32_t step) {
-        const uint32_t p1 = cells[row + xb + 1];
-        for (uint32_t p = cells[row + xa] + first; p < p1; p += step) {
-          const float4 c = pts[p];
-          const float dx = c.x - q.x, dy = c.y - q.y, dz = c.z - q.z;
-          insert4(fmaf(dz, dz, fmaf(dy, dy, dx * dx)), m[0], m[1], m[2], m[3]);
+      auto scan = [&](uint32_t p, uint32_t p1, uint32_t step) {
+        for (; p + 2 * step < p1; p += 3 * step) {  // three loads in flight
+          const float4 c0 = pts[p], c1 = pts[p + step], c2 = pts[p + 2 * step];
+          insert4(distance2(c0, q), m[0], m[1], m[2], m[3]);
+          insert4(distance2(c1, q), m[0], m[1], m[2], m[3]);
+          insert4(distance2(c2, q), m[0], m[1], m[2], m[3]);
         }
+        for (; p < p1; p += step) insert4(distance2(pts[p], q), m[0], m[1], m[2], m[3]);
       };
-      if (r == 1) {  // nine rows, often full: the lanes share each
-        for (int z = z0; z <= z1; ++z)
-          for (int y = y0; y <= y1; ++y) scan((z * grid.n[1] + y) * grid.n[0], x0, x1, sub, LANES);
+      if (r == 1) {  // nine rows, often full: the lanes share each. Lane t has row t's stretch (and t + LANES's)
+        auto stretch = [&](int t, uint32_t &p0, uint32_t &p1) {
+          const int z = cz + t / 3 - 1, y = cy + t % 3 - 1;
+          p0 = p1 = 0;
+          if (t < 9 && z >= z0 && z <= z1 && y >= y0 && y <= y1) {
+            const int row = (z * grid.n[1] + y) * grid.n[0];
+            p0 = cells[row + x0];
+            p1 = cells[row + x1 + 1];
+          }
+        };
+        uint32_t p0, p1, e0 = 0, e1 = 0;
+        stretch(sub, p0, p1);
+        if (LANES < 9) stretch(sub + LANES, e0, e1);
+        if (!FAR) {
+          uint32_t c = (p1 - p0) + (e1 - e0);
+#pragma unroll
+          for (int o = LANES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(group, c, o);
+          if (8 * (uint64_t)c > 7 * (uint64_t)n) {  // nearly all points
+            crowded = true;
+            break;
+          }
+        }
+#pragma unroll 1
+        for (int t = 0; t < 9; ++t) {
+          const uint32_t a = __shfl_sync(group, t < LANES ? p0 : e0, t % LANES, LANES),
+                         z = __shfl_sync(group, t < LANES ? p1 : e1, t % LANES, LANES);
+          scan(a + sub, z, LANES);
+        }
       } else {  // many rows, mostly empty (else the search had ended): a lane per row
         const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
         for (int t = sub; t < rows; t += LANES) {
           const int z = z0 + t / ny, y = y0 + t % ny, row = (z * grid.n[1] + y) * grid.n[0];
           if (z == cz - r || z == cz + r || y == cy - r || y == cy + r) {
-            scan(row, x0, x1, 0, 1);
+            scan(cells[row + x0], cells[row + x1 + 1], 1);
           } else {  // the middle of the row was searched before
-            if (cx - r >= 0) scan(row, cx - r, cx - r, 0, 1);
-            if (cx + r < grid.n[0]) scan(row, cx + r, cx + r, 0, 1);
+            if (cx - r >= 0) scan(cells[row + cx - r], cells[row + cx - r + 1], 1);
+            if (cx + r < grid.n[0]) scan(cells[row + cx + r], cells[row + cx + r + 1], 1);
           }
         }
       }
-#pragma unroll
-      for (int o = LANES / 2; o > 0; o >>= 1) {
-        float t[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) t[k] = __shfl_xor_sync(group, m[k], o);
-        merge4(m, t);
-      }
+      merge_group<LANES>(group, m);
       merge4(b, m);
       // distance to the nearest face of the box that has cells behind it
       float d = inf;
@@ -918,18 +1021,15 @@ __global__ void __launch_bounds__(256) rads_knn_kernel(const float4 *pts, int64_
       far[atomicAdd(&st->n_far, 1u)] = (uint32_t)i;
       continue;
     }
-    // b[0] is the point itself (0); the others are the nearest other points
-    const int kk = n - 1 < 3 ? (int)(n - 1) : 3;
-    float m = 0.f;
-    if (kk >= 1) m += b[1];
-    if (kk >= 2) m += b[2];
-    if (kk >= 3) m += b[3];
-    m = kk > 0 ? m / (float)kk : 0.f;
-    const float ls = 0.5f * logf(fmaxf(m, 1e-7f));
-    const int64_t o = __float_as_uint(q.w);
-    log_scales[3 * o] = ls;
-    log_scales[3 * o + 1] = ls;
-    log_scales[3 * o + 2] = ls;
+    if (crowded) {
+      far[n - 1 - atomicAdd(&st->n_crowd, 1u)] = (uint32_t)i;
+      continue;
+    }
+    knn_scale(q, n, b, log_scales);
+  }
+  if constexpr (FAR) {
+    __shared__ float4 s_p[CROWD_TILE];
+    knn_crowded(pts, n, (int64_t)st->n_crowd, far, s_p, log_scales);
   }
 }
 
@@ -1145,13 +1245,13 @@ extern "C" ddgs_status ddgs_rads(const ddgs_volume *vol, int32_t n1, int32_t n2,
     }
     {
       LaunchScope ls(KID_RADS_KNN, st);
-      launch_next(rads_knn_kernel<8, false>, (unsigned)((n * 8 + 255) / 256), 256u, 0, st, pts, n, grid, cells, state,
-                  far, log_scales);
+      launch_next(rads_knn_kernel<8, false>, (unsigned)((n * 8 + KNN_T - 1) / KNN_T), KNN_T, 0, st, pts, n, grid, cells,
+                  state, far, log_scales);
     }
     {
       LaunchScope ls(KID_RADS_KNN, st);
-      const unsigned g = (unsigned)std::min<int64_t>((n * 32 + 255) / 256, 8 * device_sms());
-      launch_next(rads_knn_kernel<32, true>, g, 256u, 0, st, pts, n, grid, cells, state, far, log_scales);
+      const unsigned g = (unsigned)std::min<int64_t>((n * 32 + KNN_T - 1) / KNN_T, 8 * device_sms());
+      launch_next(rads_knn_kernel<32, true>, g, KNN_T, 0, st, pts, n, grid, cells, state, far, log_scales);
     }
     RCK(cudaGetLastError());
   }
