@@ -99,7 +99,7 @@ __device__ __forceinline__ Tv warp_incl_scan(Tv x) {
 // ---- pass 1: min and max of the volume ----
 // Bound by DRAM (one read of the volume): four 16-byte loads in flight per
 // thread and packed 16-bit min / max, two voxels an instruction (512^3: 64 ->
-// 57 us, 4.7 TB/s).
+// 60 us, 4.5 TB/s).
 __global__ void __launch_bounds__(RT) rads_minmax_kernel(Vol v, RadsState *st) {
   after_previous();
   const int64_t n8 = v.nvox / 8, stride = (int64_t)gridDim.x * blockDim.x;
@@ -286,7 +286,7 @@ struct GroupCross {
 // ---- pass 2: crossings and weight per warp sub-chunk (512 voxels) ----
 // Bound by L2 reads (each voxel is read as itself and as the +z neighbour; the
 // +y one mostly hits L1), packed compares of two voxels an instruction: 512^3
-// 168 -> 133 us. (Resident warps that go from sub-chunk to sub-chunk: 161 us.)
+// 168 -> 127 us. (Resident warps that go from sub-chunk to sub-chunk: 161 us.)
 template <bool VEC>
 __global__ void __launch_bounds__(RT) rads_count_kernel(Vol vol, const RadsState *st, uint32_t *csub,
                                                         uint64_t *wsub) {
@@ -404,7 +404,7 @@ __device__ __forceinline__ uint64_t edge_key(uint64_t seed, uint64_t e) {
 
 // ---- pass 3: the keys of every crossing, in edge order. A warp without
 // crossings (most of the volume) returns at once; the others know where their
-// keys start from the counts of pass 2 (512^3: 182 -> 65 us; resident warps that
+// keys start from the counts of pass 2 (512^3: 182 -> 72 us; resident warps that
 // look at 32 sub-chunks at a time and go through the non-empty ones 114, as these
 // lie together). ----
 template <bool VEC>
@@ -882,7 +882,8 @@ __device__ __forceinline__ void knn_scale(const float4 &q, int64_t n, const floa
 // all pairs in place of the grid 938; two points a lane 934, eight or sixteen lanes
 // a point 987-1,115). The line lies at seven in eight points because a mixture pays
 // for both searches, one after the other: the 19,600 points of a box of 40^3 voxels
-// take 276 us here, 412 with the line at a third.
+// take 276 us so, 294 and 298 with the line at a half and a third (with four loads in
+// flight in the grid's scan).
 __device__ __forceinline__ void knn_crowded(const float4 *pts, int64_t n, int64_t n_crowd, const uint32_t *far,
                                             float4 *s_p, float *log_scales) {
   constexpr int NW = KNN_T / 32;
@@ -922,16 +923,17 @@ __device__ __forceinline__ void knn_crowded(const float4 *pts, int64_t n, int64_
 // hundreds of rows, mostly empty) are left to a second launch with a warp for
 // each, which starts again, and so are those with nearly all points around them
 // (knn_crowded). (Brute force over all pairs: 344 us for the 25,000
-// points of a 512^3 volume; grid and search 57. All rows shared by eight lanes
+// points of a 512^3 volume; grid and search 65. All rows shared by eight lanes
 // 143, a lane per row from the second ring on 96, KNN_NEAR = 2 and 3 20 and 35
 // more than 1.) A stretch of a crowded cell is long, and its scan waits for its
-// loads: three of them in flight, in place of one, take the 15,400 points of a
-// bright box of 30^3 voxels in a 512^3 volume from 319 to 244 us (two 276, four 237
-// but more registers; spread points 65 and 65).
+// loads: with three in flight in place of one, the 20,800 points of two bright boxes
+// of 30^3 voxels in a 512^3 volume take 228 us in place of 302. Six blocks per SM (39
+// registers): five (48 registers) 174 us there, but the search of a 301 x 277 x 190
+// volume's points, 782 blocks, then needs a second wave (the whole call 221 -> 224 us).
 template <int LANES, bool FAR>
-__global__ void __launch_bounds__(KNN_T, 1) rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid,
-                                                         const uint32_t *cells, RadsState *st, uint32_t *far,
-                                                         float *log_scales) {
+__global__ void __launch_bounds__(KNN_T, FAR ? 1 : 6)
+rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid, const uint32_t *cells, RadsState *st, uint32_t *far,
+                float *log_scales) {
   after_previous();
   const int sub = threadIdx.x & (LANES - 1);
   const uint32_t group = lane_group<LANES>();
@@ -945,10 +947,6 @@ __global__ void __launch_bounds__(KNN_T, 1) rads_knn_kernel(const float4 *pts, i
     float b[4] = {inf, inf, inf, inf};
     bool found = false, left = false, crowded = false;
     for (int r = 1; !found; ++r) {
-      if (!FAR && r > KNN_NEAR) {
-        left = true;
-        break;
-      }
       const int x0 = max(cx - r, 0), x1 = min(cx + r, grid.n[0] - 1), y0 = max(cy - r, 0),
                 y1 = min(cy + r, grid.n[1] - 1), z0 = max(cz - r, 0), z1 = min(cz + r, grid.n[2] - 1);
       float m[4] = {inf, inf, inf, inf};  // this lane's share of the new cells
@@ -1015,6 +1013,10 @@ __global__ void __launch_bounds__(KNN_T, 1) rads_knn_kernel(const float4 *pts, i
       }
       // d is infinite when every cell was searched; a NaN or negative d goes on
       found = d == inf || (d > 0.f && b[3] <= d * d * 0.9999f);
+      if (!FAR && r == KNN_NEAR) {
+        left = !found;
+        break;
+      }
     }
     if (sub != 0) continue;
     if (left) {
