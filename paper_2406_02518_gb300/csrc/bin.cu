@@ -784,7 +784,6 @@ __global__ void __launch_bounds__(NT, MINB) bin_sort_block_kernel(const uint64_t
       dmin = min(dmin, s_red[0][x]);
       dmax = max(dmax, s_red[1][x]);
     }
-    bool sorted = false;
     if (dmin != dmax && m > 1) {
       // buckets: 2^lg >= m of them (at least 32, at most NW x 256)
       int lg = 32 - __clz((uint32_t)m - 1u);
@@ -868,9 +867,9 @@ __global__ void __launch_bounds__(NT, MINB) bin_sort_block_kernel(const uint64_t
     const int rows = (rows_all + NW - 1) / NW, seg = rows * 32;
     // depth digits first; only if two depths tie, redo with the index digits
     // below them (least significant first)
-    const int nd = sorted || dmin == dmax ? 0 : (39 - __clz(dmin ^ dmax)) / 8;
+    const int nd = dmin == dmax ? 0 : (39 - __clz(dmin ^ dmax)) / 8;
     int nl = 0;
-    for (int round = 0; round < 2 && !sorted; ++round) {
+    for (int round = 0; round < 2; ++round) {
       for (int p = 0; p < nl + nd; ++p) {
         const int shift = p < nl ? 8 * p : 32 + 8 * (p - nl);
         block_digit_pass<NT, E>(cur, oth, m, seg, rows, shift, cnt, s_wsum);

@@ -140,7 +140,10 @@ struct ZeroList {
 // without: a persistent kernel with much shared memory must not start on SMs
 // still set up for the small share of the kernel before it, where too few of its
 // blocks fit and stay (the sorts of 69 M pairs: the step 5.31 -> 5.63 ms; the
-// backward preprocess at 2M Gaussians: 6.64 -> 6.72).
+// backward preprocess at 2M Gaussians: 6.64 -> 6.72). The rasterisers start early all
+// the same: their warps take items from a queue, so that an SM with fewer blocks does
+// less (64 poses of 256^2 5.15 ms early or late, 2M Gaussians on 8 of 1024^2 6.35 and
+// 6.35; 4,096 Gaussians on 128^2 108 and 110 us).
 template <class... KArgs, class... Args>
 inline cudaError_t launch_kernel(bool early, void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem,
                                  cudaStream_t st, Args... args) {

@@ -106,8 +106,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Pixel-space box of the q <= q_max ellipse: the record's packed
 // half-extents (computed from the 2D covariance by the preprocess).
-__device__ __forceinline__ float4 ellipse_box(float4 r0, float4 r1, float q_max) {
-  (void)q_max;
+__device__ __forceinline__ float4 ellipse_box(float4 r0, float4 r1) {
   const float2 e = unpack_halfwidths(r1.w);
   return make_float4(r0.x - e.x, r0.x + e.x, r0.y - e.y, r0.y + e.y);
 }
@@ -319,7 +318,7 @@ __device__ __forceinline__ void fwd_lane_item(const RasterArgs &a, int64_t gt, i
     if (__all_sync(0xffffffffu, done)) break;
     uint32_t cover;
     pk.fill(st, nullptr, nullptr,
-            [&](float4 r0, float4 r1) { return region_cover<ROWS>(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+            [&](float4 r0, float4 r1) { return region_cover<ROWS>(ellipse_box(r0, r1), cx, cy); },
             [&](int k, float4 r0, float4 r1, uint32_t, uint32_t) { sm.a[k] = r0; sm.b[k] = r1; }, cover);
     uint32_t mine = transpose32(cover);  // staged entries covering this lane's pixel
     if (done) mine = 0;
@@ -389,7 +388,12 @@ __global__ void __launch_bounds__(WARPS * 32, 5) raster_fwd_lane_kernel(RasterAr
 //     that the mean and conic gradients need follow from those moments.
 // No lane reduces another lane's values and no shared-memory atomic is used.
 constexpr int AB_STRIDE = 32;  // float2 per pixel row of the (pixel, entry) table
-constexpr int LANE_WARPS = 8;  // warps per block of the per-lane backward (3 blocks per SM)
+// Warps per block of the per-lane backward: 77 KB, two blocks per SM. Three (a
+// batch's covers and walk indices in the table's place make room for them) are no
+// faster: these renders have few items, and a warp that shares its SM with more of
+// them finishes the longest list later (raster_bwd, 100k Gaussians, one view at tile
+// 8: 256^2 63 and 63 us, 300^2 60 and 79, 360^2 68 and 75; 340^2 at tile 32 86 and 110).
+constexpr int LANE_WARPS = 8;
 
 struct LaneBwdSmem {
   float4 a[33], b[33];  // entry 32: a sentinel that no pixel adds
@@ -431,7 +435,7 @@ __device__ __forceinline__ void bwd_lane_item(const RasterArgs &a, int64_t gt, i
     uint32_t cover;
     const int cnt = pk.fill(
         st, sm.cover, sm.j,
-        [&](float4 r0, float4 r1) { return region_cover<false>(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+        [&](float4 r0, float4 r1) { return region_cover<false>(ellipse_box(r0, r1), cx, cy); },
         [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) { sm.a[k] = r0; sm.b[k] = r1; sm.id[k] = id; },
         cover);
     uint32_t mine = transpose32(cover);
@@ -713,7 +717,7 @@ __device__ __forceinline__ void fwd_pair_item(const RasterArgs &a, int64_t gt, i
     if (st.more() || pk.left()) {
       uint32_t cover;
       pk.fill(st, sm.cover, sm.j + half,
-              [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+              [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1), cx, cy); },
               [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) {
                 sm.slot.put(half + k, pair_entry(r0, r1));
                 if (PIX) sm.z[half + k] = a.rec2[rg.rec_base + id];
@@ -898,7 +902,7 @@ __device__ __forceinline__ void bwd_pair_item(const RasterArgs &a, int64_t gt, i
     uint32_t cover;
     const int cnt = pk.fill(
         st, sm.cover, sm.j,
-        [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1, a.P.q_max), cx, cy); },
+        [&](float4 r0, float4 r1) { return pair_cover(ellipse_box(r0, r1), cx, cy); },
         [&](int k, float4 r0, float4 r1, uint32_t id, uint32_t) {
           sm.slot.put(k, pair_entry(r0, r1));
           sm.id[k] = id;
