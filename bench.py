@@ -117,10 +117,10 @@ class Clocks:
 # shape and workload match; otherwise traffic is null.
 TRAFFIC = {
     "raster_bwd": {
-        "sources_sha256": {"raster.cu": "70586b0a056fc1ee8a87e4831d250651f238395b978c966ea2ca900c7a822ea5",
-                           "ddgs_internal.cuh": "f95d7930bf87fcb211fca5e9c600c2d990ed908d118cc5783b5c7e7f8b603b2b"},
+        "sources_sha256": {"raster.cu": "6ebc3dce501614b0137091691e62624b09e0c221e21d0f27ee916ba6d2623a42",
+                           "ddgs_internal.cuh": "ea195fea1a98d7022cd3d42a639db7e3e5cdcc27a87aa82729de2d4ac7fcfc7c"},
         "tile": 8, "batch_depth": 32, "views": 64, "gaussians": 500_000,
-        "bytes_per_launch": 5373.5e6 + 797.6e6,
+        "bytes_per_launch": 5375.6e6 + 797.9e6,
         "how": "one-pass ncu launch list (dram__bytes_read.sum + dram__bytes_write.sum) of the "
                "64-pose registration step",
     },

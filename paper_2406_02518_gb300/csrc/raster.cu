@@ -594,9 +594,10 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 
-// A staged entry: mean, a', 2b', c', -alpha, colour. Shared memory bounds the
-// pair kernels (its pipe was busy 84 % forward, 86 % backward when each lane
-// loaded 48 bytes a trip, the values duplicated for the packed units), so an
+// A staged entry: mean, a', 2b', c', -alpha, colour. The pair kernels are bound by
+// issue slots and by shared memory, whose pipe was busy 84 % forward and 86 %
+// backward when each lane loaded 48 bytes a trip, the values duplicated for the
+// packed units (now 68 and 76 %, issue 81 and 70 %). So an
 // entry is two 16-byte pieces, in arrays of their own so that eight consecutive
 // entries meet no bank conflict; duplicating in registers is cheaper (raster_fwd
 // and raster_bwd at 64 views of 256^2: 1068 -> 1008 and 2168 -> 2078 us, 2M
