@@ -37,6 +37,7 @@ constexpr int SEL_CAND = 4096;  // keys that the select's last step orders in on
 constexpr int KNN_CELLS = 32768;  // most cells of the neighbour search's grid
 constexpr int KNN_NEAR = 1;     // rings of cells searched by eight lanes a point, then by a warp
 constexpr int KNN_T = 256;      // threads per block of the search
+constexpr uint32_t CROWD_SPREAD = 16;  // see knn_crowded
 constexpr int CROWD_TILE = 1024;  // points staged at a time for those in crowded cells
 
 // Output number i + 1 of SplitMix64 (Steele, Lea and Flood, OOPSLA 2014)
@@ -874,16 +875,18 @@ __device__ __forceinline__ void knn_scale(const float4 &q, int64_t n, const floa
   log_scales[3 * o + 2] = ls;
 }
 
-// Points with nearly all others around them (the n_crowd last entries of `far`,
-// backwards): a block compares 32 of them, one a lane, with every point,
-// CROWD_TILE at a time in shared memory, of which each warp takes its share. The
-// grid spares such a point nothing, and its scan costs more a pair (40,216 points
-// in one cell: pass 920 us, with the grid alone 1,410 or more, with a search over
-// all pairs in place of the grid 938; two points a lane 934, eight or sixteen lanes
-// a point 987-1,115). The line lies at seven in eight points because a mixture pays
-// for both searches, one after the other: the 19,600 points of a box of 40^3 voxels
-// take 276 us so, 294 and 298 with the line at a half and a third (with four loads in
-// flight in the grid's scan).
+// Points of a crowd (the n_crowd last entries of `far`, backwards): a block compares
+// 32 of them, one a lane, with every point, CROWD_TILE at a time in shared memory,
+// of which each warp takes its share. The grid spares such a point nothing, and its
+// scan costs more a pair (40,216 points in one cell: the whole call 912 us, with the
+// grid alone 2,062, with a search over all pairs in place of the grid 937; two points
+// a lane 934, eight or sixteen lanes a point 987-1,115, tiles of 256 points 1,015).
+// A point is of a crowd when more than seven in eight of all points are in its first
+// ring, and no axis of cells has one in CROWD_SPREAD of these on both its sides: there
+// the points further out see fewer, stay with the grid, and both searches are paid for
+// one after the other (the 19,600 points of a box of 40^3 voxels in a 512^3 volume:
+// call 662 us, 523 with this rule; lines at a half and a third of the points were
+// slower still). y and z are looked at, whose rows have been counted.
 __device__ __forceinline__ void knn_crowded(const float4 *pts, int64_t n, int64_t n_crowd, const uint32_t *far,
                                             float4 *s_p, float *log_scales) {
   constexpr int NW = KNN_T / 32;
@@ -921,10 +924,9 @@ __device__ __forceinline__ void knn_crowded(const float4 *pts, int64_t n, int64_
 // point outside can be nearer. The rows of cells along x are stretches of
 // consecutive points. Points that need more than KNN_NEAR cells (isolated ones:
 // hundreds of rows, mostly empty) are left to a second launch with a warp for
-// each, which starts again, and so are those with nearly all points around them
-// (knn_crowded). (Brute force over all pairs: 344 us for the 25,000
-// points of a 512^3 volume; grid and search 65. All rows shared by eight lanes
-// 143, a lane per row from the second ring on 96, KNN_NEAR = 2 and 3 20 and 35
+// each, which starts again, and so are those of a crowd (knn_crowded). (Brute force
+// over all pairs: 344 us for the 25,000 points of a 512^3 volume; grid and search 65.
+// All rows shared by eight lanes 143, a lane per row from the second ring on 96, KNN_NEAR = 2 and 3 20 and 35
 // more than 1.) A stretch of a crowded cell is long, and its scan waits for its
 // loads: with three in flight in place of one, the 20,800 points of two bright boxes
 // of 30^3 voxels in a 512^3 volume take 228 us in place of 302. Six blocks per SM (39
@@ -951,12 +953,6 @@ rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid, const uint32_t *cell
                 y1 = min(cy + r, grid.n[1] - 1), z0 = max(cz - r, 0), z1 = min(cz + r, grid.n[2] - 1);
       float m[4] = {inf, inf, inf, inf};  // this lane's share of the new cells
       auto scan = [&](uint32_t p, uint32_t p1, uint32_t step) {
-        for (; p + 2 * step < p1; p += 3 * step) {  // three loads in flight
-          const float4 c0 = pts[p], c1 = pts[p + step], c2 = pts[p + 2 * step];
-          insert4(distance2(c0, q), m[0], m[1], m[2], m[3]);
-          insert4(distance2(c1, q), m[0], m[1], m[2], m[3]);
-          insert4(distance2(c2, q), m[0], m[1], m[2], m[3]);
-        }
         for (; p < p1; p += step) insert4(distance2(pts[p], q), m[0], m[1], m[2], m[3]);
       };
       if (r == 1) {  // nine rows, often full: the lanes share each. Lane t has row t's stretch (and t + LANES's)
@@ -973,19 +969,33 @@ rads_knn_kernel(const float4 *pts, int64_t n, KnnGrid grid, const uint32_t *cell
         stretch(sub, p0, p1);
         if (LANES < 9) stretch(sub + LANES, e0, e1);
         if (!FAR) {
-          uint32_t c = (p1 - p0) + (e1 - e0);
+          auto group_sum = [&](uint32_t x) {
 #pragma unroll
-          for (int o = LANES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(group, c, o);
-          if (8 * (uint64_t)c > 7 * (uint64_t)n) {  // nearly all points
-            crowded = true;
-            break;
+            for (int o = LANES / 2; o > 0; o >>= 1) x += __shfl_xor_sync(group, x, o);
+            return x;
+          };
+          const uint32_t own = p1 - p0, ninth = e1 - e0;  // the points of row sub, and (first lane) of row 8
+          const uint32_t c = group_sum(own + ninth);
+          if (8 * (uint64_t)c > 7 * (uint64_t)n) {  // nearly all points: a crowd? (knn_crowded)
+            const uint32_t zl = group_sum(sub < 3 ? own : 0u), zh = group_sum((sub >= 6 ? own : 0u) + ninth);
+            const uint32_t yl = group_sum(sub % 3 == 0 ? own : 0u), yh = group_sum((sub % 3 == 2 ? own : 0u) + ninth);
+            crowded = max(min(zl, zh), min(yl, yh)) <= c / CROWD_SPREAD;
+            if (crowded) break;
           }
         }
 #pragma unroll 1
         for (int t = 0; t < 9; ++t) {
           const uint32_t a = __shfl_sync(group, t < LANES ? p0 : e0, t % LANES, LANES),
                          z = __shfl_sync(group, t < LANES ? p1 : e1, t % LANES, LANES);
-          scan(a + sub, z, LANES);
+          uint32_t p = a + sub;
+          if (!FAR)
+            for (; p + 2 * LANES < z; p += 3 * LANES) {  // three loads in flight
+              const float4 c0 = pts[p], c1 = pts[p + LANES], c2 = pts[p + 2 * LANES];
+              insert4(distance2(c0, q), m[0], m[1], m[2], m[3]);
+              insert4(distance2(c1, q), m[0], m[1], m[2], m[3]);
+              insert4(distance2(c2, q), m[0], m[1], m[2], m[3]);
+            }
+          scan(p, z, LANES);
         }
       } else {  // many rows, mostly empty (else the search had ended): a lane per row
         const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);

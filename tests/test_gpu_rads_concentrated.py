@@ -33,6 +33,7 @@ ONE = [(7, 9, 11, 1)]  # six crossings
     ((64, 64, 64), ONE, 0, 100, 1018),     # 1,024 points, a staged tile
     ((64, 64, 64), ONE, 0, 100, 1019),
     ((96, 96, 96), [(10, 10, 10, 3), (90, 90, 90, 1)], 0, 500, 3000),  # 27 in 28 points crowded, the others not
+    ((96, 96, 96), [(40, 40, 40, 12)], 0, 800, 1200),  # crowds in cells next to one another: some spread, some not
     ((160, 160, 160), [(8, 8, 8, 8), (140, 140, 140, 8)], 0, 3000, 2500),  # half of all points around each: the grid
     ((96, 96, 96), [(40, 40, 40, 10)], 400, 2000, 3000)])  # a crowd and a haze: the grid
 def test_concentrated_points(shape, blobs, noise, n1, n2, ws):
